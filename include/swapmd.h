@@ -390,10 +390,11 @@ SWP_API int swp_set_withhold_arrival(swp_ctx* ctx, int on);
  * [9] = U2, U3, W xx yy zz xy xz yz, n_bonds.  Velocities are taken as zero
  * and masses as one; the context's own state is not touched.
  *
- * Scratch: a file-scope device array of SWP_STATIC_SCRATCH_BYTES (8 MiB)
- * that every GPU loading this library keeps until the process exits.  The
- * state copy, cell list and neighbour list of the system must fit in it
- * (about 10,000 particles at max_nn 64 and liquid densities); larger systems
+ * Scratch: a file-scope device array of 1.5 x SWP_STATIC_SCRATCH_BYTES (12
+ * MiB) that every GPU loading this library keeps until the process exits.  The
+ * state copy, cell list and neighbour list (six bytes per entry; the rest of
+ * the array holds the rows' padding) of the system must fit in
+ * SWP_STATIC_SCRATCH_BYTES (about 10,000 particles at max_nn 64 and liquid densities); larger systems
  * are rejected with SWP_ERR_INVALID and a message giving the bytes needed.
  * Every call shares that one array and leaves its contents behind (each call
  * re-initialises what must start at zero), so calls that overlap on the GPU

@@ -184,18 +184,32 @@ int derive_cells(swp_ctx* c)
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Neighbour-list buffer: entries of every block's region (capacity
-// (n + max_blocks) * max_nn, enough for any grid of at most max_blocks
-// blocks): partner slots, then owner indices (both int32).
-size_t list_entries(const swp_ctx* c) { return ((size_t)std::max(c->n, 1) + c->max_blocks) * c->max_nn; }
+// Entries per particle in the list buffer: FP32 rows are padded to multiples of
+// four (at most six entries of padding per particle) and start at multiples of
+// four.
+int list_stride(const swp_ctx* c) { return c->precision == SWP_FP32 ? (c->max_nn + 6 + 3) & ~3 : c->max_nn; }
 
-size_t list_bytes(const swp_ctx* c) { return align256(list_entries(c) * 4) + align256(list_entries(c) * 2); }
+// Neighbour-list buffer: entries of every block's region (list_stride x
+// (n + max_blocks), enough for any grid of at most max_blocks blocks): partner
+// slots, then (FP64) owner indices or (FP32) the threads' list ranges.
+size_t list_particles(const swp_ctx* c) { return (size_t)std::max(c->n, 1) + c->max_blocks; }
+
+size_t list_entries(const swp_ctx* c) { return list_particles(c) * list_stride(c); }
+
+size_t list_bytes(const swp_ctx* c)
+{
+    return align256(list_entries(c) * 4) +
+           align256(c->precision == SWP_FP32 ? list_particles(c) * sizeof(int4) : list_entries(c) * 2);
+}
 
 template <typename Real>
 void set_list(const swp_ctx* c, char* base, Dev<Real>* d)
 {
+    char* second = base ? base + align256(list_entries(c) * 4) : nullptr;
+    d->list_stride = list_stride(c);
     d->ent_j = (int*)base;
-    d->ent_o = base ? (unsigned short*)(base + align256(list_entries(c) * 4)) : nullptr;
+    d->ent_o = sizeof(Real) == 4 ? nullptr : (unsigned short*)second;
+    d->tinfo = sizeof(Real) == 4 ? (int4*)second : nullptr;
 }
 
 // Carves the workspace; with base == nullptr only measures it.
@@ -250,6 +264,8 @@ size_t layout(swp_ctx* c, char* base, Dev<Real>* d)
             d->hL[k] = (Real)(0.5 * (double)(Real)L);
             d->inv_cw[k] = (Real)(c->nc[k] / L);
             d->iL[k] = (Real)(1.0 / (double)(Real)L);
+            d->Lf[k] = (float)L;
+            d->iLf[k] = (float)(1.0 / L);
             d->fmul[k] = (unsigned long long)(((unsigned __int128)1 << 96) / (unsigned __int128)q);
             d->fscale[k] = (float)((double)q * 0x1p-80);
         }
@@ -297,6 +313,7 @@ template <typename Real>
 void fill_pair_table(const swp_ctx* c, PairP<Real>* t)
 {
     std::memset(t, 0, sizeof(PairP<Real>) * kMaxTypes * kMaxTypes);
+    const double Lm = std::max(c->box[0], std::max(c->box[1], c->box[2]));
     for (int k = 0; k < c->ntypes * c->ntypes; k++) {
         const PairHost& p = c->pairs[k];
         PairP<Real> e;
@@ -328,6 +345,8 @@ void fill_pair_table(const swp_ctx* c, PairP<Real>* t)
                                       : p.sigma * std::pow((1.0 - std::sqrt(0.5)) / 2.0, -1.0 / p.n);
             e.rbond2 = (Real)(rb * rb);
         }
+        const double reach = pair_cut(p) + 0x1p-18 * Lm;
+        e.reach2 = p.kind == KIND_NONE ? 0.0f : (float)(reach * reach * (1.0 + 1e-6));
         t[k] = e;
     }
 }
@@ -502,7 +521,8 @@ int run(swp_ctx* c, RunArgs a)
 {
     Dev<Real>& d = dev<Real>(c);
     int bps = 0;
-    SWP_CUDA(c, run_occupancy<Real>(kBlock, &bps));
+    const int block = sizeof(Real) == 4 ? kBlock : kBlock64;
+    SWP_CUDA(c, run_occupancy<Real>(block, &bps));
     if (bps < 1) return fail(c, SWP_ERR_CUDA, "step kernel does not fit on an SM");
     if (c->bps_req > 0) bps = std::min(bps, c->bps_req);
     bps = std::min(bps, c->max_blocks / std::max(c->num_sms, 1));
@@ -534,7 +554,7 @@ int run(swp_ctx* c, RunArgs a)
     c->withhold = 0;  // one launch consumes the request
     SWP_CUDA(c, cudaMemsetAsync(&d.ctl->barrier, 0, sizeof(unsigned long long), c->stream));
     if (wide) SWP_CUDA(c, launch_run_wide<Real>(d, a, c->grid, c->stream));
-    else SWP_CUDA(c, launch_run<Real>(d, a, c->grid, kBlock, c->stream));
+    else SWP_CUDA(c, launch_run<Real>(d, a, c->grid, block, c->stream));
     return SWP_OK;
 }
 
@@ -1537,7 +1557,11 @@ namespace {
 constexpr size_t kStaticScratchBytes = (size_t)SWP_STATIC_SCRATCH_BYTES;
 constexpr int kMaxStaticDevices = 64;
 
-static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
+// The systems the entry point takes are those whose layout with max_nn entries
+// of six bytes per particle fits SWP_STATIC_SCRATCH_BYTES; the array also holds
+// what the FP32 rows' padding and the threads' list ranges add to that (at most
+// 52 bytes per particle, of at least 100).
+static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes + kStaticScratchBytes / 2];
 
 // Device address of g_static_scratch per device (host code sees only a
 // stand-in symbol; the address comes from cudaGetSymbolAddress).
@@ -1573,8 +1597,9 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
     if (!c->bond_host.empty()) return fail(c, SWP_ERR_INVALID, "bonded systems are not supported here");
     char* base = (char*)g_static_addr[dev];
     const size_t ws = layout<Real>(c, nullptr, nullptr);
-    const size_t nl = list_bytes(c);
-    if (ws + nl > kStaticScratchBytes) {
+    const size_t plain = list_particles(c) * c->max_nn;
+    const size_t nl = align256(plain * 4) + align256(plain * 2);
+    if (ws + nl > kStaticScratchBytes || ws + list_bytes(c) > sizeof(g_static_scratch)) {
         char buf[200];
         std::snprintf(buf, sizeof buf,
                       "system needs %zu bytes of scratch; the static scratch holds %zu "
@@ -1604,7 +1629,8 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
     SWP_CUDA(c, launch_set_state<Real>(d, s));
 
     int bps = 0;
-    SWP_CUDA(c, run_occupancy<Real>(kBlock, &bps));
+    const int block = sizeof(Real) == 4 ? kBlock : kBlock64;
+    SWP_CUDA(c, run_occupancy<Real>(block, &bps));
     if (bps < 1) return fail(c, SWP_ERR_CUDA, "step kernel does not fit on an SM");
     if (c->bps_req > 0) bps = std::min(bps, c->bps_req);
     bps = std::min(bps, c->max_blocks / std::max(c->num_sms, 1));
@@ -1614,7 +1640,7 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
     a.timeout_ns = c->timeout_ns;
     a.skin_eff = c->skin;
     a.seed = c->seed;
-    SWP_CUDA(c, launch_run<Real>(d, a, step_grid(c, bps), kBlock, s));
+    SWP_CUDA(c, launch_run<Real>(d, a, step_grid(c, bps), block, s));
     SWP_CUDA(c, cudaMemcpyAsync(&h, d.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
     SWP_CUDA(c, cudaStreamSynchronize(s));
     if (h.status & kStatusTimeout) return fail(c, SWP_ERR_TIMEOUT, "a device-side wait timed out");

@@ -11,7 +11,8 @@ namespace swp {
 constexpr int kMaxTypes = 8;       // type-pair table is kMaxTypes^2 entries at most
 constexpr int kNQ = 12;            // per-block thermo partials: see Q_* below
 constexpr int kTypeBits = 4;       // packed word: (tag << kTypeBits) | type
-constexpr int kBlock = 768;        // threads per block of the step kernel (one block per SM, 80 registers)
+constexpr int kBlock = 768;        // threads per block of the FP32 step kernel (one block per SM, 80 registers)
+constexpr int kBlock64 = 512;      // of the FP64 step kernel
 constexpr int kMaxGrid = 320;      // largest grid of the step kernel (blocks)
 constexpr int kBlockBatch = 1024;  // threads per block of the batched kernel
 constexpr int kBlockWide = 1024;   // threads per block of the step kernel of bonded networks
@@ -35,7 +36,7 @@ struct PairP {
     int kind;   // PairKind
     int nhalf;  // exponent n = 2*nhalf + odd
     int odd;
-    int pad;
+    float reach2;  // FP64: squared cut-off of the FP32 sorting-out of listed pairs (see may_reach)
     Real four_eps;    // 4 eps
     Real n_real;      // n
     Real sig2;        // sigma^2
@@ -117,13 +118,15 @@ struct Dev {
     typedef typename PosVec<Real>::type P4;
     int n;
     int ntypes;
-    int max_nn;
+    int max_nn;       // capacity of the list: entries per particle, on average over a block
+    int list_stride;  // entries per particle in the list buffer (FP32: max_nn and the rows' padding)
     int ncell;
     int nc[3];
     Real L[3];
     Real hL[3];
     Real inv_cw[3];  // cells per unit length
     Real iL[3];      // 1 / L
+    float Lf[3], iLf[3];  // the same in FP32 (FP64 runs: the sorting-out of listed pairs)
     long long Lq[3]; // box in fixed-point units
     // FP32 snapshot coordinates: u = floor(q fmul / 2^64) with q the fixed-point
     // coordinate and fmul = floor(2^96 / Lq), a 32-bit fraction of the box edge;
@@ -137,15 +140,16 @@ struct Dev {
     R4* vel[2];        // (vx, vy, vz, 1/m), two sets
     R4* force;         // (fx, fy, fz, 0)
     Real* S;           // per-centre sum of a*vh over reactive partners
-    int* ent_j;            // neighbour entries: partner slot (block-compact layout)
-    unsigned short* ent_o; // neighbour entries: owner's index inside its sub-chunk (< 1024)
+    int* ent_j;            // neighbour entries: partner slot
+    unsigned short* ent_o; // FP64: neighbour entries: owner's index inside its sub-chunk (< 1024)
+    int4* tinfo;           // FP32: pinfo in the order in which a block's threads take its particles (perm)
     int4* pinfo;           // per particle: (first reactive entry, count, first other entry, count)
     const int* cell_rank;  // [2 * ncell]: cell linear index -> rank in the sorted cell order,
                            // then rank -> linear index
     int* cell_cnt;     // [ncell]
     int* cell_start;   // [ncell + 1]
     int* cell_fill;    // [ncell]
-    int* perm;         // [n] new slot -> old slot
+    int* perm;         // [n] new slot -> old slot while the list is built; then (FP32) the particle of every thread
     int* bsum;         // [max_blocks] per-block cell-count sums (scan)
     double* partials;  // [max_blocks][kNQ]
     Ctl* ctl;

@@ -67,16 +67,17 @@ constexpr bool kBatched = SWP_BATCHED != 0;
 // shared memory rather than the constant bank; its block shapes trade
 // registers per thread (spills at 1024 threads, 64 registers) against warps
 // per SM, and SwapBatch.autotune times them on the batch at hand.  The
-// single-system kernel runs 768 threads (80 registers): its resident step
+// single-system kernel runs 768 threads in FP32 (80 registers: its resident step
 // keeps a thread's row, the integrator's state and the pair arithmetic in
-// registers at once.
+// registers at once) and 512 in FP64 (128 registers: eight warps fill the FP64
+// pipe, and spills cost more than more warps bring).
 #if SWP_BATCHED
 constexpr int kThreads = SWP_BATCH_THREADS;
 constexpr int kMinBlocks = SWP_BATCH_MINB;
 #elif SWP_WIDE
 constexpr int kThreads = kBlockWide;
 #else
-constexpr int kThreads = kBlock;
+constexpr int kThreads = SWP_BLOCK;
 #endif
 
 // ---------------------------------------------------------------------------
@@ -476,21 +477,27 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float bh, float bl)
 }
 
 // Block sums of the per-thread thermo accumulators (energies, virial, bond
-// count), added to the block's FP64 running sums blk[q]; with out given,
-// blk[q] is then written to out[q] (the block's partial of the pass) and
-// cleared.  Each thread holds the terms of one sub-chunk at most (multi-chunk
-// passes flush after every sub-chunk), so the error does not grow with the
-// system size; block partials are summed over blocks in FP64
-// (run_reduce_thermo).
+// count), written to out[q] (the block's partial of the pass; block partials
+// are summed over blocks in FP64, run_reduce_thermo).
 //
-// FP32 runs: each warp folds its lanes' values by a shuffle tree (at most five
-// roundings of the warp's sum of magnitudes) into s_wpart[q][warp]; warp q
-// then sums quantity q over the block's warps compensated (double-float).
-// FP64 runs: the values are staged in shared memory (stage: kNQA x blockDim)
-// and warp q sums them in FP64.
+// FP32 two-barrier passes: a warp folds its lanes' terms after every 32
+// particles (a shuffle tree, at most five roundings of the sum of magnitudes),
+// lane q carries quantity q in FP64, and the warps meet in s_wacc in FP64
+// (block_sums_from_rows), so the error does not grow with the system size.
+//
+// FP64 passes: every thread's terms, staged in shared memory and summed by one
+// warp per quantity over the threads that had any (block_sums_from_threads;
+// with 13 particles on a block the sums over every thread's zeros were a tenth
+// of a step).
+//
+// The resident step: one row per thread, the warps' shuffle-tree sums in
+// s_wpart; warp q then sums quantity q over the block's warps compensated
+// (double-float).
+static __shared__ double s_wacc[32][kNQA];
 static __shared__ float s_wpart[kNQA][32];
 
-__device__ __forceinline__ float warp_sum(float x)
+template <typename T>
+__device__ __forceinline__ T warp_sum(T x)
 {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -504,15 +511,15 @@ __device__ __forceinline__ void warp_part(float x, int q)
     if ((threadIdx.x & 31) == 0) s_wpart[q][threadIdx.x >> 5] = x;
 }
 
-// Sums s_wpart over the block's warps into blk / out (see above); out2, when
-// given with out, gets the same values.  The caller orders the s_wpart writes
-// before and the next ones after (block_sums_from_warps: two __syncthreads).
-__device__ __forceinline__ void warp_sums_to(double* blk, double* out, double* out2)
+// Sums s_wpart over the block's warps into out (and out2, when given).  The
+// caller orders the s_wpart writes before and the next ones after
+// (block_sums_from_warps: two __syncthreads).
+__device__ __forceinline__ void warp_sums_to(double* out, double* out2)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     for (int q = warp; q < kNQ; q += nw) {  // quantity q by warp q mod nw (blocks of fewer warps)
         if (q >= kNQA) {
-            if (out && lane == 0) {
+            if (lane == 0) {
                 out[q] = 0.0;
                 if (out2) out2[q] = 0.0;
             }
@@ -525,61 +532,53 @@ __device__ __forceinline__ void warp_sums_to(double* blk, double* out, double* o
             df_add(hi, lo, h2, l2);
         }
         if (lane == 0) {
-            const double tot = blk[q] + ((double)hi + (double)lo);
-            if (out) {
-                out[q] = tot;
-                if (out2) out2[q] = tot;
-                blk[q] = 0.0;
-            } else {
-                blk[q] = tot;
-            }
+            const double tot = (double)hi + (double)lo;
+            out[q] = tot;
+            if (out2) out2[q] = tot;
         }
     }
 }
 
-__device__ __forceinline__ void block_sums_from_warps(double* blk, double* out, double* out2 = nullptr)
+__device__ __forceinline__ void block_sums_from_warps(double* out, double* out2)
 {
     __syncthreads();
-    warp_sums_to(blk, out, out2);
+    warp_sums_to(out, out2);
     __syncthreads();
 }
 
-__device__ __forceinline__ void block_sums(const float* acc, float*, double* blk, double* out,
-                                           double* out2 = nullptr)
+// Sums s_wacc over the first nact warps (those that had particles; 0: none) into
+// out (and out2, when given).
+__device__ __forceinline__ void block_sums_from_rows(int nact, double* out, double* out2)
 {
-#pragma unroll
-    for (int q = 0; q < kNQA; q++) warp_part(acc[q], q);
-    block_sums_from_warps(blk, out, out2);
-}
-
-__device__ __forceinline__ void block_sums(const double* acc, double* stage, double* blk, double* out,
-                                           double* out2 = nullptr)
-{
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, B = blockDim.x, nw = (B + 31) >> 5;
-#pragma unroll
-    for (int q = 0; q < kNQA; q++) stage[q * B + t] = acc[q];
     __syncthreads();
-    for (int q = warp; q < kNQ; q += nw) {  // quantity q by warp q mod nw
-        if (q >= kNQA) {
-            if (out && lane == 0) {
-                out[q] = 0.0;
-                if (out2) out2[q] = 0.0;
-            }
-            continue;
-        }
-        double x = 0.0;
-        for (int k = lane; k < B; k += 32) x += stage[q * B + k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    for (int q = warp; q < kNQ; q += nw) {
+        double x = lane < nact && q < kNQA ? s_wacc[lane][q] : 0.0;
+        if (q < kNQA)
+            for (int o = 1; o < nact; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if (lane == 0) {
-            const double tot = blk[q] + x;
-            if (out) {
-                out[q] = tot;
-                if (out2) out2[q] = tot;
-                blk[q] = 0.0;
-            } else {
-                blk[q] = tot;
-            }
+            out[q] = x;
+            if (out2) out2[q] = x;
+        }
+    }
+    __syncthreads();
+}
+
+// FP64: the sums of stage[q][thread] over the first nact threads (the others'
+// terms are zero).
+__device__ __forceinline__ void block_sums_from_threads(const double* stage, int nact, double* out, double* out2)
+{
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, B = blockDim.x, nw = (B + 31) >> 5;
+    for (int q = warp; q < kNQ; q += nw) {
+        double x = 0.0;
+        if (q < kNQA) {
+            for (int k = lane; k < nact; k += 32) x += stage[q * B + k];
+            x = warp_sum(x);
+        }
+        if (lane == 0) {
+            out[q] = x;
+            if (out2) out2[q] = x;
         }
     }
     __syncthreads();
@@ -768,20 +767,31 @@ __device__ void ph_gather(const Dev<Real>& d, int pc, int ac, int t, int nt)
     }
 }
 
+// Every block's dynamic shared memory; the regions of its users (the list build,
+// the passes, the resident step) sit at compile-time offsets, so that every
+// access is a direct shared-memory access.
+extern __shared__ __align__(32) unsigned char g_dyn[];
+
 // ---------------------------------------------------------------------------
-// Block ownership and the compact neighbour list.
+// Block ownership and the neighbour list.
 //
 // Block b of a G-block launch owns the contiguous (Morton-ordered, hence
 // spatially compact) particle range [b*Pb, min((b+1)*Pb, n)), Pb = ceil(n/G),
 // processed in sub-chunks of at most blockDim.x particles.  The neighbour
 // entries of a sub-chunk are stored contiguously in the block's region of the
-// list buffer (capacity Pb * max_nn entries): first the reactive entries of
-// all its particles (in particle order), then the other entries.  Entry e
-// holds the partner slot ent_j[e] and the owner's index inside its sub-chunk
-// ent_o[e]; pinfo[p] = (first reactive entry, n_reactive, first other entry,
-// n_other).  The S and F passes then give one thread to one entry, so the
-// lanes of a warp neither idle on short rows nor diverge between the two
-// kinds of pair, and each owner thread sums its entries in entry order.
+// list buffer: first the reactive rows of all its particles, then the other
+// rows; entry e holds the partner slot ent_j[e], and pinfo[p] = (first reactive
+// entry, n_reactive, first other entry, n_other).  Entry positions are
+// unsigned 32-bit.
+//
+// FP32: one thread works through one particle's rows.  The threads of a
+// sub-chunk take its particles in descending order of (n_reactive, n_other),
+// so that the 32 rows of a warp have alike lengths (perm[q0 + t] = particle of
+// thread t, tinfo[q0 + t] = its pinfo); rows are stored in that order, each
+// padded with the particle's own slot to a multiple of four entries, so that a
+// thread loads its partners four at a time.
+// FP64: rows in particle order without padding, ent_o[e] = the owner's index
+// inside its sub-chunk (one lane works on one entry).
 
 template <typename Real>
 __device__ __forceinline__ void block_range(const Dev<Real>& d, int& b0, int& b1)
@@ -791,155 +801,211 @@ __device__ __forceinline__ void block_range(const Dev<Real>& d, int& b0, int& b1
     b1 = min(b0 + Pb, d.n);
 }
 
-// Builds the block's entries (last rebuild phase), one warp per cell: the warp
-// loads the 27 stencil ranges of its cell once, then tests its member
-// particles against the candidates 32 at a time with warp ballots.  A
-// counting sweep, a block scan that places every particle's runs (reactive
-// entries of the sub-chunk first, then the others), and a writing sweep;
-// candidates keep the stencil order, so the output is deterministic.
-// cnt: blockDim.x int2 of shared memory.  Returns the block's entry count
-// per particle (rounded up), the row length a capacity check needs.
-template <typename Real>
-__device__ __forceinline__ int rank_of(const Dev<Real>& d, const typename Dev<Real>::P4& p)
+// Stable counting sort, largest key first, of one item per thread (key in
+// [0, 255], -1: no item): returns the item's rank.  Equal keys keep the thread
+// order.  wh: scratch of blockDim / 32 x 256 u16 counts; hist: 256 ints; sh:
+// block_excl_scan's scratch; blockDim >= 256.
+static __device__ int rank_desc(int key, unsigned short* wh, int* hist, int* sh)
 {
-    int cx, cy, cz;
-    cell_coords(d, p, cx, cy, cz);
-    return __ldg(&d.cell_rank[(cz * d.nc[1] + cy) * d.nc[0] + cx]);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, NW = blockDim.x >> 5;
+    __syncthreads();  // a previous call's readers are done with wh and hist
+    for (int k = t; k < NW * 256; k += blockDim.x) wh[k] = 0;
+    __syncthreads();
+    // the warp's lanes with this key, and how many come before this lane
+    const unsigned m = __match_any_sync(0xffffffffu, key);
+    const int before = __popc(m & ((1u << lane) - 1u));
+    if (key >= 0 && before == 0) wh[warp * 256 + key] = (unsigned short)__popc(m);
+    __syncthreads();
+    // per key: the counts of the warps before each warp, and the key's total
+    if (t < 256) {
+        int run = 0;
+        for (int w = 0; w < NW; w++) {
+            const int c = wh[w * 256 + t];
+            wh[w * 256 + t] = (unsigned short)run;
+            run += c;
+        }
+        hist[t] = run;
+    }
+    __syncthreads();
+    // keys in descending order: the first rank of key b is the count above it
+    const int b = 255 - t;
+    int tot;
+    const int ex = block_excl_scan(t < 256 ? hist[b] : 0, sh, &tot);
+    if (t < 256) hist[b] = ex;  // every thread read hist before the scan's barriers
+    __syncthreads();
+    return key >= 0 ? hist[key] + wh[warp * 256 + key] + before : 0;
 }
 
-template <typename Real>
-__device__ int ph_build_cells(const Dev<Real>& d, const PairP<Real>* tab, int pc, int2* cnt,
-                              int* sh, int* overflow)
+// Shared-memory scratch of the list build.
+struct BuildStage {
+    static constexpr int kCap = 24;  // partners a thread holds before they are placed
+    static constexpr size_t B = kThreads;
+    static constexpr size_t O_HITS = 0;                       // [kCap][B] partner slots: reactive from the front, others from the back
+    static constexpr size_t O_CNT = O_HITS + kCap * B * 4;    // [B] int2 row lengths, then row starts, by particle
+    static constexpr size_t O_SIZE = O_CNT + B * 8;           // [B] int2 row sizes, then places, by thread order
+    static constexpr size_t O_WH = O_SIZE + B * 8;            // rank_desc's scratch
+    static constexpr size_t O_HIST = O_WH + B / 32 * 512;
+    static constexpr size_t kBytes = O_HIST + 1024;
+};
+
+// One lane's share [c0, c1) of the 27 stencil cells of particle i (cell cx, cy,
+// cz): hit(q, reactive) for every partner q inside the list radius, in stencil
+// order.  The next cell's range is loaded while the present one's candidates
+// are tested, two at a time.
+template <typename Real, typename F>
+__device__ __forceinline__ void sweep_cells(const Dev<Real>& d, const PairP<Real>* row, const typename Dev<Real>::P4* pos,
+                                            const typename Dev<Real>::P4& pi, int i, int cx, int cy, int cz, int c0,
+                                            int c1, F&& hit)
 {
     typedef typename Dev<Real>::P4 P4;
-    constexpr int NCH = 4;  // candidate chunks of 32 held at once
+    auto range = [&](int c, int& s, int& e) {
+        int x = cx + c % 3 - 1, y = cy + (c / 3) % 3 - 1, z = cz + c / 9 - 1;
+        x = x < 0 ? x + d.nc[0] : (x >= d.nc[0] ? x - d.nc[0] : x);
+        y = y < 0 ? y + d.nc[1] : (y >= d.nc[1] ? y - d.nc[1] : y);
+        z = z < 0 ? z + d.nc[2] : (z >= d.nc[2] ? z - d.nc[2] : z);
+        const int r = __ldg(&d.cell_rank[(z * d.nc[1] + y) * d.nc[0] + x]);
+        s = d.cell_start[r];
+        e = d.cell_start[r + 1];
+    };
+    auto test = [&](int q, const P4& pj) {
+        const PairP<Real>& p = row[type_of(pj)];
+        Real dx, dy, dz;
+        if (q != i && dist2(pi, pj, d, dx, dy, dz) < p.rlist2) hit(q, p.kind == KIND_SWAP);
+    };
+    int s = 0, e = 0;
+    if (c0 < c1) range(c0, s, e);
+    for (int c = c0; c < c1; c++) {
+        const int s0 = s, e0 = e;
+        if (c + 1 < c1) range(c + 1, s, e);
+        for (int q = s0; q < e0; q += 2) {
+            const bool two = q + 1 < e0;
+            const P4 pa = pos[q], pb = pos[two ? q + 1 : q];
+            test(q, pa);
+            if (two) test(q + 1, pb);
+        }
+    }
+}
+
+// Builds the block's rows (last rebuild phase).  G lanes (a power of two, as
+// many as the block's particles leave) share a particle: each tests the
+// candidates of its share of the 27 stencil cells and keeps the partners it
+// finds in shared memory; the sub-chunk's rows are then placed and written, in
+// stencil order whatever G is.  (Rows longer than the lanes can hold: the
+// cells are gone through once more to write them.)  One warp per cell with the
+// candidates across the lanes, in a counting and a writing sweep, spent 540
+// warp instructions per particle, most of them on handing out candidates and
+// on ballots: 2.8 -> 1.0 ms per build at 2M beads.
+// Returns the block's entry count per particle (rounded up), the row length a
+// capacity check needs.
+template <typename Real>
+__device__ int ph_build_rows(const Dev<Real>& d, const PairP<Real>* tab, int pc, int* sh, int* overflow)
+{
+    typedef typename Dev<Real>::P4 P4;
+    typedef BuildStage BS;
+    constexpr bool kRows = sizeof(Real) == 4;  // sorted and padded rows
     const P4* pos = d.pos[pc];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
+    int* hits = (int*)(g_dyn + BS::O_HITS);
+    int2* cnt = (int2*)(g_dyn + BS::O_CNT);
+    int2* size = (int2*)(g_dyn + BS::O_SIZE);
+    const int t = threadIdx.x, B = blockDim.x;
     int b0, b1;
     block_range(d, b0, b1);
     const int Pb = (d.n + g_size() - 1) / g_size();
-    const long long cap_beg = (long long)g_rank() * Pb * d.max_nn;
-    const long long cap_end = cap_beg + (long long)Pb * d.max_nn;
-    long long base = cap_beg;
-    for (int q0 = b0; q0 < b1; q0 += blockDim.x) {
-        const int q1 = min(q0 + (int)blockDim.x, b1);
-        const int P = q1 - q0;
-        const int r_lo = rank_of(d, pos[q0]);
-        const int r_hi = rank_of(d, pos[q1 - 1]);
-        if ((int)threadIdx.x < P) cnt[threadIdx.x] = make_int2(0, 0);
-        __syncthreads();
-        bool fits = true;
-        for (int pass = 0; pass < 2; pass++) {
-            if (pass == 1) {
-                // place the runs: reactive entries of the sub-chunk, then the others
-                const int t = threadIdx.x;
-                const int2 c = t < P ? cnt[t] : make_int2(0, 0);
-                int Er, Ew;
-                const int offr = block_excl_scan(c.x, sh, &Er);
-                const int offw = block_excl_scan(c.y, sh, &Ew);
-                fits = base + Er + Ew <= cap_end;
-                if (t < P) {
-                    const int ro = (int)(base + offr), wo = (int)(base + Er + offw);
-                    d.pinfo[q0 + t] = make_int4(ro, c.x, wo, c.y);
-                    cnt[t] = make_int2(ro, wo);  // running write positions
-                }
-                if (!fits && t == 0) *overflow = 1;
-                base += Er + Ew;
-                __syncthreads();
-                if (!fits) break;
+    // the block's region: list_stride entries per particle (max_nn and the padding)
+    long long base = (long long)g_rank() * Pb * d.list_stride;
+    long long used = 0;  // entries without padding
+    for (int q0 = b0; q0 < b1; q0 += B) {
+        const int P = min(B, b1 - q0);
+        int lg = 0;
+        while (lg < 5 && (P << (lg + 1)) <= B) lg++;
+        const int G = 1 << lg, g = t & (G - 1), pl = t >> lg;
+        const bool has = pl < P;
+        const int i = q0 + (has ? pl : 0);
+        const P4 pi = pos[i];
+        const PairP<Real>* row = tab + type_of(pi) * d.ntypes;
+        int cx, cy, cz;
+        cell_coords(d, pi, cx, cy, cz);
+        const int c0 = has ? 27 * g / G : 0, c1 = has ? 27 * (g + 1) / G : 0;
+        int nr = 0, nw = 0;
+        sweep_cells(d, row, pos, pi, i, cx, cy, cz, c0, c1, [&](int q, bool react) {
+            if (nr + nw < BS::kCap) hits[(react ? nr : BS::kCap - 1 - nw) * B + t] = q;
+            nr += react;
+            nw += !react;
+        });
+        // the lane's place in its particle's rows, and the rows' lengths
+        int er = nr, ew = nw;
+        for (int o = 1; o < G; o <<= 1) {
+            const int a = __shfl_up_sync(0xffffffffu, er, o, G), b = __shfl_up_sync(0xffffffffu, ew, o, G);
+            if (g >= o) {
+                er += a;
+                ew += b;
             }
-            for (int r = r_lo + warp; r <= r_hi; r += nwarps) {
-                const int m0 = max(d.cell_start[r], q0), m1 = min(d.cell_start[r + 1], q1);
-                if (m0 >= m1) continue;
-                // the 27 stencil ranges (lane l < 27 holds range l)
-                const int lin = __ldg(&d.cell_rank[d.ncell + r]);
-                const int cx = lin % d.nc[0], cy = (lin / d.nc[0]) % d.nc[1], cz = lin / (d.nc[0] * d.nc[1]);
-                int s = 0, len = 0;
-                if (lane < 27) {
-                    int x = cx + lane % 3 - 1, y = cy + (lane / 3) % 3 - 1, z = cz + lane / 9 - 1;
-                    x = x < 0 ? x + d.nc[0] : (x >= d.nc[0] ? x - d.nc[0] : x);
-                    y = y < 0 ? y + d.nc[1] : (y >= d.nc[1] ? y - d.nc[1] : y);
-                    z = z < 0 ? z + d.nc[2] : (z >= d.nc[2] ? z - d.nc[2] : z);
-                    const int rr = __ldg(&d.cell_rank[(z * d.nc[1] + y) * d.nc[0] + x]);
-                    s = d.cell_start[rr];
-                    len = d.cell_start[rr + 1] - s;
+        }
+        const int tr = __shfl_sync(0xffffffffu, er, G - 1, G), tw = __shfl_sync(0xffffffffu, ew, G - 1, G);
+        er -= nr;
+        ew -= nw;
+        if (has && g == 0) cnt[pl] = make_int2(tr, tw);
+        const bool again = __syncthreads_or(nr + nw > BS::kCap);
+        // places: the reactive rows of the sub-chunk, then the others, in thread order
+        const int2 c = t < P ? cnt[t] : make_int2(0, 0);
+        int rk = t;
+        if (kRows)
+            rk = rank_desc(t < P ? (min(c.x, 15) << 4 | min(c.y, 15)) : -1, (unsigned short*)(g_dyn + BS::O_WH),
+                           (int*)(g_dyn + BS::O_HIST), sh);
+        if (kRows && ((q0 - b0) / B & 1)) rk = P - 1 - rk;  // every warp gets long and short rows in turn
+        const int pad = kRows ? 3 : 0;
+        if (t < P) size[rk] = make_int2((c.x + pad) & ~pad, (c.y + pad) & ~pad);
+        __syncthreads();
+        const int2 z = t < P ? size[t] : make_int2(0, 0);
+        int Er, Ew, Ec;
+        const int offr = block_excl_scan(z.x, sh, &Er);
+        const int offw = block_excl_scan(z.y, sh, &Ew);
+        block_excl_scan(c.x + c.y, sh, &Ec);
+        if (t < P) size[t] = make_int2(offr, offw);
+        __syncthreads();
+        used += Ec;
+        const bool fits = used <= (long long)Pb * d.max_nn;
+        if (fits) {
+            if (t < P) {
+                const int2 o = size[rk];
+                const int ro = (int)(unsigned)(base + o.x), wo = (int)(unsigned)(base + Er + o.y);
+                const int4 inf = make_int4(ro, c.x, wo, c.y);
+                d.pinfo[q0 + t] = inf;
+                if constexpr (kRows) {
+                    d.tinfo[q0 + rk] = inf;
+                    d.perm[q0 + rk] = q0 + t;
                 }
-                int pre = len;  // inclusive prefix over the lanes
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, pre, o);
-                    if (lane >= o) pre += y;
-                }
-                const int C = __shfl_sync(0xffffffffu, pre, 31);
-                for (int g0 = 0; g0 < C; g0 += 32 * NCH) {
-                    // this group's candidates: slot and position per lane and chunk.
-                    // Candidate tc lies in the range idx = number of ranges that end
-                    // at or before it; every lane runs every shuffle (no divergence).
-                    int cq[NCH];
-                    P4 cp[NCH];
-                    int idx[NCH];
-#pragma unroll
-                    for (int k = 0; k < NCH; k++) idx[k] = 0;
-                    for (int l = 0; l < 27; l++) {
-                        const int pl = __shfl_sync(0xffffffffu, pre, l);
-#pragma unroll
-                        for (int k = 0; k < NCH; k++) idx[k] += (pl <= g0 + 32 * k + lane) ? 1 : 0;
-                    }
-#pragma unroll
-                    for (int k = 0; k < NCH; k++) {
-                        const int tc = g0 + 32 * k + lane;
-                        const int rg = min(idx[k], 26);
-                        const int sl = __shfl_sync(0xffffffffu, s, rg);
-                        const int pb = __shfl_sync(0xffffffffu, pre - len, rg);
-                        cq[k] = tc < C ? sl + (tc - pb) : -1;
-                    }
-#pragma unroll
-                    for (int k = 0; k < NCH; k++)
-                        if (cq[k] >= 0) cp[k] = pos[cq[k]];
-                    for (int i = m0; i < m1; i++) {
-                        const P4 pi = pos[i];
-                        const int ti = type_of(pi);
-                        int2 run = cnt[i - q0];
-#pragma unroll
-                        for (int k = 0; k < NCH; k++) {
-                            bool react = false, other = false;
-                            if (cq[k] >= 0 && cq[k] != i) {
-                                const PairP<Real>& p = tab[ti * d.ntypes + type_of(cp[k])];
-                                Real dx, dy, dz;
-                                if (dist2(pi, cp[k], d, dx, dy, dz) < p.rlist2) {
-                                    react = p.kind == KIND_SWAP;
-                                    other = !react;
-                                }
-                            }
-                            const unsigned br = __ballot_sync(0xffffffffu, react);
-                            const unsigned bw = __ballot_sync(0xffffffffu, other);
-                            if (pass == 1) {
-                                if (react) {
-                                    const int e = run.x + __popc(br & lt);
-                                    d.ent_j[e] = cq[k];
-                                    d.ent_o[e] = (unsigned short)(i - q0);
-                                }
-                                if (other) {
-                                    const int e = run.y + __popc(bw & lt);
-                                    d.ent_j[e] = cq[k];
-                                    d.ent_o[e] = (unsigned short)(i - q0);
-                                }
-                            }
-                            run.x += __popc(br);
-                            run.y += __popc(bw);
-                        }
-                        __syncwarp();
-                        if (lane == 0) cnt[i - q0] = run;
-                        __syncwarp();
-                    }
-                }
+                cnt[t] = make_int2(ro, wo);
             }
             __syncthreads();
+            if (has) {
+                const unsigned ro = (unsigned)cnt[pl].x, wo = (unsigned)cnt[pl].y;
+                unsigned kr = ro + er, kw = wo + ew;
+                auto put = [&](unsigned& k, int q) {
+                    d.ent_j[k] = q;
+                    if constexpr (!kRows) d.ent_o[k] = (unsigned short)pl;
+                    k++;
+                };
+                if (!again) {
+                    for (int k = 0; k < nr; k++) put(kr, hits[k * B + t]);
+                    for (int k = 0; k < nw; k++) put(kw, hits[(BS::kCap - 1 - k) * B + t]);
+                } else {
+                    sweep_cells(d, row, pos, pi, i, cx, cy, cz, c0, c1,
+                                [&](int q, bool react) { put(react ? kr : kw, q); });
+                }
+                if (kRows && g == G - 1) {
+                    while (kr & 3u) put(kr, i);  // rows start at multiples of four
+                    while (kw & 3u) put(kw, i);
+                }
+            }
+        } else if (t == 0) {
+            *overflow = 1;
         }
+        base += Er + Ew;
+        __syncthreads();  // cnt, size and hits are free
     }
     const int np = b1 - b0;
-    return np > 0 ? (int)((base - cap_beg + np - 1) / np) : 0;
+    return np > 0 ? (int)((used + np - 1) / np) : 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -954,36 +1020,64 @@ __device__ __forceinline__ const PairP<Real>& pair_of(const PairP<Real>* tab, in
     return UNI ? uni : tab[ti * nt + tj];
 }
 
-// Shared-memory staging of one sub-chunk (dynamic shared memory): the
-// sub-chunk's own particles and the per-entry results of one wave.  The
-// regions sit at compile-time offsets from one namespace-scope extern
-// __shared__ array, so every access is a direct shared-memory access.
-extern __shared__ __align__(32) unsigned char g_dyn[];
+// The two-barrier passes: nothing in a pass waits for another warp, so that one
+// warp's gathers overlap the arithmetic of the others.
+//
+// FP32 (s_pass_rows, f_pass_rows): one thread per particle, in the order of
+// the build (alike rows in a warp).  A thread loads its partners four at a
+// time and gathers them together.  An entry-parallel version (one lane per
+// entry, results through shared memory to the owners) spent 2,900 warp
+// instructions per 32 particles and step, this one 1,700; block barriers around
+// 768-particle waves before that: mix of 1M particles 197 ->
+// 125 us per step, 20-step launches with a list build in each.
+//
+// FP64 (s_pass_waves, f_pass_waves): the bound is the FP64 pipe, which takes 19
+// cycles per warp instruction on the whole SM however many of its lanes are on
+// (24 warps; one warp alone 64).  So every FP64 instruction is given as many
+// lanes as there are, and pairs that cannot contribute none: the block sorts
+// out a wave of entries with FP32 distances (conservative, see may_reach: half
+// of the listed pairs lie in the skin), lines up the rest, evaluates them one
+// per thread, and the owners sum the rows.  The reactive pairs' values of the S
+// pass are kept in shared memory for the force pass where they fit.  (Every
+// listed entry evaluated, twice if reactive, took
+// 57 us per step of 20,000 particles and 31 of 2,000, this takes 28 and 20.)
 
+constexpr int kBeyond = 1 << 15;  // FP64: marks a lined-up entry, a kept pair outside r_min
+
+// Shared-memory staging of the passes: slot t holds thread t's particle (FP32,
+// in the threads' order) or particle t of the sub-chunk (FP64).
 template <typename Real>
 struct Stage {
     typedef typename Dev<Real>::R4 R4;
     typedef typename Dev<Real>::P4 P4;
-    // entries per wave: 8 (FP32) or 3 (FP64) per thread of a batched block shape
-    static constexpr int kWave = kBatched ? (sizeof(Real) == 4 ? 8 : 3) * kThreads : (sizeof(Real) == 4 ? 8192 : 3072);
+    static constexpr bool kWaves = sizeof(Real) == 8;
+    static constexpr int kWave = !kWaves ? 0 : kThreads > 512 ? 2048 : 3072;  // entries of a wave
     static constexpr size_t B = kThreads;
     static constexpr size_t O_POS = 0;                                  // [B] P4 positions
     static constexpr size_t O_VEL = O_POS + B * sizeof(P4);             // [B] R4 velocities
     static constexpr size_t O_XQ = O_VEL + B * sizeof(R4);              // [3B] fixed-point positions
-    static constexpr size_t O_INFO = O_XQ + 3 * B * sizeof(long long);  // [B] int4 pinfo
+    static constexpr size_t O_INFO = O_XQ + 3 * B * sizeof(long long);  // [B] int4 list ranges
     static constexpr size_t O_S = O_INFO + B * sizeof(int4);            // [B] S
-    static constexpr size_t O_W = O_S + B * sizeof(Real);               // [kWave] R4 entry results
-    static constexpr size_t kBytes = O_W + (size_t)kWave * sizeof(R4);
-    static size_t bytes(int) { return kBytes; }
+    static constexpr size_t O_IDX = O_S + B * sizeof(Real);             // FP32: [B] particle slots
+    static constexpr size_t O_W = O_IDX + (kWaves ? 0 : B * 4);         // FP64: [3][kWave] entry results
+    static constexpr size_t O_LIST = O_W + (size_t)kWave * 24;          // [kWave] int2 entries lined up (entry of the
+                                                                        // wave | owner << 16, partner)
+    static constexpr size_t O_KEEP = O_LIST + (size_t)kWave * 8;        // [6][kKeep] reactive pairs' values
+    static constexpr int kKeep = !kWaves ? 0 : (int)((212 * 1024 - O_KEEP) / 48);
+    static constexpr size_t kPassBytes = O_KEEP + (size_t)kKeep * 48;
+    static_assert(kWave <= kBeyond, "an entry of the wave in 15 bits");
+    static_assert(!kWaves || kPassBytes - O_W >= kNQA * B * 8, "the thermo terms fit behind the particles' state");
+    static constexpr size_t kBytes = kPassBytes > BuildStage::kBytes ? kPassBytes : BuildStage::kBytes;
 
     static __device__ __forceinline__ P4* pos() { return (P4*)(g_dyn + O_POS); }
     static __device__ __forceinline__ R4* vel() { return (R4*)(g_dyn + O_VEL); }
     static __device__ __forceinline__ long long* xq() { return (long long*)(g_dyn + O_XQ); }
     static __device__ __forceinline__ int4* info() { return (int4*)(g_dyn + O_INFO); }
     static __device__ __forceinline__ Real* S() { return (Real*)(g_dyn + O_S); }
+    static __device__ __forceinline__ int* idx() { return (int*)(g_dyn + O_IDX); }
     static __device__ __forceinline__ Real* w() { return (Real*)(g_dyn + O_W); }
-    static __device__ __forceinline__ R4* w4() { return (R4*)(g_dyn + O_W); }
-    static constexpr int wave = kWave;
+    static __device__ __forceinline__ int2* list() { return (int2*)(g_dyn + O_LIST); }
+    static __device__ __forceinline__ Real* keep() { return (Real*)(g_dyn + O_KEEP); }
 };
 
 // Asynchronous global -> shared copies (no register staging).
@@ -1029,112 +1123,259 @@ __device__ __forceinline__ Real s_term(const Dev<Real>& d, const PairP<Real>* ta
     return r2 < p.rc2 ? mul_rn(p.a, vh) : Real(0);
 }
 
-// End of the block's region of the list (entries of its particles are
-// placed inside [rank * Pb * max_nn, (rank + 1) * Pb * max_nn)).
-template <typename Real>
-__device__ __forceinline__ long long block_list_end(const Dev<Real>& d)
+// Brings the first line of each of a thread's rows into L2 (the rows of a warp
+// are neighbours) while the warp works on other entries.
+__device__ __forceinline__ void prefetch_row(const Dev<float>& d, int first)
 {
-    const long long Pb = (d.n + g_size() - 1) / g_size();
-    return (long long)(g_rank() + 1) * Pb * d.max_nn;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(&d.ent_j[(unsigned)first]));
 }
 
-// Brings list entries [e0, e1) (partner slots and owner indices) into L2, one
-// 128-byte line per thread, while the block works on other entries.
-template <typename Real>
-__device__ __forceinline__ void prefetch_entries(const Dev<Real>& d, long long e0, long long e1)
+__device__ __forceinline__ int4 load_four(const Dev<float>& d, int first, int k)
 {
-    if (e1 <= e0) return;
-    const long long nj = ((e1 - 1) >> 5) - (e0 >> 5) + 1;  // 32 partner slots per line
-    const long long no = ((e1 - 1) >> 6) - (e0 >> 6) + 1;  // 64 owner indices per line
-    for (long long k = threadIdx.x; k < nj + no; k += blockDim.x) {
-        const void* p = k < nj ? (const void*)&d.ent_j[max(((e0 >> 5) + k) << 5, e0)]
-                               : (const void*)&d.ent_o[max(((e0 >> 6) + k - nj) << 6, e0)];
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-    }
+    return __ldcs((const int4*)&d.ent_j[(unsigned)first + (unsigned)k]);  // streamed: keep L2 for the snapshots
 }
 
-// Entries per thread whose gathers a two-barrier pass issues together (S
-// pass, force pass).
-constexpr int kGather = 4;
-constexpr int kGatherF = 2;
-
-// staged: the block has one sub-chunk and the shared copies of its positions
-// and list ranges are current (kept by the previous force pass), so they are
-// not loaded again.  With one sub-chunk the block's S values also stay in
-// shared memory for the force pass.
-template <typename Real, bool UNI>
-__device__ void s_pass_block(const Dev<Real>& d, const PairP<Real>* tab, int pc,
-                             const PairP<Real>& ps, bool staged)
+// FP32.  staged: the block has one sub-chunk and the shared copies of its
+// positions and list ranges are current (kept by the previous force pass), so
+// they are not loaded again; its S values also stay in shared memory for the
+// force pass.
+template <bool UNI>
+__device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc, const PairP<float>& ps, bool staged)
 {
-    typedef Stage<Real> SM;
-    typedef typename Dev<Real>::P4 P4;
-    const P4* pos = d.pos[pc];
+    typedef Stage<float> SM;
+    const int4* pos = d.pos[pc];
     int b0, b1;
     block_range(d, b0, b1);
     const int t = threadIdx.x;
-    const bool single = b1 - b0 <= (int)blockDim.x;
-    for (int q0 = b0; q0 < b1; q0 += blockDim.x) {
-        const int P = min((int)blockDim.x, b1 - q0);
-        if (!staged) {
-            if (t < P) {
-                SM::pos()[t] = pos[q0 + t];
-                SM::info()[t] = d.pinfo[q0 + t];
-            }
-            __syncthreads();
+    const bool single = b1 - b0 <= kThreads;
+    if (t >= b1 - b0) return;
+    // what the thread's next row needs is loaded while it works on the present one
+    int4 ti, pi;
+    int i;
+    if (staged) {
+        ti = SM::info()[t];
+        i = SM::idx()[t];
+        pi = SM::pos()[t];
+    } else {
+        ti = d.tinfo[b0 + t];
+        i = d.perm[b0 + t];
+        pi = pos[i];
+        if (single) {
+            SM::info()[t] = ti;
+            SM::idx()[t] = i;
+            SM::pos()[t] = pi;
         }
-        const int e_beg = SM::info()[0].x;
-        const int e_end = SM::info()[P - 1].x + SM::info()[P - 1].y;
-        {
-            // into L2 while this sub-chunk runs: the next sub-chunk's reactive
-            // entries (sized like this one's), or after the last one the
-            // block's first sub-chunk, which the force pass starts with
-            const int4 last = SM::info()[P - 1];
-            const long long full = (long long)last.z + last.w;
-            const long long cap = block_list_end(d);
-            if (q0 + P < b1)
-                prefetch_entries(d, full, min(full + (e_end - e_beg), cap));
-            else {
-                const long long f0 = cap - (long long)((d.n + g_size() - 1) / g_size()) * d.max_nn;
-                prefetch_entries(d, f0, min(f0 + (full - e_beg), cap));
+    }
+    int4 jn = ti.y > 0 ? load_four(d, ti.x, 0) : make_int4(0, 0, 0, 0);
+    for (int q = b0 + t; q < b1; q += kThreads) {
+        const int qn = q + kThreads;
+        int4 tn = make_int4(0, 0, 0, 0);
+        int in = i;
+        if (qn < b1) {
+            tn = d.tinfo[qn];
+            in = d.perm[qn];
+        }
+        // groups of four, then one by one: the order of every path
+        float s = 0.0f;
+        const int cnt = ti.y;
+        for (int k = 0; k < cnt; k += 4) {
+            const int4 j = jn;
+            if (k + 4 < cnt) jn = load_four(d, ti.x, k + 4);
+            const int4 p0 = pos[j.x], p1 = pos[j.y], p2 = pos[j.z], p3 = pos[j.w];  // padding: the own slot
+            const float w0 = s_term<float, UNI>(d, tab, ps, pi, p0);
+            if (k + 4 <= cnt) {
+                const float w1 = s_term<float, UNI>(d, tab, ps, pi, p1);
+                const float w2 = s_term<float, UNI>(d, tab, ps, pi, p2);
+                const float w3 = s_term<float, UNI>(d, tab, ps, pi, p3);
+                s += (w0 + w1) + (w2 + w3);
+            } else {
+                s += w0;
+                if (k + 1 < cnt) s += s_term<float, UNI>(d, tab, ps, pi, p1);
+                if (k + 2 < cnt) s += s_term<float, UNI>(d, tab, ps, pi, p2);
             }
         }
-        Real s = Real(0);
-        for (int wb = e_beg; wb < e_end; wb += SM::wave) {
-            const int we = min(wb + SM::wave, e_end);
-            // the thread's entries e, e + B, ... in groups of kGather: the group's
-            // index loads, then its partner gathers, are independent of one
-            // another, so that many are in flight when the partners come from DRAM
-            const int B = blockDim.x;
-            for (int e0 = wb + t; e0 < we; e0 += kGather * B) {
-                int jj[kGather], oo[kGather];
+        d.S[i] = s;
+        if (single) SM::S()[t] = s;
+        if (qn < b1) {
+            ti = tn;
+            i = in;
+            pi = pos[i];
+            if (ti.y > 0) jn = load_four(d, ti.x, 0);
+            // the row after that, into L2
+            if (qn + kThreads < b1) prefetch_row(d, d.tinfo[qn + kThreads].x);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 waves.
+
+static __shared__ int s_nlist;  // entries lined up
+static __shared__ int s_nkeep;  // reactive pairs whose values the S pass kept (-1: not kept)
+
+// The float below a non-negative double, from its bits (the conversion
+// instruction runs on the FP64 pipe).
+__device__ __forceinline__ float float_below(double x)
+{
+    return __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), (unsigned)max(__double2hiint(x) - 0x38000000, 0), 3));
+}
+
+// Whether a listed pair may lie inside its cut-off (p.reach2: the cut-off plus
+// 2^-18 of the box, far above the error of these FP32 distances, squared).
+__device__ __forceinline__ bool may_reach(const Dev<double>& d, const dbl4& pi, const dbl4& pj, float reach2)
+{
+    const double xi[3] = {pi.x, pi.y, pi.z}, xj[3] = {pj.x, pj.y, pj.z};
+    float r2 = 0.0f;
 #pragma unroll
-                for (int u = 0; u < kGather; u++) {
-                    const int e = e0 + u * B;
-                    jj[u] = e < we ? __ldcs(&d.ent_j[e]) : 0;  // streamed: keep L2 for the snapshots
-                    oo[u] = e < we ? __ldcs(&d.ent_o[e]) : 0;
-                }
-                P4 pp[kGather];
+    for (int c = 0; c < 3; c++) {
+        float dx = float_below(xj[c]) - float_below(xi[c]);
+        dx = fmaf(-d.Lf[c], rintf(dx * d.iLf[c]), dx);
+        r2 = fmaf(dx, dx, r2);
+    }
+    return r2 < reach2;
+}
+
+// dist2_listed with the wrap, 9 of its 17 FP64 instructions, left to the pairs
+// across a face (|dx| below half an edge wraps by zero): the same bits.
+__device__ __forceinline__ double dist2_near(const dbl4& pi, const dbl4& pj, const Dev<double>& d, double& dx,
+                                             double& dy, double& dz)
+{
+    dx = sub_rn(pj.x, pi.x);
+    dy = sub_rn(pj.y, pi.y);
+    dz = sub_rn(pj.z, pi.z);
+    auto far = [](double v, double h) { return (__double2hiint(v) & 0x7fffffff) >= __double2hiint(h); };
+    if (far(dx, d.hL[0]) | far(dy, d.hL[1]) | far(dz, d.hL[2])) {
+        dx = wrap_rint(dx, d.L[0], d.iL[0]);
+        dy = wrap_rint(dy, d.L[1], d.iL[1]);
+        dz = wrap_rint(dz, d.L[2], d.iL[2]);
+    }
+    double s = mul_rn(dx, dx);
+    s = add_rn(s, mul_rn(dy, dy));
+    return add_rn(s, mul_rn(dz, dz));
+}
+
+// Lines up the entries [e0, e1) that may lie inside their cut-off behind the
+// entries already in the list (any order: results go to the entries' places),
+// zeroes the wave's results of the others, and (react) of the lined-up ones
+// too.  nres: results per entry (1 or 3).  The caller's barrier completes it.
+template <bool UNI>
+__device__ __forceinline__ void line_up(const Dev<double>& d, const PairP<double>* tab, const PairP<double>& pu,
+                                        const dbl4* pos, unsigned wb, unsigned e0, unsigned e1, int nres)
+{
+    typedef Stage<double> SM;
+    const int lane = threadIdx.x & 31;
+    for (unsigned eb = e0 + (threadIdx.x & ~31u); eb < e1; eb += kThreads) {  // the same in the whole warp
+        const unsigned e = eb + lane;
+        bool in = false;
+        int j = 0, o = 0;
+        if (e < e1) {
+            j = d.ent_j[e];
+            o = d.ent_o[e];
+            const dbl4 pi = SM::pos()[o], pj = pos[j];
+            const PairP<double>& p = pair_of<double, UNI>(tab, type_of(pi), type_of(pj), d.ntypes, pu);
+            in = may_reach(d, pi, pj, p.reach2);
+            if (!in)
+                for (int c = 0; c < nres; c++) SM::w()[c * SM::kWave + (e - wb)] = 0.0;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        int base = 0;
+        if (lane == 0 && m) base = atomicAdd(&s_nlist, __popc(m));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (in) SM::list()[base + __popc(m & ((1u << lane) - 1u))] = make_int2((int)(e - wb) | o << 16, j);
+    }
+}
+
+// Adds the results at w[k - wb] of entries [k0, k1) to f in entry order.  Zeros
+// are passed over (they change nothing), each lane to its own next entry, so
+// that a warp's FP64 additions are as many as its longest row has pairs inside
+// the cut-off.
+template <int N>
+__device__ __forceinline__ void sum_row(const double* w, int k0, int k1, double (&f)[N])
+{
+    typedef Stage<double> SM;
+    int k = k0;
+    while (__any_sync(0xffffffffu, k < k1)) {
+        bool some = false;
+        while (k < k1 && !some) {
+            unsigned long long b = 0;
 #pragma unroll
-                for (int u = 0; u < kGather; u++) pp[u] = pos[jj[u]];  // slot 0 for a missing entry
+            for (int c = 0; c < N; c++) b |= (unsigned long long)__double_as_longlong(w[c * SM::kWave + k]);
+            some = (b << 1) != 0;  // +-0
+            k++;
+        }
+        __syncwarp();
+        if (some)
 #pragma unroll
-                for (int u = 0; u < kGather; u++) {
-                    const int e = e0 + u * B;
-                    if (e < we) SM::w()[e - wb] = s_term<Real, UNI>(d, tab, ps, SM::pos()[oo[u]], pp[u]);
-                }
-            }
+            for (int c = 0; c < N; c++) f[c] += w[c * SM::kWave + k - 1];
+    }
+}
+
+// S_i, summed in entry order.  staged: as in s_pass_rows.  th: the force pass
+// samples the energies (it needs the pair energies of the kept pairs).
+template <bool UNI>
+__device__ void s_pass_waves(const Dev<double>& d, const PairP<double>* tab, int pc, const PairP<double>& ps,
+                             bool staged, bool th)
+{
+    typedef Stage<double> SM;
+    const dbl4* pos = d.pos[pc];
+    int b0, b1;
+    block_range(d, b0, b1);
+    const int t = threadIdx.x;
+    const bool single = b1 - b0 <= kThreads;
+    if (t == 0) s_nkeep = -1;
+    for (int q0 = b0; q0 < b1; q0 += kThreads) {
+        const int P = min(kThreads, b1 - q0);
+        if (!staged && t < P) {
+            SM::pos()[t] = pos[q0 + t];
+            SM::info()[t] = d.pinfo[q0 + t];
+        }
+        if (t == 0) s_nlist = 0;
+        __syncthreads();
+        const int4 inf = SM::info()[min(t, P - 1)];
+        const int4 last = SM::info()[P - 1];
+        const unsigned e_beg = SM::info()[0].x, e_end = (unsigned)(last.x + last.y);
+        // the values are kept for the force pass when it takes the same wave
+        const bool keep = single && (unsigned)(last.z + last.w) - e_beg <= (unsigned)SM::kWave;
+        double s[1] = {0.0};
+        for (unsigned wb = e_beg; wb < e_end; wb += SM::kWave) {
+            const unsigned we = min(wb + SM::kWave, e_end);
+            line_up<UNI>(d, tab, ps, pos, wb, wb, we, 1);
             __syncthreads();
-            if (t < P) {
-                const int4 inf = SM::info()[t];
-                const int k0 = max(inf.x, wb), k1 = min(inf.x + inf.y, we);
-                int k = k0;
-                for (; k + 4 <= k1; k += 4) s += (SM::w()[k - wb] + SM::w()[k + 1 - wb]) + (SM::w()[k + 2 - wb] + SM::w()[k + 3 - wb]);
-                for (; k < k1; k++) s += SM::w()[k - wb];
+            const int m = s_nlist;
+            const bool kept = keep && m <= SM::kKeep;
+            for (int c = t; c < m; c += kThreads) {
+                const int2 it = SM::list()[c];
+                const int x = it.x & (kBeyond - 1);
+                const dbl4 pi = SM::pos()[it.x >> 16], pj = pos[it.y];
+                const PairP<double>& p = pair_of<double, UNI>(tab, type_of(pi), type_of(pj), d.ntypes, ps);
+                double dx, dy, dz, v, ft;
+                const double r2 = dist2_near(pi, pj, d, dx, dy, dz);
+                lj_eval(p, r2, v, ft);
+                const bool in = r2 < p.rc2;
+                const double vh = r2 > p.rmin2 ? (p.vshift - v) * p.inv_epshat : 1.0;
+                SM::w()[x] = in ? mul_rn(p.a, vh) : 0.0;
+                if (kept) {
+                    double* k = SM::keep() + c;
+                    k[0] = in ? ft : 0.0;
+                    k[SM::kKeep] = vh;
+                    k[2 * SM::kKeep] = dx;
+                    k[3 * SM::kKeep] = dy;
+                    k[4 * SM::kKeep] = dz;
+                    if (th) k[5 * SM::kKeep] = v;
+                    if (r2 > p.rmin2) SM::list()[c].x = it.x | kBeyond;
+                }
             }
+            if (kept && t == 0) s_nkeep = m;
+            __syncthreads();
+            const unsigned r0 = (unsigned)inf.x, r1 = r0 + (unsigned)inf.y;
+            const bool on = t < P && r1 > wb && r0 < we;
+            sum_row(SM::w(), on ? (int)(max(r0, wb) - wb) : 0, on ? (int)(min(r1, we) - wb) : 0, s);
+            if (t == 0 && !kept) s_nlist = 0;
             __syncthreads();
         }
         if (t < P) {
-            d.S[q0 + t] = s;
-            if (single) SM::S()[t] = s;
+            d.S[q0 + t] = s[0];
+            if (single) SM::S()[t] = s[0];
         }
     }
 }
@@ -1315,42 +1556,227 @@ __device__ __forceinline__ void entry_force(const Dev<Real>& d, const PairP<Real
     acc.q[Q_W0 + 5] += hf * dy * dz;
 }
 
-// Adds the per-entry forces w[k - wb] (one vector load each) of entries
-// [k0, k1) to f in entry order (the result does not depend on the launch).
-template <typename Real, typename R4>
-__device__ __forceinline__ void sum_run(const R4* w, int wb, int k0, int k1, Real& fx, Real& fy,
-                                        Real& fz)
+// The harmonic bonds of particle pi (vitrimer chains): F_i = k (r - r0) (x_j -
+// x_i) / r, half of the energy and virial to each end (added to the two-body
+// terms).
+template <typename Real, bool TH>
+__device__ __forceinline__ void bond_forces(const Dev<Real>& d, const typename Dev<Real>::P4* pos,
+                                            const typename Dev<Real>::P4& pi, Acc<Real>& acc, Real& fx, Real& fy,
+                                            Real& fz)
 {
-#pragma unroll 2
-    for (int k = k0; k < k1; k++) {
-        const R4 p = w[k - wb];
-        fx += p.x;
-        fy += p.y;
-        fz += p.z;
+    const int tag = pos_bits(pi) >> kTypeBits;
+    for (int b = 0; b < kMaxBonds; b++) {
+        const int pt = d.bond_tag[tag * kMaxBonds + b];
+        if (pt < 0) break;
+        const typename Dev<Real>::P4 pj = pos[d.slot_of_tag[pt]];
+        Real dx, dy, dz;
+        const Real r = sqrt(dist2_listed(pi, pj, d, dx, dy, dz));
+        const Real dr = r - d.bond_r0;
+        const Real g = d.bond_k * dr / r;
+        fx += g * dx;
+        fy += g * dy;
+        fz += g * dz;
+        if (!TH) continue;
+        acc.q[Q_U2] += Real(0.25) * d.bond_k * dr * dr;
+        const Real hf = Real(-0.5) * g;
+        acc.q[Q_W0 + 0] += hf * dx * dx;
+        acc.q[Q_W0 + 1] += hf * dy * dy;
+        acc.q[Q_W0 + 2] += hf * dz * dz;
+        acc.q[Q_W0 + 3] += hf * dx * dy;
+        acc.q[Q_W0 + 4] += hf * dx * dz;
+        acc.q[Q_W0 + 5] += hf * dy * dz;
     }
 }
 
-// With one sub-chunk per block the S pass of the same step left the block's
-// positions, list ranges and S values in shared memory, and the integrator
-// keeps the shared positions current for the next S pass.  TH: the sampled
-// step (thermo terms summed into the block's running sums blk).
-template <typename Real, bool UNI, bool BONDS, bool TH>
-__device__ float f_pass_block(const Dev<Real>& d, const PairP<Real>* tab, const RunArgs& a, int pc,
-                              int ac, int flags, long long step, Acc<Real>& acc,
-                              const PairP<Real>& ps, const PairP<Real>& pw, double* blk)
+// Where the S pass of the same step left the block's positions, list ranges and
+// S values in shared memory (one sub-chunk or unit per warp), they are taken
+// from there, and the integrator keeps the shared positions current for the
+// next S pass.  TH: the sampled step (the warps' thermo terms are left in
+// s_wacc, see block_sums_from_rows).  Returns the thread's largest squared
+// drift displacement.
+template <bool UNI, bool BONDS, bool TH>
+__device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const RunArgs& a, int pc, int ac, int flags,
+                             long long step, const PairP<float>& ps, const PairP<float>& pw)
 {
-    typedef Stage<Real> SM;
-    typedef typename Dev<Real>::R4 R4;
-    typedef typename Dev<Real>::P4 P4;
-    const P4* pos = d.pos[pc];
+    typedef Stage<float> SM;
+    const int4* pos = d.pos[pc];
     int b0, b1;
     block_range(d, b0, b1);
-    const int t = threadIdx.x;
     const int n = d.n;
-    const bool single = b1 - b0 <= (int)blockDim.x;
+    const int t = threadIdx.x, lane = t & 31;
+    const bool single = b1 - b0 <= kThreads;
     float dmax = 0.0f;
-    for (int q0 = b0; q0 < b1; q0 += blockDim.x) {
-        const int P = min((int)blockDim.x, b1 - q0);
+    [[maybe_unused]] double run = 0.0;  // lane q: quantity q of the warp's particles so far
+    const int4 none = make_int4(0, 0, 0, 0);
+    // what the thread's next rows need is loaded while it works on the present ones
+    int4 ti = none;
+    int i = b0;
+    if (b0 + t < b1) {
+        ti = single ? SM::info()[t] : d.tinfo[b0 + t];
+        i = single ? SM::idx()[t] : d.perm[b0 + t];
+    }
+    int4 jn = ti.y > 0 ? load_four(d, ti.x, 0) : none;
+    for (int q0 = b0; q0 < b1; q0 += kThreads) {
+        const int P = min(kThreads, b1 - q0);
+        if ((t & ~31) >= P) break;  // the same in the whole warp
+        const bool on = t < P;
+        const int qn = q0 + kThreads + t;
+        int4 tn = none, pi = none;
+        int in = i;
+        float Si = 0.0f;
+        if (on) {
+            // integrator inputs: asynchronous copies, waited for after the entries
+            cp_async_r4(&SM::vel()[t], &d.vel[ac][i]);
+            if (flags & F_OPENING)
+                for (int c = 0; c < 3; c++) cp_async(&SM::xq()[3 * t + c], &d.xq[ac][c * n + i], 8);
+            cp_async_commit();
+            if (single) {
+                pi = SM::pos()[t];
+                Si = SM::S()[t];
+            } else {
+                pi = pos[i];
+                Si = d.S[i];
+                if (qn < b1) {
+                    tn = d.tinfo[qn];
+                    in = d.perm[qn];
+                }
+            }
+        }
+        float fx = 0.0f, fy = 0.0f, fz = 0.0f, gx = 0.0f, gy = 0.0f, gz = 0.0f;  // reactive and other rows' sums
+        Acc<float> acc;
+        if (TH)
+#pragma unroll
+            for (int q = 0; q < kNQA; q++) acc.q[q] = 0.0f;
+        auto reactive = [&](const int4& pj, float Sj) {
+            float ex, ey, ez;
+            entry_force<float, UNI, true, TH>(d, tab, pi, pj, Si, Sj, ps, acc, ex, ey, ez);
+            fx = __fadd_rn(fx, ex);
+            fy = __fadd_rn(fy, ey);
+            fz = __fadd_rn(fz, ez);
+        };
+        auto other = [&](const int4& pj) {
+            float ex, ey, ez;
+            entry_force<float, UNI, false, TH>(d, tab, pi, pj, 0.0f, 0.0f, pw, acc, ex, ey, ez);
+            gx = __fadd_rn(gx, ex);
+            gy = __fadd_rn(gy, ey);
+            gz = __fadd_rn(gz, ez);
+        };
+        int4 jo = ti.w > 0 ? load_four(d, ti.z, 0) : none;
+        for (int k = 0; k < ti.y; k += 4) {
+            const int4 j = jn;
+            if (k + 4 < ti.y) jn = load_four(d, ti.x, k + 4);
+            const int4 p0 = pos[j.x], p1 = pos[j.y], p2 = pos[j.z], p3 = pos[j.w];  // padding: the own slot
+            const float s0 = d.S[j.x], s1 = d.S[j.y], s2 = d.S[j.z], s3 = d.S[j.w];
+            reactive(p0, s0);
+            if (k + 1 < ti.y) reactive(p1, s1);
+            if (k + 2 < ti.y) reactive(p2, s2);
+            if (k + 3 < ti.y) reactive(p3, s3);
+        }
+        for (int k = 0; k < ti.w; k += 4) {
+            const int4 j = jo;
+            if (k + 4 < ti.w) jo = load_four(d, ti.z, k + 4);
+            const int4 p0 = pos[j.x], p1 = pos[j.y], p2 = pos[j.z], p3 = pos[j.w];
+            other(p0);
+            if (k + 1 < ti.w) other(p1);
+            if (k + 2 < ti.w) other(p2);
+            if (k + 3 < ti.w) other(p3);
+        }
+        // the force: the reactive row's sum plus the other row's (the order of
+        // the resident step, so both paths give the same bits)
+        fx = __fadd_rn(fx, gx);
+        fy = __fadd_rn(fy, gy);
+        fz = __fadd_rn(fz, gz);
+        if (BONDS && d.has_bonds && on)  // BONDS: some system of the launch has bonds
+            bond_forces<float, TH>(d, pos, pi, acc, fx, fy, fz);
+        // the pair terms join the running sums now, so that they hold no
+        // registers at the integrator's peak
+        if (TH)
+#pragma unroll
+            for (int q = 0; q < kNQA; q++)
+                if (q != Q_K) {
+                    const float x = warp_sum(acc.q[q]);
+                    if (lane == q) run += (double)x;
+                }
+        if (qn < b1) {
+            if (tn.y > 0) jn = load_four(d, tn.x, 0);
+            if (tn.w > 0) prefetch_row(d, tn.z);
+        }
+        float kin = 0.0f;
+        if (on) {
+            if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(&d.ctl->status, kStatusNonfinite);
+            if (flags & F_STORE) d.force[i] = make_float4(fx, fy, fz, 0.0f);
+            cp_async_wait_all();
+            PState<float> st;
+            st.v = SM::vel()[t];
+            if (flags & F_OPENING)
+                for (int c = 0; c < 3; c++) st.q[c] = SM::xq()[3 * t + c];
+            dmax = fmaxf(dmax, integrate_one(d, a, pc, ac, i, fx, fy, fz, flags, step, st, pos_bits(pi), kin,
+                                             single ? &SM::pos()[t] : (int4*)nullptr));
+        }
+        if (TH) {
+            const float x = warp_sum(kin);
+            if (lane == Q_K) run += (double)x;
+        }
+        ti = tn;
+        i = in;
+    }
+    if (TH && lane < kNQA) s_wacc[t >> 5][lane] = run;
+    return dmax;
+}
+
+// One pair's force on its owner into the wave's results at place x, from the
+// pair force ft (zero outside the cut-off) and, when TH, its share of the
+// virial.
+template <bool TH>
+__device__ __forceinline__ void put_force(double ft, double dx, double dy, double dz, int x, Acc<double>& acc)
+{
+    typedef Stage<double> SM;
+    SM::w()[x] = -ft * dx;
+    SM::w()[SM::kWave + x] = -ft * dy;
+    SM::w()[2 * SM::kWave + x] = -ft * dz;
+    if (!TH) return;
+    const double hf = 0.5 * ft;
+    acc.q[Q_W0 + 0] += hf * dx * dx;
+    acc.q[Q_W0 + 1] += hf * dy * dy;
+    acc.q[Q_W0 + 2] += hf * dz * dz;
+    acc.q[Q_W0 + 3] += hf * dx * dy;
+    acc.q[Q_W0 + 4] += hf * dx * dz;
+    acc.q[Q_W0 + 5] += hf * dy * dz;
+}
+
+// A reactive pair: the three-body factor on its two-body force (outside r_min).
+template <bool TH>
+__device__ __forceinline__ void put_reactive(const PairP<double>& p, double r2, bool in, double v, double ft, double vh,
+                                             bool beyond, double dx, double dy, double dz, double Si, double Sj, int x,
+                                             Acc<double>& acc)
+{
+    const double h = p.a * (Si + Sj - 2.0 * p.a * vh);
+    if (beyond) ft = ft * (1.0 - h * p.inv_epshat);
+    if (TH && in) {
+        acc.q[Q_U2] += 0.5 * (v + p.ushift);
+        acc.q[Q_U3] += 0.5 * p.a * vh * (Si - p.a * vh);
+        if (r2 < p.rbond2) acc.q[Q_BONDS] += 0.5;
+    }
+    put_force<TH>(ft, dx, dy, dz, x, acc);
+}
+
+template <bool UNI, bool BONDS, bool TH>
+__device__ float f_pass_waves(const Dev<double>& d, const PairP<double>* tab, const RunArgs& a, int pc, int ac,
+                              int flags, long long step, const PairP<double>& ps, const PairP<double>& pw)
+{
+    typedef Stage<double> SM;
+    const dbl4* pos = d.pos[pc];
+    int b0, b1;
+    block_range(d, b0, b1);
+    const int t = threadIdx.x, n = d.n;
+    const bool single = b1 - b0 <= kThreads;
+    float dmax = 0.0f;
+    Acc<double> acc;
+    if (TH)
+#pragma unroll
+        for (int q = 0; q < kNQA; q++) acc.q[q] = 0.0;
+    for (int q0 = b0; q0 < b1; q0 += kThreads) {
+        const int P = min(kThreads, b1 - q0);
         if (t < P) {
             const int i = q0 + t;
             // integrator inputs: asynchronous copies, waited for after the entries
@@ -1358,151 +1784,121 @@ __device__ float f_pass_block(const Dev<Real>& d, const PairP<Real>* tab, const 
             if (flags & F_OPENING)
                 for (int c = 0; c < 3; c++) cp_async(&SM::xq()[3 * t + c], &d.xq[ac][c * n + i], 8);
             cp_async_commit();
-        }
-        if (!single) {
-            if (t < P) {
-                const int i = q0 + t;
+            if (!single) {
                 SM::pos()[t] = pos[i];
                 SM::S()[t] = d.S[i];
                 SM::info()[t] = d.pinfo[i];
             }
-            __syncthreads();
         }
-        const int e_beg = SM::info()[0].x;
-        const int e_rend = SM::info()[P - 1].x + SM::info()[P - 1].y;
-        const int e_end = SM::info()[P - 1].z + SM::info()[P - 1].w;
-        {
-            // into L2 while this sub-chunk runs: the next sub-chunk's entries
-            // (sized like this one's), or after the last one the reactive
-            // entries of the block's first sub-chunk, which the next S pass
-            // starts with
-            const long long cap = block_list_end(d);
-            if (q0 + P < b1)
-                prefetch_entries(d, e_end, min((long long)e_end + (e_end - e_beg), cap));
-            else {
-                const long long f0 = cap - (long long)((d.n + g_size() - 1) / g_size()) * d.max_nn;
-                prefetch_entries(d, f0, min(f0 + (e_rend - e_beg), cap));
-            }
-        }
-        Real fx = 0, fy = 0, fz = 0, gx = 0, gy = 0, gz = 0;  // reactive and other entries' sums
-        for (int wb = e_beg; wb < e_end; wb += SM::wave) {
-            const int we = min(wb + SM::wave, e_end);
-            // groups of kGatherF entries per thread, their gathers issued together
-            const int B = blockDim.x;
-            for (int e0 = wb + t; e0 < we; e0 += kGatherF * B) {
-                int jj[kGatherF], oo[kGatherF];
-#pragma unroll
-                for (int u = 0; u < kGatherF; u++) {
-                    const int e = e0 + u * B;
-                    jj[u] = e < we ? __ldcs(&d.ent_j[e]) : 0;  // streamed: keep L2 for the snapshots
-                    oo[u] = e < we ? __ldcs(&d.ent_o[e]) : 0;
-                }
-                P4 pj[kGatherF];
-                Real sj[kGatherF];
-#pragma unroll
-                for (int u = 0; u < kGatherF; u++) {
-                    pj[u] = pos[jj[u]];  // slot 0 for a missing entry
-                    sj[u] = e0 + u * B < e_rend ? d.S[jj[u]] : Real(0);
-                }
-#pragma unroll
-                for (int u = 0; u < kGatherF; u++) {
-                    const int e = e0 + u * B;
-                    if (e >= we) continue;
-                    Real ex, ey, ez;
-                    if (e < e_rend)
-                        entry_force<Real, UNI, true, TH>(d, tab, SM::pos()[oo[u]], pj[u], SM::S()[oo[u]], sj[u], ps,
-                                                         acc, ex, ey, ez);
-                    else
-                        entry_force<Real, UNI, false, TH>(d, tab, SM::pos()[oo[u]], pj[u], Real(0), Real(0), pw, acc,
-                                                          ex, ey, ez);
-                    R4 r;
-                    r.x = ex;
-                    r.y = ey;
-                    r.z = ez;
-                    r.w = Real(0);
-                    SM::w4()[e - wb] = r;
+        const int nkeep = single ? s_nkeep : -1;  // kept pairs: the first nkeep of the list
+        if (nkeep < 0 && t == 0) s_nlist = 0;
+        __syncthreads();
+        const int4 inf = SM::info()[min(t, P - 1)];
+        const int4 last = SM::info()[P - 1];
+        const unsigned e_beg = SM::info()[0].x, e_rend = (unsigned)(last.x + last.y), e_end = (unsigned)(last.z + last.w);
+        double f[3] = {0.0, 0.0, 0.0}, g[3] = {0.0, 0.0, 0.0};  // reactive and other rows' sums
+        for (unsigned wb = e_beg; wb < e_end; wb += SM::kWave) {
+            const unsigned we = min(wb + SM::kWave, e_end);
+            const unsigned wr = min(max(e_rend, wb), we);  // reactive entries before, others from here
+            int nre = nkeep;  // reactive pairs in the list
+            if (nkeep < 0) {
+                line_up<UNI>(d, tab, ps, pos, wb, wb, wr, 3);
+                __syncthreads();
+                nre = s_nlist;
+                __syncthreads();
+            } else {
+                // kept: the places of the pairs that were left out (line_up has
+                // zeroed the first of their three results, and the pairs' own
+                // places are all written below)
+                for (unsigned e = wb + t; e < wr; e += kThreads) {
+                    SM::w()[e - wb] = 0.0;
+                    SM::w()[SM::kWave + (e - wb)] = 0.0;
+                    SM::w()[2 * SM::kWave + (e - wb)] = 0.0;
                 }
             }
+            line_up<UNI>(d, tab, pw, pos, wb, wr, we, 3);
             __syncthreads();
-            if (t < P) {
-                const int4 inf = SM::info()[t];
-                sum_run(SM::w4(), wb, max(inf.x, wb), min(inf.x + inf.y, we), fx, fy, fz);
-                sum_run(SM::w4(), wb, max(inf.z, wb), min(inf.z + inf.w, we), gx, gy, gz);
+            const int m = s_nlist;
+            for (int c = t; c < m; c += kThreads) {
+                const int2 it = SM::list()[c];
+                const int x = it.x & (kBeyond - 1), o = it.x >> 16;
+                double dx, dy, dz, v = 0.0, ft;
+                if (c < nkeep) {
+                    const double Sj = d.S[it.y];
+                    const double* k = SM::keep() + c;
+                    const bool beyond = it.x & kBeyond;
+                    dx = k[2 * SM::kKeep];
+                    dy = k[3 * SM::kKeep];
+                    dz = k[4 * SM::kKeep];
+                    double r2 = 0.0;
+                    bool in = true;
+                    const PairP<double>* p = &ps;
+                    if (!UNI) p = &tab[type_of(SM::pos()[o]) * d.ntypes + type_of(pos[it.y])];
+                    if (TH) {
+                        v = k[5 * SM::kKeep];
+                        r2 = add_rn(add_rn(mul_rn(dx, dx), mul_rn(dy, dy)), mul_rn(dz, dz));
+                        in = r2 < p->rc2;
+                    }
+                    put_reactive<TH>(*p, r2, in, v, k[0], k[SM::kKeep], beyond, dx, dy, dz, SM::S()[o], Sj, x, acc);
+                } else {
+                    const dbl4 pi = SM::pos()[o], pj = pos[it.y];
+                    const bool react = c < nre;
+                    const PairP<double>& p = UNI ? (react ? ps : pw) : tab[type_of(pi) * d.ntypes + type_of(pj)];
+                    const double Sj = react ? d.S[it.y] : 0.0;
+                    const double r2 = dist2_near(pi, pj, d, dx, dy, dz);
+                    const bool in = r2 < p.rc2;
+                    lj_eval(p, r2, v, ft);
+                    ft = in ? ft : 0.0;
+                    if (react) {
+                        const bool beyond = r2 > p.rmin2;
+                        const double vh = beyond ? (p.vshift - v) * p.inv_epshat : 1.0;
+                        put_reactive<TH>(p, r2, in, v, ft, vh, beyond, dx, dy, dz, SM::S()[o], Sj, x, acc);
+                    } else {
+                        if (TH && in) acc.q[Q_U2] += 0.5 * (v + p.ushift);
+                        put_force<TH>(ft, dx, dy, dz, x, acc);
+                    }
+                }
             }
             __syncthreads();
+            if (t == 0) s_nlist = 0;
+            auto part = [&](unsigned r0, unsigned r1, double (&sum)[3]) {
+                const bool on = t < P && r1 > wb && r0 < we;
+                sum_row(SM::w(), on ? (int)(max(r0, wb) - wb) : 0, on ? (int)(min(r1, we) - wb) : 0, sum);
+            };
+            part((unsigned)inf.x, (unsigned)inf.x + (unsigned)inf.y, f);
+            part((unsigned)inf.z, (unsigned)inf.z + (unsigned)inf.w, g);
+            __syncthreads();
         }
-        // the force: the reactive entries' sum plus the others' (the order of
-        // the resident step, so both paths give the same bits)
-        fx = add_rn(fx, gx);
-        fy = add_rn(fy, gy);
-        fz = add_rn(fz, gz);
-        // harmonic bonds (vitrimer chains): F_i = k (r - r0) (x_j - x_i) / r, half
-        // of the energy and virial to each end (added to the two-body terms)
-        if (BONDS && d.has_bonds && t < P) {  // BONDS: some system of the launch has bonds
-            const P4 pi = SM::pos()[t];
-            const int tag = pos_bits(pi) >> kTypeBits;
-            for (int b = 0; b < kMaxBonds; b++) {
-                const int pt = d.bond_tag[tag * kMaxBonds + b];
-                if (pt < 0) break;
-                const P4 pj = pos[d.slot_of_tag[pt]];
-                Real dx, dy, dz;
-                const Real r = sqrt(dist2_listed(pi, pj, d, dx, dy, dz));
-                const Real dr = r - d.bond_r0;
-                const Real g = d.bond_k * dr / r;
-                fx += g * dx;
-                fy += g * dy;
-                fz += g * dz;
-                if (!TH) continue;
-                acc.q[Q_U2] += Real(0.25) * d.bond_k * dr * dr;
-                const Real hf = Real(-0.5) * g;
-                acc.q[Q_W0 + 0] += hf * dx * dx;
-                acc.q[Q_W0 + 1] += hf * dy * dy;
-                acc.q[Q_W0 + 2] += hf * dz * dz;
-                acc.q[Q_W0 + 3] += hf * dx * dy;
-                acc.q[Q_W0 + 4] += hf * dx * dz;
-                acc.q[Q_W0 + 5] += hf * dy * dz;
-            }
-        }
-        // FP32: park the thermo accumulators in the (now free) wave buffer while
-        // the integrator runs, so they do not hold registers at its peak
-        constexpr bool kPark = TH && sizeof(Real) == 4;
-        if (kPark)
-#pragma unroll
-            for (int q = 0; q < kNQA; q++) SM::w()[q * blockDim.x + t] = acc.q[q];
-        Real kin = Real(0);
+        double fx = add_rn(f[0], g[0]), fy = add_rn(f[1], g[1]), fz = add_rn(f[2], g[2]);
+        if (BONDS && d.has_bonds && t < P)  // BONDS: some system of the launch has bonds
+            bond_forces<double, TH>(d, pos, SM::pos()[t], acc, fx, fy, fz);
+        double kin = 0.0;
         if (t < P) {
             const int i = q0 + t;
             if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(&d.ctl->status, kStatusNonfinite);
             if (flags & F_STORE) {
-                R4 f;
-                f.x = fx;
-                f.y = fy;
-                f.z = fz;
-                f.w = Real(0);
-                d.force[i] = f;
+                dbl4 fo;
+                fo.x = fx;
+                fo.y = fy;
+                fo.z = fz;
+                fo.w = 0.0;
+                d.force[i] = fo;
             }
             cp_async_wait_all();
-            PState<Real> st;
+            PState<double> st;
             st.v = SM::vel()[t];
             if (flags & F_OPENING)
                 for (int c = 0; c < 3; c++) st.q[c] = SM::xq()[3 * t + c];
-            dmax = fmaxf(dmax, integrate_one(d, a, pc, ac, i, fx, fy, fz, flags, step, st, pos_bits(SM::pos()[t]),
-                                             kin, single ? &SM::pos()[t] : (P4*)nullptr));
+            dmax = fmaxf(dmax, integrate_one(d, a, pc, ac, i, fx, fy, fz, flags, step, st, pos_bits(SM::pos()[t]), kin,
+                                             single ? &SM::pos()[t] : (dbl4*)nullptr));
         }
-        if (kPark)
-#pragma unroll
-            for (int q = 0; q < kNQA; q++) acc.q[q] = SM::w()[q * blockDim.x + t];
         if (TH) acc.q[Q_K] += kin;
-        __syncthreads();
-        if (TH && !single) {
-            // several sub-chunks: fold this one's terms into the block's FP64
-            // running sums, so no thread accumulates more than one sub-chunk
-            // (per-warp running sums without the block barriers, tried in FP64
-            // and in double-float, measured slower)
-            block_sums(acc.q, SM::w(), blk, (double*)nullptr);
+        if (!single) __syncthreads();  // the staging is free
+    }
+    if (TH) {
+        // staged for block_sums_from_threads (the waves' buffer is free)
 #pragma unroll
-            for (int q = 0; q < kNQA; q++) acc.q[q] = Real(0);
-        }
+        for (int q = 0; q < kNQA; q++) SM::w()[q * kThreads + t] = acc.q[q];
     }
     return dmax;
 }
@@ -1556,7 +1952,6 @@ struct LoopState {
 
 static __shared__ __align__(16) unsigned char s_tab_raw[kMaxTypes * kMaxTypes * sizeof(PairP<double>)];
 static __shared__ double s_red[32];
-static __shared__ double s_blk[kNQ];  // the block's FP64 running thermo sums of the current pass
 static __shared__ int s_int[64];
 static __shared__ LoopState s_ls;
 
@@ -1602,7 +1997,7 @@ __device__ SWP_COLD int run_rebuild(const Dev<Real>& d, const RunArgs& a)
     }
     if (!grid_barrier(ctl, a.timeout_ns, 6)) return 2;
     int ovf = 0;
-    const int need = ph_build_cells<Real>(d, stab<Real>(), pc0 ^ 1, (int2*)Stage<Real>::w(), s_int, &ovf);
+    const int need = ph_build_rows<Real>(d, stab<Real>(), pc0 ^ 1, s_int, &ovf);
     if (threadIdx.x == 0) {
         atomicMax(&ctl->max_row, need);
         if (ovf) atomicOr(&ctl->overflow, 1);
@@ -1622,19 +2017,23 @@ __device__ SWP_COLD int run_rebuild(const Dev<Real>& d, const RunArgs& a)
     return 0;
 }
 
-// One sub-chunk per block: the block's particles fit one shared staging.
+// At most one unit per warp: the block's particles fit one shared staging.
 template <typename Real>
 __device__ __forceinline__ bool single_chunk(const Dev<Real>& d)
 {
     return (d.n + g_size() - 1) / g_size() <= (int)blockDim.x;
 }
 
+// The caller sets s_ls.own_ok after the grid barrier that follows (every warp
+// has read it by then).
 template <typename Real, bool UNI>
-__device__ __forceinline__ void run_s_pass(const Dev<Real>& d, const RunArgs& a)
+__device__ __forceinline__ void run_s_pass(const Dev<Real>& d, const RunArgs& a, [[maybe_unused]] bool th)
 {
-    const bool single = single_chunk(d);
-    s_pass_block<Real, UNI>(d, stab<Real>(), s_ls.pc, uni_params(a, Real(0))[0], single && s_ls.own_ok);
-    if (threadIdx.x == 0) s_ls.own_ok = single;  // every thread read it before the pass's barriers
+    const bool staged = single_chunk(d) && s_ls.own_ok;
+    if constexpr (sizeof(Real) == 4)
+        s_pass_rows<UNI>(d, stab<Real>(), s_ls.pc, uni_params(a, Real(0))[0], staged);
+    else
+        s_pass_waves<UNI>(d, stab<Real>(), s_ls.pc, uni_params(a, Real(0))[0], staged, th);
 }
 
 // Folds a thread's squared displacement into the block's shared maximum (one
@@ -1647,13 +2046,14 @@ __device__ __forceinline__ void warp_max_disp(float v)
 }
 
 template <typename Real, bool UNI, bool BONDS, bool TH>
-__device__ __forceinline__ void run_f_pass(const Dev<Real>& d, const RunArgs& a, int flags, long long stp,
-                                           Acc<Real>& acc)
+__device__ __forceinline__ void run_f_pass(const Dev<Real>& d, const RunArgs& a, int flags, long long stp)
 {
-#pragma unroll
-    for (int q = 0; q < kNQA; q++) acc.q[q] = Real(0);
-    const float dmax = f_pass_block<Real, UNI, BONDS, TH>(d, stab<Real>(), a, s_ls.pc, s_ls.ac, flags, stp, acc,
-                                                      uni_params(a, Real(0))[0], uni_params(a, Real(0))[1], s_blk);
+    const PairP<Real>*ps = &uni_params(a, Real(0))[0], *pw = &uni_params(a, Real(0))[1];
+    float dmax;
+    if constexpr (sizeof(Real) == 4)
+        dmax = f_pass_rows<UNI, BONDS, TH>(d, stab<Real>(), a, s_ls.pc, s_ls.ac, flags, stp, *ps, *pw);
+    else
+        dmax = f_pass_waves<UNI, BONDS, TH>(d, stab<Real>(), a, s_ls.pc, s_ls.ac, flags, stp, *ps, *pw);
     if (flags & F_OPENING) warp_max_disp(dmax);
 }
 
@@ -1708,22 +2108,34 @@ __device__ __forceinline__ void reduce_small(const Dev<Real>& d)
 }
 
 // Writes the block's partials of a sampled step's thermo terms (energies,
-// virial, bond count, kinetic energy) from the threads' accumulators (or, for
-// a resident step, from the per-warp sums s_wpart it left) to the launch's
-// partials (last: the last step of the launch, whose values the launch
-// reports; reduced after the loop) and/or to a thermo-log record (log).
-// Every call is followed by a grid barrier.  Steps that are neither the
-// launch's last nor logged skip the thermo terms altogether.
+// virial, bond count, kinetic energy) from the warps' sums (s_wacc, or for a
+// resident step s_wpart) to the launch's partials (last: the last step of the
+// launch, whose values the launch reports; reduced after the loop) and/or to a
+// thermo-log record (log).  Every call is followed by a grid barrier.  Steps
+// that are neither the launch's last nor logged skip the thermo terms
+// altogether.
 template <typename Real>
-__device__ __forceinline__ void thermo_partials(const Dev<Real>& d, const Acc<Real>& acc, Real* stage,
-                                                bool folded, bool last, double* log)
+__device__ __forceinline__ void thermo_partials(const Dev<Real>& d, bool resident, bool last, double* log)
 {
     double* out = last ? d.partials + (size_t)g_rank() * kNQ : log;
     double* out2 = last ? log : nullptr;
-    if (folded)
-        block_sums_from_warps(s_blk, out, out2);
-    else
-        block_sums(acc.q, stage, s_blk, out, out2);
+    if (resident) {
+        block_sums_from_warps(out, out2);
+    } else {
+        int b0, b1;
+        block_range(d, b0, b1);
+        if constexpr (sizeof(Real) == 4) {
+            block_sums_from_rows(min((b1 - b0 + 31) / 32, kThreads / 32), out, out2);
+        } else {
+            // threads that had a particle or (the lined-up pairs) an entry
+            int nact = kThreads;
+            if (b1 - b0 <= kThreads && b1 > b0) {
+                const int4 l = Stage<Real>::info()[b1 - b0 - 1];
+                nact = min(kThreads, max(b1 - b0, l.z + l.w - Stage<Real>::info()[0].x));
+            }
+            block_sums_from_threads((const double*)Stage<Real>::w(), nact, out, out2);
+        }
+    }
     if (last && threadIdx.x == 0) s_ls.have_thermo = 1;
 }
 
@@ -1786,7 +2198,7 @@ struct RStage {
     static_assert(B_END <= kBytes, "build scratch fits the own-state area");
     static_assert(kES <= 65536 && kEF <= 65536 && kL <= 65536, "16-bit local indices and offsets");
     static_assert(kBlock % 32 == 0 && kBlock / 32 <= 32, "whole warps, at most 32");
-    static_assert(kBlock >= 256 && kEF >= kBlock / 32 * 256, "force-row sort scratch (r_rank1_desc) in O_FENT");
+    static_assert(kBlock >= 256 && kEF >= kBlock / 32 * 256, "force-row sort scratch (rank_desc) in O_FENT");
 
     static __device__ __forceinline__ int4* lpos() { return (int4*)(g_dyn + O_LPOS); }
     static __device__ __forceinline__ float* lS() { return (float*)(g_dyn + O_LS); }
@@ -1800,7 +2212,7 @@ struct RStage {
     static __device__ __forceinline__ long long* xq() { return (long long*)(g_dyn + O_XQ); }
     static __device__ __forceinline__ int* img() { return (int*)(g_dyn + O_IMG); }
 };
-static_assert(RStage::kBytes <= Stage<float>::kBytes + 32768, "the resident layout fits the kernel's shared memory");
+static_assert(RStage::kBytes <= 227 * 1024 - 12 * 1024, "the resident layout fits beside the static shared memory");
 
 __device__ __forceinline__ void cp_async_cg16(void* smem, const void* gmem)
 {
@@ -1875,41 +2287,6 @@ __device__ void r_sort_desc(const int (&key)[R], int (&pos)[R], int* hist)
     }
 }
 
-// Stable counting sort, largest key first, of one item per thread (key in
-// [0, 255], -1: no item): returns the item's rank.  Equal keys keep the thread
-// order.  wh: scratch of blockDim / 32 x 256 u16 counts; hist: 256 ints;
-// blockDim >= 256.
-static __device__ int r_rank1_desc(int key, unsigned short* wh, int* hist)
-{
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, NW = blockDim.x >> 5;
-    __syncthreads();  // a previous call's readers are done with wh and hist
-    for (int k = t; k < NW * 256; k += blockDim.x) wh[k] = 0;
-    __syncthreads();
-    // the warp's lanes with this key, and how many come before this lane
-    const unsigned m = __match_any_sync(0xffffffffu, key);
-    const int before = __popc(m & ((1u << lane) - 1u));
-    if (key >= 0 && before == 0) wh[warp * 256 + key] = (unsigned short)__popc(m);
-    __syncthreads();
-    // per key: the counts of the warps before each warp, and the key's total
-    if (t < 256) {
-        int run = 0;
-        for (int w = 0; w < NW; w++) {
-            const int c = wh[w * 256 + t];
-            wh[w * 256 + t] = (unsigned short)run;
-            run += c;
-        }
-        hist[t] = run;
-    }
-    __syncthreads();
-    // keys in descending order: the first rank of key b is the count above it
-    const int b = 255 - t;
-    int tot;
-    const int ex = block_excl_scan(t < 256 ? hist[b] : 0, s_int, &tot);
-    if (t < 256) hist[b] = ex;  // every thread read hist before the scan's barriers
-    __syncthreads();
-    return key >= 0 ? hist[key] + wh[warp * 256 + key] + before : 0;
-}
-
 // Lays out warp blocks: rows at positions s (thread s % B, round s / B) with
 // n[r] entries each (0: no row); every warp block of 32 rows takes 32 x its
 // longest row, in order (round, warp).  Returns the total (entries), and in
@@ -1967,20 +2344,16 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     }
     __syncthreads();
     int fail = 0;
-    int e_beg = 0, e_rend = 0, e_end = 0;
-    if (P > 0) {
-        const int4 f0 = d.pinfo[b0], f1 = d.pinfo[b1 - 1];
-        e_beg = f0.x;
-        e_rend = f1.x + f1.y;
-        e_end = f1.z + f1.w;
-    }
+    int4 inf = make_int4(0, 0, 0, 0);
+    if (t < P) inf = d.pinfo[b0 + t];
     // 1. first shell: the partners of the own rows outside the block
-    for (int e = e_beg + t; e < e_end; e += B) {
-        const int q = d.ent_j[e];
+    for (int k = 0; k < inf.y + inf.w; k++) {
+        const bool react = k < inf.y;
+        const int q = d.ent_j[(unsigned)(react ? inf.x + k : inf.z + k - inf.y)];
         if (q < b0 || q >= b1) {
             const int h = r_insert(key, q);
             if (h < 0) fail = 1;
-            else if (e < e_rend) atomicOr(&val[h], 1);
+            else if (react) atomicOr(&val[h], 1);
         }
     }
     if (__syncthreads_or(fail)) return 0;
@@ -1997,8 +2370,8 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     // 3. second shell: the reactive partners of the reactive first shell
     for (int k = t; k < Hr; k += B) {
         const int4 fi = d.pinfo[key[hr[k]]];
-        for (int e = fi.x; e < fi.x + fi.y; e++) {
-            const int q = d.ent_j[e];
+        for (int m = 0; m < fi.y; m++) {
+            const int q = d.ent_j[(unsigned)(fi.x + m)];
             if ((q < b0 || q >= b1) && r_insert(key, q) < 0) fail = 1;
         }
     }
@@ -2027,8 +2400,6 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     // rows of a warp are alike in each loop and the warps' totals even out.
     const int NS = P + Hr;
     const int rounds = (NS + B - 1) / B;
-    int4 inf = make_int4(0, 0, 0, 0);
-    if (t < P) inf = d.pinfo[b0 + t];
     if (inf.y > 255 || inf.w > 255) fail = 1;
     int skey[RR + 1], spos[RR + 1], hrow[RR], hcnt[RR];
     skey[0] = t < P ? min(inf.y, 255) : -1;
@@ -2049,8 +2420,8 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     }
     r_sort_desc<RR + 1>(skey, spos, hist);
     const int W32 = (P + 31) & ~31;
-    const int rpos = r_rank1_desc(t < P ? inf.y : -1, RS::fent(), hist);
-    const int wrank = r_rank1_desc(t < P ? inf.w : -1, RS::fent(), hist);
+    const int rpos = rank_desc(t < P ? inf.y : -1, RS::fent(), hist, s_int);
+    const int wrank = rank_desc(t < P ? inf.w : -1, RS::fent(), hist, s_int);
     const int wpos = W32 - 32 - (wrank & ~31) + (wrank & 31);  // rank chunk c -> warp W32/32 - 1 - c
     for (int q = t; q < rounds * B; q += B) RS::sdesc()[q] = make_int2(0, -1);  // no row here
     if (t < W32) RS::fdesc()[t] = make_int4(0, 0, 0, -1);  // no rows; centres 0xffff
@@ -2106,7 +2477,7 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
                 const int lid = cen[q];
                 for (int m = 0; m < src.y; m++)
                     RS::sent()[first[r] + 32 * m] =
-                        (unsigned short)r_lid(key, val, d.ent_j[src.x + m], b0, b1, P, fail);
+                        (unsigned short)r_lid(key, val, d.ent_j[(unsigned)(src.x + m)], b0, b1, P, fail);
                 RS::sdesc()[q] = make_int2(first[r], lid | (src.y << 16));
             }
         }
@@ -2114,9 +2485,9 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     if (t < W32) {
         unsigned short* fe = RS::fent();
         for (int m = 0; m < nrc[0]; m++)
-            fe[rfirst[0] + 32 * m] = (unsigned short)r_lid(key, val, d.ent_j[fd.x + m], b0, b1, P, fail);
+            fe[rfirst[0] + 32 * m] = (unsigned short)r_lid(key, val, d.ent_j[(unsigned)(fd.x + m)], b0, b1, P, fail);
         for (int m = 0; m < nwc[0]; m++)
-            fe[ER + wfirst[0] + 32 * m] = (unsigned short)r_lid(key, val, d.ent_j[fd.y + m], b0, b1, P, fail);
+            fe[ER + wfirst[0] + 32 * m] = (unsigned short)r_lid(key, val, d.ent_j[(unsigned)(fd.y + m)], b0, b1, P, fail);
         RS::fdesc()[t] = make_int4(rfirst[0], ER + wfirst[0], fd.z, fd.w);
     }
     if (t < P) lpos[t] = d.pos[pc][b0 + t];  // own snapshots by local index
@@ -2197,8 +2568,9 @@ __device__ __forceinline__ float r_row_s(const Dev<float>& d, const PairP<float>
 // warp in s_wpart (thermo_partials completes the block sums).  Returns the
 // thread's squared drift displacement.
 template <bool UNI, bool TH>
-__device__ float r_step(const Dev<float>& d, const RunArgs& a, int flags, long long step, Acc<float>& acc)
+__device__ float r_step(const Dev<float>& d, const RunArgs& a, int flags, long long step)
 {
+    Acc<float> acc;
     typedef RStage RS;
     const int t = threadIdx.x, B = blockDim.x;
     const int P = s_ls.r_np, NQ = (P + s_ls.r_nhr + B - 1) / B * B;  // positions of the rows of S
@@ -2359,7 +2731,6 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
     PairP<Real>* tab = (PairP<Real>*)s_tab_raw;
     const int ntt = d.ntypes * d.ntypes;
     for (int t = threadIdx.x; t < ntt; t += blockDim.x) tab[t] = d.table[t];
-    if (threadIdx.x < kNQ) s_blk[threadIdx.x] = 0.0;
     if (threadIdx.x == 0) {
         s_withhold = a.withhold && g_rank() == 0;
         s_ls.bar_target = 0;
@@ -2421,12 +2792,12 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
                 __syncthreads();
             }
             if (s_ls.rc == 0) {
-                run_s_pass<Real, UNI>(d, a);
+                run_s_pass<Real, UNI>(d, a, true);
                 if (!grid_barrier(ctl, a.timeout_ns, 10)) return false;
-                Acc<Real> acc;
-                run_f_pass<Real, UNI, BONDS, true>(d, a, F_STORE, s_ls.step, acc);
+                if (threadIdx.x == 0) s_ls.own_ok = single_chunk(d);
+                run_f_pass<Real, UNI, BONDS, true>(d, a, F_STORE, s_ls.step);
                 if (threadIdx.x == 0) s_ls.state = 0;  // read again only after the barrier
-                thermo_partials(d, acc, Stage<Real>::w(), false, true, (double*)nullptr);
+                thermo_partials(d, false, true, (double*)nullptr);
                 if (!grid_barrier(ctl, a.timeout_ns, 11)) return false;
             }
         }
@@ -2484,27 +2855,27 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
             const bool logged = s_ls.tlog_left == 1;
             const bool th = !more || logged;
             const int flags = F_CLOSING | (more ? F_OPENING : F_STORE);
-            Acc<Real> acc;
             bool resident = false;
 #if SWP_HAS_RESIDENT
             if constexpr (kRes) {
                 if (s_ls.r_try)
                     if (!r_enter(d, a)) return false;
                 if (s_ls.r_valid) {
-                    const float dmax = th ? r_step<UNI, true>(d, a, flags, stp + 1, acc)
-                                          : r_step<UNI, false>(d, a, flags, stp + 1, acc);
+                    const float dmax = th ? r_step<UNI, true>(d, a, flags, stp + 1)
+                                          : r_step<UNI, false>(d, a, flags, stp + 1);
                     if (more) warp_max_disp(dmax);
                     resident = true;
                 }
             }
 #endif
             if (!resident) {
-                run_s_pass<Real, UNI>(d, a);
+                run_s_pass<Real, UNI>(d, a, th);
                 if (!grid_barrier(ctl, a.timeout_ns, 20)) return false;
+                if (threadIdx.x == 0) s_ls.own_ok = single_chunk(d);
                 if (th)
-                    run_f_pass<Real, UNI, BONDS, true>(d, a, flags, stp + 1, acc);
+                    run_f_pass<Real, UNI, BONDS, true>(d, a, flags, stp + 1);
                 else
-                    run_f_pass<Real, UNI, BONDS, false>(d, a, flags, stp + 1, acc);
+                    run_f_pass<Real, UNI, BONDS, false>(d, a, flags, stp + 1);
             }
             if (threadIdx.x == 0) {  // every thread read `remaining` before the pass's barriers
                 s_ls.step = stp + 1;
@@ -2522,13 +2893,13 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
             // read after the launch); the launch's last step writes the
             // partials the launch reduces, before its arrival
             const bool late = resident && more;
-            if (th && !late) thermo_partials(d, acc, Stage<Real>::w(), resident, !more, lg);
+            if (th && !late) thermo_partials(d, resident, !more, lg);
             unsigned* pub = more ? &ctl->dmax2[(stp + 1) & 1] : nullptr;
             {
                 BarState bs;
                 bs.target = s_ls.bar_target;
                 bar_arrive(ctl, bs, pub, &s_ls.dmax_bits);
-                if (th && late) warp_sums_to(s_blk, lg, nullptr);  // bar_arrive ordered the s_wpart writes
+                if (th && late) warp_sums_to(lg, nullptr);  // bar_arrive ordered the s_wpart writes
                 if (threadIdx.x == 0) s_ls.bar_target = bs.target;
                 if (!bar_wait(ctl, bs, a.timeout_ns, 21, &s_ls.ok)) return false;
             }
@@ -2738,10 +3109,10 @@ __global__ void k_get_nlist(Dev<Real> d, int pc, int* rows, int* counts, int wid
         counts[2 * tag + 1] = inf.y + inf.w;
         int* out = rows + (size_t)tag * width;
         int k = 0;
-        for (int e = inf.x; e < inf.x + inf.y && k < width; e++, k++)
-            out[k] = pos_bits(d.pos[pc][d.ent_j[e]]) >> kTypeBits;
-        for (int e = inf.z; e < inf.z + inf.w && k < width; e++, k++)
-            out[k] = pos_bits(d.pos[pc][d.ent_j[e]]) >> kTypeBits;
+        for (int m = 0; m < inf.y && k < width; m++, k++)
+            out[k] = pos_bits(d.pos[pc][d.ent_j[(unsigned)(inf.x + m)]]) >> kTypeBits;
+        for (int m = 0; m < inf.w && k < width; m++, k++)
+            out[k] = pos_bits(d.pos[pc][d.ent_j[(unsigned)(inf.z + m)]]) >> kTypeBits;
     }
 }
 
@@ -2805,8 +3176,8 @@ __global__ void k_pgrad_sums(Dev<Real> d, int pc, double* sd, double* part)
         if (i < n) {
             const typename Dev<Real>::P4 pi = d.pos[pc][i];
             const int4 inf = d.pinfo[i];
-            for (int e = inf.x + g; e < inf.x + inf.y; e += kPgLanes) {
-                const typename Dev<Real>::P4 pj = d.pos[pc][d.ent_j[e]];
+            for (int m = g; m < inf.y; m += kPgLanes) {
+                const typename Dev<Real>::P4 pj = d.pos[pc][d.ent_j[(unsigned)(inf.x + m)]];
                 const PairP<Real>& p = d.table[type_of(pi) * d.ntypes + type_of(pj)];
                 Real dx, dy, dz;
                 const Real r2 = dist2_listed(pi, pj, d, dx, dy, dz);
@@ -2875,8 +3246,8 @@ __global__ void k_pgrad_forces(Dev<Real> d, int pc, const double* sd, const doub
             const int4 inf = d.pinfo[i];
             const double Si = sd[2 * i], Di = sd[2 * i + 1];
             tag = pos_bits(pi) >> kTypeBits;
-            for (int e = inf.x + g; e < inf.x + inf.y; e += kPgLanes) {
-                const int j = d.ent_j[e];
+            for (int m = g; m < inf.y; m += kPgLanes) {
+                const int j = d.ent_j[(unsigned)(inf.x + m)];
                 const typename Dev<Real>::P4 pj = d.pos[pc][j];
                 const PairP<Real>& p = d.table[type_of(pi) * d.ntypes + type_of(pj)];
                 Real dx, dy, dz;

@@ -26,8 +26,18 @@ static void* run_fn(int uni, int bonds = 0)
 template <typename Real>
 size_t run_smem_bytes()
 {
-    // the two-barrier step's staging or the resident step's structures (one buffer)
-    return std::max(Stage<Real>::kBytes, single::RStage::kBytes);
+    // the two-barrier step's staging or (FP32) the resident step's structures (one buffer)
+    return sizeof(Real) == 4 ? std::max(Stage<Real>::kBytes, single::RStage::kBytes) : Stage<Real>::kBytes;
+}
+
+// What one launch takes: a launch that cannot step resident leaves the resident
+// structures' share of the SM's memory to L1, where the passes' gathers of
+// neighbouring warps meet.
+template <typename Real>
+static size_t launch_smem_bytes(const Dev<Real>& d, const RunArgs& a, int grid)
+{
+    const bool resident = a.resident && !d.has_bonds && (d.n + grid - 1) / grid <= kBlock;
+    return resident ? run_smem_bytes<Real>() : Stage<Real>::kBytes;
 }
 
 // Opts every variant into the dynamic shared memory it needs (once).
@@ -47,7 +57,7 @@ cudaError_t launch_run(const Dev<Real>& d, const RunArgs& a, int grid, int block
     Dev<Real> dd = d;
     RunArgs aa = a;
     void* args[] = {(void*)&dd, (void*)&aa};
-    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, run_smem_bytes<Real>(), s);
+    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, launch_smem_bytes(d, a, grid), s);
 }
 
 template <typename Real>
