@@ -289,6 +289,7 @@ size_t layout(swp_ctx* c, char* base, Dev<Real>* d)
         d->bsum = bsum;
         d->partials = partials;
         d->ctl = ctl;
+        d->agree = ctl ? ctl->agree : nullptr;
         d->io = io;
         d->io_int = io_int;
         d->table = table;
@@ -458,9 +459,10 @@ bool same_pair(const PairHost& a, const PairHost& b)
 void uniform_pairs(const swp_ctx* c, RunArgs* a)
 {
     int sw = -1, ot = -1;
-    bool uni = true;
+    bool uni = true, even = true;
     for (int k = 0; k < c->ntypes * c->ntypes; k++) {
         const PairHost& p = c->pairs[k];
+        even &= p.kind == KIND_NONE || p.n % 2 == 0;
         if (p.kind == KIND_SWAP) {
             if (sw < 0) sw = k;
             else if (!same_pair(p, c->pairs[sw])) uni = false;
@@ -469,7 +471,9 @@ void uniform_pairs(const swp_ctx* c, RunArgs* a)
             else if (!same_pair(p, c->pairs[ot])) uni = false;
         }
     }
-    a->uni = uni ? 1 : 0;
+    a->uni = uni && !c->table_only ? 1 : 0;  // table_only: the device table holds coefficients the host copy does not
+    a->expo = even ? kExpoEven : kExpoAny;
+    if (a->uni && (sw < 0 || c->pairs[sw].n == 10) && (ot < 0 || c->pairs[ot].n == 6)) a->expo = kExpoStd;
     a->uni_swap = sw < 0 ? 0 : sw;
     a->uni_other = ot < 0 ? 0 : ot;
 }
@@ -550,9 +554,9 @@ int run(swp_ctx* c, RunArgs a)
     a.resident = c->resident;
     a.withhold = c->withhold;
     a.tlog_every = d.tlog ? c->tlog_every : 0;
-    if (c->table_only) a.uni = 0;  // the device table holds coefficients the host copy does not
     c->withhold = 0;  // one launch consumes the request
-    SWP_CUDA(c, cudaMemsetAsync(&d.ctl->barrier, 0, sizeof(unsigned long long), c->stream));
+    // the agreement words and the barrier counter, the control block's first
+    SWP_CUDA(c, cudaMemsetAsync(d.ctl, 0, offsetof(Ctl, barrier) + sizeof(unsigned long long), c->stream));
     if (wide) SWP_CUDA(c, launch_run_wide<Real>(d, a, c->grid, c->stream));
     else SWP_CUDA(c, launch_run<Real>(d, a, c->grid, block, c->stream));
     return SWP_OK;
@@ -1640,6 +1644,7 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
     a.timeout_ns = c->timeout_ns;
     a.skin_eff = c->skin;
     a.seed = c->seed;
+    a.expo = kExpoAny;
     SWP_CUDA(c, launch_run<Real>(d, a, step_grid(c, bps), block, s));
     SWP_CUDA(c, cudaMemcpyAsync(&h, d.ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
     SWP_CUDA(c, cudaStreamSynchronize(s));

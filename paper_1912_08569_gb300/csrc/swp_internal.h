@@ -51,7 +51,8 @@ struct PairP {
 };
 
 // Device-side control block (one per context, in the workspace).
-struct Ctl {
+struct alignas(16) Ctl {
+    unsigned long long agree[4]; // resident steps' agreement, two 16-byte words (see r_post; zeroed before each launch)
     unsigned long long barrier;  // grid-barrier arrival counter (zeroed before each launch)
     int status;                  // latched SWP_* error bits (see kStatus*)
     int state;                   // 0: full step, forces valid; 1: forces invalid; 2: mid-step
@@ -153,6 +154,7 @@ struct Dev {
     int* bsum;         // [max_blocks] per-block cell-count sums (scan)
     double* partials;  // [max_blocks][kNQ]
     Ctl* ctl;
+    unsigned long long* agree;  // resident steps: ctl->agree
     double* io;        // host-exchange staging: [3n] x, [3n] v, [n] mass
     int* io_int;       // staging: [n] types, [3n] images
     const PairP<Real>* table;  // [ntypes * ntypes]
@@ -166,6 +168,11 @@ struct Dev {
     long long* tlog_step;
     int tlog_cap;
 };
+
+// Exponents of a run's pairs (RunArgs::expo).
+constexpr int kExpoStd = 0;   // uniform coefficients, n = 10 reactive and n = 6 other
+constexpr int kExpoEven = 1;  // every n even
+constexpr int kExpoAny = 2;
 
 // What one launch of the step kernel does.
 struct RunArgs {
@@ -187,6 +194,7 @@ struct RunArgs {
     int withhold;       // test hook: block 0 withholds its arrival at the launch's first grid barrier
     int tlog_every;     // > 0: the steps whose number is a multiple of it write a thermo-log record
     int uni;            // 1: uniform coefficients (see uni_swap / uni_other)
+    int expo;           // kExpo*
     int uni_swap;       // table index of the reactive pair coefficients (UNI)
     int uni_other;      // table index of the other pairs' coefficients (UNI)
     // Uniform coefficients ([0] reactive, [1] other), read by the kernels

@@ -23,6 +23,8 @@
 // so that the code a group of one block or a group of fewer blocks than
 // thermo quantities needs costs the single-system kernel nothing.
 
+#include <type_traits>
+
 #include "swp_internal.h"
 
 #ifndef SWP_BATCHED
@@ -283,14 +285,44 @@ __device__ __forceinline__ float recip(float x)
 }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
+// (sigma/r)^n from s2 = (sigma/r)^2.  X says what the run's exponents are
+// (RunArgs::expo): kExpoStd n = 10 for reactive pairs (REACT) and n = 6 for the
+// others, kExpoEven any even n, kExpoAny any n.  FP32 code is free of branches
+// but for kExpoAny's odd n, so that the pairs a thread works on overlap: with a
+// loop over the bits of n (n = 100), or merely a test for n = 10, they went one
+// after the other and one pair of a lone warp took 600 to 900 cycles.  The
+// products are those of ipow in the same order: the same bits.  (FP64 is bound
+// by the number of multiplications.)
+template <int X, bool REACT, typename Real>
+__device__ __forceinline__ Real pair_power(const PairP<Real>& p, Real s2)
+{
+    if (sizeof(Real) == 8) {
+        Real x = ipow(s2, p.nhalf);
+        if (p.odd) x *= sqrt(s2);
+        return x;
+    }
+    if (X == kExpoStd) {
+        const Real b2 = s2 * s2;
+        return REACT ? b2 * b2 * s2 : b2 * s2;
+    }
+    const int e = p.nhalf;  // at most 64
+    Real b = s2, r = e & 1 ? s2 : Real(1);
+#pragma unroll
+    for (int k = 1; k < 7; k++) {
+        b *= b;
+        r = e >> k & 1 ? r * b : r;
+    }
+    if (X == kExpoAny && p.odd) r *= sqrt(s2);
+    return r;
+}
+
 // Eq. 2b at squared distance r2: v and f = -(dv/dr)/r.
-template <typename Real>
+template <int X, bool REACT, typename Real>
 __device__ __forceinline__ void lj_eval(const PairP<Real>& p, Real r2, Real& v, Real& f)
 {
     Real ir2 = recip(r2);
     Real s2 = p.sig2 * ir2;
-    Real x = ipow(s2, p.nhalf);
-    if (p.odd) x *= sqrt(s2);
+    Real x = pair_power<X, REACT>(p, s2);
     Real x2 = x * x;
     v = p.four_eps * (x2 - x);
     f = p.four_eps * p.n_real * (Real(2) * x2 - x) * ir2;
@@ -1110,7 +1142,7 @@ __device__ __forceinline__ void cp_async_r4(R4* smem, const R4* gmem)
 
 // One reactive entry's term of S_i: a vh(r_ij) inside r_cut, else 0 (evaluated
 // for every listed pair and selected by the cut-off decision, see entry_force).
-template <typename Real, bool UNI>
+template <typename Real, bool UNI, int X>
 __device__ __forceinline__ Real s_term(const Dev<Real>& d, const PairP<Real>* tab, const PairP<Real>& ps,
                                        const typename Dev<Real>::P4& pi, const typename Dev<Real>::P4& pj)
 {
@@ -1118,7 +1150,7 @@ __device__ __forceinline__ Real s_term(const Dev<Real>& d, const PairP<Real>* ta
     Real dx, dy, dz;
     const Real r2 = dist2_listed(pi, pj, d, dx, dy, dz);
     Real v, f;
-    lj_eval(p, r2, v, f);
+    lj_eval<X, true>(p, r2, v, f);
     const Real vh = r2 > p.rmin2 ? (p.vshift - v) * p.inv_epshat : Real(1);
     return r2 < p.rc2 ? mul_rn(p.a, vh) : Real(0);
 }
@@ -1139,7 +1171,7 @@ __device__ __forceinline__ int4 load_four(const Dev<float>& d, int first, int k)
 // positions and list ranges are current (kept by the previous force pass), so
 // they are not loaded again; its S values also stay in shared memory for the
 // force pass.
-template <bool UNI>
+template <bool UNI, int X>
 __device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc, const PairP<float>& ps, bool staged)
 {
     typedef Stage<float> SM;
@@ -1182,16 +1214,16 @@ __device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc
             const int4 j = jn;
             if (k + 4 < cnt) jn = load_four(d, ti.x, k + 4);
             const int4 p0 = pos[j.x], p1 = pos[j.y], p2 = pos[j.z], p3 = pos[j.w];  // padding: the own slot
-            const float w0 = s_term<float, UNI>(d, tab, ps, pi, p0);
+            const float w0 = s_term<float, UNI, X>(d, tab, ps, pi, p0);
             if (k + 4 <= cnt) {
-                const float w1 = s_term<float, UNI>(d, tab, ps, pi, p1);
-                const float w2 = s_term<float, UNI>(d, tab, ps, pi, p2);
-                const float w3 = s_term<float, UNI>(d, tab, ps, pi, p3);
+                const float w1 = s_term<float, UNI, X>(d, tab, ps, pi, p1);
+                const float w2 = s_term<float, UNI, X>(d, tab, ps, pi, p2);
+                const float w3 = s_term<float, UNI, X>(d, tab, ps, pi, p3);
                 s += (w0 + w1) + (w2 + w3);
             } else {
                 s += w0;
-                if (k + 1 < cnt) s += s_term<float, UNI>(d, tab, ps, pi, p1);
-                if (k + 2 < cnt) s += s_term<float, UNI>(d, tab, ps, pi, p2);
+                if (k + 1 < cnt) s += s_term<float, UNI, X>(d, tab, ps, pi, p1);
+                if (k + 2 < cnt) s += s_term<float, UNI, X>(d, tab, ps, pi, p2);
             }
         }
         d.S[i] = s;
@@ -1350,7 +1382,7 @@ __device__ void s_pass_waves(const Dev<double>& d, const PairP<double>* tab, int
                 const PairP<double>& p = pair_of<double, UNI>(tab, type_of(pi), type_of(pj), d.ntypes, ps);
                 double dx, dy, dz, v, ft;
                 const double r2 = dist2_near(pi, pj, d, dx, dy, dz);
-                lj_eval(p, r2, v, ft);
+                lj_eval<kExpoAny, true>(p, r2, v, ft);
                 const bool in = r2 < p.rc2;
                 const double vh = r2 > p.rmin2 ? (p.vshift - v) * p.inv_epshat : 1.0;
                 SM::w()[x] = in ? mul_rn(p.a, vh) : 0.0;
@@ -1435,11 +1467,11 @@ __device__ __forceinline__ long long advance_fix(long long q0, long long Lq, lon
 // step that ends, the kinetic energy, and (opening) the half kick, half drift,
 // Langevin O step and half drift of the next (BAOAB; velocity Verlet without
 // O).  q[] (fixed point) and v are advanced in place, w[] gets the image
-// changes, np the new snapshot.  Returns the squared displacement of the drift
-// (0 when not opening).
+// changes, np the new snapshot.  z: the O step's normals (Langevin, opening).
+// Returns the squared displacement of the drift (0 when not opening).
 template <typename Real>
 __device__ __forceinline__ float advance_particle(const Dev<Real>& d, const RunArgs& a, Real fx, Real fy, Real fz,
-                                                  int flags, long long step, int wbits,
+                                                  int flags, const Real (&z)[3], int wbits,
                                                   typename Dev<Real>::R4& v, long long q[3], int w[3], Real& kin,
                                                   typename Dev<Real>::P4& np)
 {
@@ -1459,8 +1491,6 @@ __device__ __forceinline__ float advance_particle(const Dev<Real>& d, const RunA
         v.z += hdt * fz * im;
         Real ddx = hdt * v.x, ddy = hdt * v.y, ddz = hdt * v.z;
         if (a.langevin) {
-            Real z[3];
-            normals3(a.seed, step, (unsigned)(wbits >> kTypeBits), z);
             const Real c1 = pick(Real(0), a.c1_f, a.c1_d);
             const Real sd = pick(Real(0), a.c2_f, a.c2_d) * sqrt(im);
             v.x = c1 * v.x + sd * z[0];
@@ -1494,7 +1524,9 @@ __device__ __forceinline__ float integrate_one(const Dev<Real>& d, const RunArgs
     typename Dev<Real>::R4 v = st.v;
     typename Dev<Real>::P4 np;
     int w[3];
-    const float disp2 = advance_particle(d, a, fx, fy, fz, flags, step, wbits, v, st.q, w, kin, np);
+    Real z[3] = {Real(0), Real(0), Real(0)};
+    if ((flags & F_OPENING) && a.langevin) normals3(a.seed, step, (unsigned)(wbits >> kTypeBits), z);
+    const float disp2 = advance_particle(d, a, fx, fy, fz, flags, z, wbits, v, st.q, w, kin, np);
     if (flags & F_OPENING) {
         const int n = d.n;
 #pragma unroll
@@ -1516,7 +1548,7 @@ __device__ __forceinline__ float integrate_one(const Dev<Real>& d, const RunArgs
 // f (x_i - x_j)), with the entry's share of energies, virial and bond count
 // when TH (the sampled step of a launch).  REACT: a reactive pair (two-body
 // plus the three-body factor); else a purely two-body pair.
-template <typename Real, bool UNI, bool REACT, bool TH>
+template <typename Real, bool UNI, int X, bool REACT, bool TH>
 __device__ __forceinline__ void entry_force(const Dev<Real>& d, const PairP<Real>* tab,
                                             const typename Dev<Real>::P4& pi,
                                             const typename Dev<Real>::P4& pj, Real Si, Real Sj,
@@ -1530,7 +1562,7 @@ __device__ __forceinline__ void entry_force(const Dev<Real>& d, const PairP<Real
     // (no divergent branch: about half of the listed pairs lie in the skin)
     const bool in = r2 < p.rc2;
     Real v, ft;
-    lj_eval(p, r2, v, ft);
+    lj_eval<X, REACT>(p, r2, v, ft);
     if (TH) acc.q[Q_U2] += in ? Real(0.5) * (v + p.ushift) : Real(0);
     if (REACT) {
         const bool beyond = r2 > p.rmin2;
@@ -1594,7 +1626,7 @@ __device__ __forceinline__ void bond_forces(const Dev<Real>& d, const typename D
 // next S pass.  TH: the sampled step (the warps' thermo terms are left in
 // s_wacc, see block_sums_from_rows).  Returns the thread's largest squared
 // drift displacement.
-template <bool UNI, bool BONDS, bool TH>
+template <bool UNI, int X, bool BONDS, bool TH>
 __device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const RunArgs& a, int pc, int ac, int flags,
                              long long step, const PairP<float>& ps, const PairP<float>& pw)
 {
@@ -1649,14 +1681,14 @@ __device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const
             for (int q = 0; q < kNQA; q++) acc.q[q] = 0.0f;
         auto reactive = [&](const int4& pj, float Sj) {
             float ex, ey, ez;
-            entry_force<float, UNI, true, TH>(d, tab, pi, pj, Si, Sj, ps, acc, ex, ey, ez);
+            entry_force<float, UNI, X, true, TH>(d, tab, pi, pj, Si, Sj, ps, acc, ex, ey, ez);
             fx = __fadd_rn(fx, ex);
             fy = __fadd_rn(fy, ey);
             fz = __fadd_rn(fz, ez);
         };
         auto other = [&](const int4& pj) {
             float ex, ey, ez;
-            entry_force<float, UNI, false, TH>(d, tab, pi, pj, 0.0f, 0.0f, pw, acc, ex, ey, ez);
+            entry_force<float, UNI, X, false, TH>(d, tab, pi, pj, 0.0f, 0.0f, pw, acc, ex, ey, ez);
             gx = __fadd_rn(gx, ex);
             gy = __fadd_rn(gy, ey);
             gz = __fadd_rn(gz, ez);
@@ -1847,7 +1879,7 @@ __device__ float f_pass_waves(const Dev<double>& d, const PairP<double>* tab, co
                     const double Sj = react ? d.S[it.y] : 0.0;
                     const double r2 = dist2_near(pi, pj, d, dx, dy, dz);
                     const bool in = r2 < p.rc2;
-                    lj_eval(p, r2, v, ft);
+                    lj_eval<kExpoAny, true>(p, r2, v, ft);
                     ft = in ? ft : 0.0;
                     if (react) {
                         const bool beyond = r2 > p.rmin2;
@@ -1940,7 +1972,8 @@ struct LoopState {
     // resident mode (section below)
     int r_try;           // build the resident structures before the next step
     int r_valid;         // every block's resident structures are built and current
-    int r_gathered;      // the next step's copies were issued after the last barrier
+    int r_rb;            // threads that hold rows
+    unsigned r_epoch;    // publications of this launch
     int r_round;         // agreement round (selects ctl->rfail[round & 1])
     int r_fail;          // this block's structures do not fit
     int r_np, r_nh, r_nhr;  // own particles, halo particles, halo rows of S
@@ -2024,6 +2057,16 @@ __device__ __forceinline__ bool single_chunk(const Dev<Real>& d)
     return (d.n + g_size() - 1) / g_size() <= (int)blockDim.x;
 }
 
+// Runs f(std::integral_constant<int, X>) for the run's exponents (the same in
+// the whole block); uniform coefficients only can be kExpoStd.
+template <bool UNI, typename F>
+__device__ __forceinline__ void expo_switch(const RunArgs& a, F&& f)
+{
+    if (UNI && a.expo == kExpoStd) f(std::integral_constant<int, UNI ? kExpoStd : kExpoAny>());
+    else if (!kBatched && a.expo == kExpoEven) f(std::integral_constant<int, kBatched ? kExpoAny : kExpoEven>());
+    else f(std::integral_constant<int, kExpoAny>());
+}
+
 // The caller sets s_ls.own_ok after the grid barrier that follows (every warp
 // has read it by then).
 template <typename Real, bool UNI>
@@ -2031,7 +2074,9 @@ __device__ __forceinline__ void run_s_pass(const Dev<Real>& d, const RunArgs& a,
 {
     const bool staged = single_chunk(d) && s_ls.own_ok;
     if constexpr (sizeof(Real) == 4)
-        s_pass_rows<UNI>(d, stab<Real>(), s_ls.pc, uni_params(a, Real(0))[0], staged);
+        expo_switch<UNI>(a, [&](auto x) {
+            s_pass_rows<UNI, decltype(x)::value>(d, stab<Real>(), s_ls.pc, uni_params(a, Real(0))[0], staged);
+        });
     else
         s_pass_waves<UNI>(d, stab<Real>(), s_ls.pc, uni_params(a, Real(0))[0], staged, th);
 }
@@ -2049,9 +2094,12 @@ template <typename Real, bool UNI, bool BONDS, bool TH>
 __device__ __forceinline__ void run_f_pass(const Dev<Real>& d, const RunArgs& a, int flags, long long stp)
 {
     const PairP<Real>*ps = &uni_params(a, Real(0))[0], *pw = &uni_params(a, Real(0))[1];
-    float dmax;
+    float dmax = 0.0f;
     if constexpr (sizeof(Real) == 4)
-        dmax = f_pass_rows<UNI, BONDS, TH>(d, stab<Real>(), a, s_ls.pc, s_ls.ac, flags, stp, *ps, *pw);
+        expo_switch<UNI>(a, [&](auto x) {
+            dmax = f_pass_rows<UNI, decltype(x)::value, BONDS, TH>(d, stab<Real>(), a, s_ls.pc, s_ls.ac, flags, stp, *ps,
+                                                                   *pw);
+        });
     else
         dmax = f_pass_waves<UNI, BONDS, TH>(d, stab<Real>(), a, s_ls.pc, s_ls.ac, flags, stp, *ps, *pw);
     if (flags & F_OPENING) warp_max_disp(dmax);
@@ -2157,15 +2205,33 @@ __device__ __forceinline__ void add_disp(Ctl* ctl, long long stp)
 // reactive partner of those that are reactive partners of an own particle --
 // the own rows, and the reactive rows of that first halo shell (each the
 // owner's row, in the owner's order), all with partners as 16-bit local
-// indices.  A step then copies the halo's new snapshots in once (one
-// asynchronous 16-byte copy each), forms S for the own particles and for the reactive halo
-// from shared memory (a halo row is its owner's row, evaluated in the same
-// order with the same operations, so both blocks hold bit-identical S), and
-// the pair forces and the integrator with no further global gather: one grid
-// barrier per step instead of two, and no chains of dependent L2 round trips
-// inside a step.  Forces and trajectories are bit-identical to the two-barrier
-// path (same per-entry operations, same summation orders); only the thermo
-// partials are grouped differently.
+// indices.  A step then reads the halo's new snapshots once, forms S for the own
+// particles and for the reactive halo from shared memory (a halo row is its
+// owner's row, evaluated in the same order with the same operations, so both
+// blocks hold bit-identical S), and the pair forces and the integrator with no
+// further global gather.  Forces and trajectories are bit-identical to the
+// two-barrier path (same per-entry operations, same summation orders); only
+// the thermo partials are grouped differently.
+//
+// Steps follow one another by the data itself, without a grid barrier: a block
+// publishes each own snapshot as one 16-byte store whose top bit tells the
+// step (its parity over the writes of that buffer), and the blocks that hold
+// the particle in their halo read it until the bit is the expected one.  What
+// all blocks have to agree on, the displacement bound that asks for a list
+// build, comes along late: one warp posts the block's largest displacement and
+// its arrival, and waits for every block's while the others read the halo and
+// work on S and the forces; the step is thrown away before the integrator if
+// the list turns out to have to be rebuilt first.  A block posts publication k
+// after it has read its halo of publication k - 1, and writes publication k + 1
+// (into the buffer of k - 1) once all have posted k, so no snapshot is
+// overwritten early.
+// The posts are relaxed atomics on one cell of each of two 16-byte words in
+// turn: an agreement of 152 blocks that way takes 1,790 cycles, with release and
+// acquire 2,550, and with a slot per block that every block reads 6,100 (with
+// fences 9,500): the readers crowd the lines that are being written.  With a
+// grid barrier per step (arrival, poll, then the halo copies, nine block
+// barriers in all) a step of 512 particles took 7.3 us (6.2 this way, 4.1 with
+// the branch-free powers of pair_power), one of 100,000 14.8 (14.2, 12.4).
 
 struct RStage {
     static constexpr int kL = 3072;    // local particles: own (at most blockDim), then halo
@@ -2213,12 +2279,6 @@ struct RStage {
     static __device__ __forceinline__ int* img() { return (int*)(g_dyn + O_IMG); }
 };
 static_assert(RStage::kBytes <= 227 * 1024 - 12 * 1024, "the resident layout fits beside the static shared memory");
-
-__device__ __forceinline__ void cp_async_cg16(void* smem, const void* gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
 
 __device__ __forceinline__ unsigned r_hash(int q) { return ((unsigned)q * 2654435761u) >> 20; }
 
@@ -2287,8 +2347,8 @@ __device__ void r_sort_desc(const int (&key)[R], int (&pos)[R], int* hist)
     }
 }
 
-// Lays out warp blocks: rows at positions s (thread s % B, round s / B) with
-// n[r] entries each (0: no row); every warp block of 32 rows takes 32 x its
+// Lays out warp blocks: rows by (thread, round r) with n[r] entries each (0: no
+// row); every warp block of 32 rows takes 32 x its
 // longest row, in order (round, warp).  Returns the total (entries), and in
 // first[r] the entry of row r's lane (entry k of the row at first + 32 k).
 template <int R>
@@ -2391,15 +2451,17 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     }
     __syncthreads();
     // 5. rows of S (the own rows and the reactive first shell's), longest
-    // first, dealt out over the threads as a snake: rank s goes to round
-    // s / B, to thread s % B in even rounds and B - 1 - s % B in odd ones, so
+    // first, dealt out over the RB row threads as a snake: rank s goes to round
+    // s / RB, to thread s % RB in even rounds and RB - 1 - s % RB in odd ones, so
     // that a thread's second row is short when its first is long.  The force
     // pass runs two loops per thread, over a reactive row and over another
     // particle's other (purely two-body) row: reactive rows longest first
     // from warp 0, other rows longest first from the last warp, so that the
     // rows of a warp are alike in each loop and the warps' totals even out.
     const int NS = P + Hr;
-    const int rounds = (NS + B - 1) / B;
+    // the rows leave the last warp free for the slots (r_run) where they can
+    const int RB = P <= B - 32 && NS <= RR * (B - 32) ? B - 32 : B;
+    const int rounds = (NS + RB - 1) / RB;
     if (inf.y > 255 || inf.w > 255) fail = 1;
     int skey[RR + 1], spos[RR + 1], hrow[RR], hcnt[RR];
     skey[0] = t < P ? min(inf.y, 255) : -1;
@@ -2423,15 +2485,15 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     const int rpos = rank_desc(t < P ? inf.y : -1, RS::fent(), hist, s_int);
     const int wrank = rank_desc(t < P ? inf.w : -1, RS::fent(), hist, s_int);
     const int wpos = W32 - 32 - (wrank & ~31) + (wrank & 31);  // rank chunk c -> warp W32/32 - 1 - c
-    for (int q = t; q < rounds * B; q += B) RS::sdesc()[q] = make_int2(0, -1);  // no row here
+    for (int q = t; q < rounds * RB; q += B) RS::sdesc()[q] = make_int2(0, -1);  // no row here
     if (t < W32) RS::fdesc()[t] = make_int4(0, 0, 0, -1);  // no rows; centres 0xffff
     __syncthreads();
     // what each position needs: the centre and the row (start, count)
 #pragma unroll
     for (int r = 0; r <= RR; r++) {
         if (skey[r] < 0) continue;
-        const int sr = spos[r], g = sr / B, slot = sr - g * B;
-        const int q = g * B + ((g & 1) ? B - 1 - slot : slot);
+        const int sr = spos[r], g = sr / RB, slot = sr - g * RB;
+        const int q = g * RB + ((g & 1) ? RB - 1 - slot : slot);
         if (r == 0) {
             cen[q] = t;
             RS::sdesc()[q] = make_int2(inf.x, inf.y);
@@ -2458,8 +2520,8 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     int n[RR], first[RR];
 #pragma unroll
     for (int r = 0; r < RR; r++) {
-        const int q = t + r * B;
-        n[r] = r < rounds ? max(RS::sdesc()[q].y, 0) : 0;
+        const int q = t + r * RB;
+        n[r] = r < rounds && t < RB ? max(RS::sdesc()[q].y, 0) : 0;
     }
     const int ES = r_warp_layout<RR>(n, first, wl);
     const int4 fd = t < W32 ? RS::fdesc()[t] : make_int4(0, 0, 0, -1);
@@ -2470,8 +2532,8 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     // 7. the rows, partners as local indices
 #pragma unroll
     for (int r = 0; r < RR; r++) {
-        const int q = t + r * B;
-        if (r < rounds) {
+        const int q = t + r * RB;
+        if (r < rounds && t < RB) {
             const int2 src = RS::sdesc()[q];
             if (src.y >= 0) {
                 const int lid = cen[q];
@@ -2490,8 +2552,13 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
             fe[ER + wfirst[0] + 32 * m] = (unsigned short)r_lid(key, val, d.ent_j[(unsigned)(fd.y + m)], b0, b1, P, fail);
         RS::fdesc()[t] = make_int4(rfirst[0], ER + wfirst[0], fd.z, fd.w);
     }
-    if (t < P) lpos[t] = d.pos[pc][b0 + t];  // own snapshots by local index
+    if (t < P) {
+        const int4 own = d.pos[pc][b0 + t];
+        lpos[t] = own;               // own snapshots by local index
+        d.pos[pc ^ 1][b0 + t] = own; // top bit clear: the first publication into this buffer sets it
+    }
     if (t == 0) {
+        s_ls.r_rb = RB;
         s_ls.r_np = P;
         s_ls.r_nh = H;
         s_ls.r_nhr = Hr;
@@ -2511,16 +2578,18 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     return ok;
 }
 
-// Writes the own particles' state back to the global arrays (set ac): before
-// a list build reorders them, and when the run ends.
-__device__ __forceinline__ void r_flush(const Dev<float>& d, int ac)
+// Writes the own particles' state back to the global arrays (snapshots to set
+// pc, without the step's bit; the rest to set ac): before a list build reorders
+// them, and when the run ends.  Every block has read its halo of pos[pc].
+__device__ __forceinline__ void r_flush(const Dev<float>& d, int pc, int ac)
 {
     typedef RStage RS;
     const int t = threadIdx.x, n = d.n;
     if (t < s_ls.r_np) {
         int b0, b1;
         block_range(d, b0, b1);
-        const int i = b0 + (RS::fdesc()[t].w & 0xffff);
+        const int lid = RS::fdesc()[t].w & 0xffff, i = b0 + lid;
+        d.pos[pc][i] = RS::lpos()[lid];
         d.vel[ac][i] = RS::vel()[t];
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -2530,84 +2599,124 @@ __device__ __forceinline__ void r_flush(const Dev<float>& d, int ac)
     }
 }
 
-// Issues a step's copies of the halo's snapshots pos[pc] (through L2 only:
-// other blocks wrote them).
-__device__ __forceinline__ void r_gather(const Dev<float>& d, int pc)
+// A snapshot as one 16-byte access (single-copy atomic: a reader sees a whole
+// one), through L2.
+__device__ __forceinline__ int4 ld_snapshot(const int4* p)
 {
-    typedef RStage RS;
-    const int t = threadIdx.x, B = blockDim.x, P = s_ls.r_np, H = s_ls.r_nh;
-    int4* lpos = RS::lpos();
-    const int* hslot = RS::hslot();
-    const int4* pos = d.pos[pc];
-    for (int h = t; h < H; h += B) cp_async_cg16(&lpos[P + h], &pos[hslot[h]]);
-    cp_async_commit();
+    unsigned long long lo, hi;
+    asm volatile("{\n\t.reg .b128 v;\n\tld.relaxed.gpu.global.b128 v, [%2];\n\tmov.b128 {%0, %1}, v;\n\t}"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p)
+                 : "memory");
+    return make_int4((int)lo, (int)(lo >> 32), (int)hi, (int)(hi >> 32));
+}
+
+__device__ __forceinline__ void st_snapshot(int4* p, const int4& v)
+{
+    const unsigned long long lo = (unsigned)v.x | (unsigned long long)(unsigned)v.y << 32;
+    const unsigned long long hi = (unsigned)v.z | (unsigned long long)(unsigned)v.w << 32;
+    asm volatile("{\n\t.reg .b128 v;\n\tmov.b128 v, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], v;\n\t}" ::"l"(p), "l"(lo),
+                 "l"(hi)
+                 : "memory");
+}
+
+// One turn of a bounded wait: false once the time is up (or another wait's is).
+struct Patience {
+    int spins = 0;
+    long long t0 = 0;
+    __device__ __forceinline__ bool more(Ctl* ctl, long long timeout_ns, int where)
+    {
+        if (++spins < 64) return true;
+        if (spins == 64) t0 = gtimer_ns();
+        if (ld_relaxed(&ctl->status) & kStatusTimeout) return false;
+        if (gtimer_ns() - t0 > timeout_ns) {
+            atomicOr(&ctl->status, kStatusTimeout);
+            ctl->timeout_at = where;
+            return false;
+        }
+        return true;
+    }
+};
+
+// The top bit of publication k = 1, 2, ... since the resident structures were
+// built (two buffers in turn, both clear before).
+__device__ __forceinline__ unsigned r_bit(int k) { return ((unsigned)(((k - 1) >> 1) & 1) ^ 1u) << 31; }
+
+// Post and agreement of publication e = 1, 2, ... of a launch (one thread of the
+// block).  The word of e's parity: (arrivals, (publication, largest squared
+// displacement)); the second only grows, so neither is ever reset.  The
+// arrival is added after the maximum has come back.
+__device__ __forceinline__ void r_post(const Dev<float>& d, unsigned e)
+{
+    unsigned long long* w = d.agree + 2 * (e & 1);
+    const unsigned long long mine = (unsigned long long)e << 32 | s_ls.dmax_bits;
+    s_ls.dmax_bits = 0u;
+    unsigned long long old;
+    asm volatile("atom.relaxed.gpu.global.max.u64 %0, [%1], %2;" : "=l"(old) : "l"(w + 1), "l"(mine) : "memory");
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"(old == ~0ull ? 0ull : 1ull) : "memory");
+}
+
+__device__ __forceinline__ void r_agree(const Dev<float>& d, const RunArgs& a, unsigned e)
+{
+    const int4* w = (const int4*)(d.agree + 2 * (e & 1));
+    const unsigned long long want = (unsigned long long)((e + 1) / 2) * (unsigned)g_size();
+    Patience wait;
+    for (;;) {
+        const int4 v = ld_snapshot(w);
+        if (((unsigned long long)(unsigned)v.y << 32 | (unsigned)v.x) >= want) {
+            s_ls.disp += sqrtf(__int_as_float(v.z));
+            return;
+        }
+        if (!wait.more(d.ctl, a.timeout_ns, 22)) {
+            s_ls.ok = 0;
+            return;
+        }
+    }
 }
 
 // S of one row (entries e[0], e[32], ...) with the two-barrier path's order of
 // additions (groups of four, then one by one).
-template <bool UNI>
+template <bool UNI, int X>
 __device__ __forceinline__ float r_row_s(const Dev<float>& d, const PairP<float>* tab, const PairP<float>& ps,
                                          const int4* lpos, const unsigned short* e, int cnt, const int4& pi)
 {
     float s = 0.0f;
     int k = 0;
     for (; k + 4 <= cnt; k += 4) {
-        const float w0 = s_term<float, UNI>(d, tab, ps, pi, lpos[e[32 * k]]);
-        const float w1 = s_term<float, UNI>(d, tab, ps, pi, lpos[e[32 * (k + 1)]]);
-        const float w2 = s_term<float, UNI>(d, tab, ps, pi, lpos[e[32 * (k + 2)]]);
-        const float w3 = s_term<float, UNI>(d, tab, ps, pi, lpos[e[32 * (k + 3)]]);
+        const float w0 = s_term<float, UNI, X>(d, tab, ps, pi, lpos[e[32 * k]]);
+        const float w1 = s_term<float, UNI, X>(d, tab, ps, pi, lpos[e[32 * (k + 1)]]);
+        const float w2 = s_term<float, UNI, X>(d, tab, ps, pi, lpos[e[32 * (k + 2)]]);
+        const float w3 = s_term<float, UNI, X>(d, tab, ps, pi, lpos[e[32 * (k + 3)]]);
         s += (w0 + w1) + (w2 + w3);
     }
-    for (; k < cnt; k++) s += s_term<float, UNI>(d, tab, ps, pi, lpos[e[32 * k]]);
+    for (; k < cnt; k++) s += s_term<float, UNI, X>(d, tab, ps, pi, lpos[e[32 * k]]);
     return s;
 }
 
-// One resident step: S of the own particles and the reactive halo, the pair
-// forces of the own rows (entry order: reactive, then the others), the
-// integrator.  TH (the sampled step): the thermo terms are left summed per
-// warp in s_wpart (thermo_partials completes the block sums).  Returns the
-// thread's squared drift displacement.
-template <bool UNI, bool TH>
-__device__ float r_step(const Dev<float>& d, const RunArgs& a, int flags, long long step)
+// The pair forces of a thread's rows: the other (purely two-body) row of one
+// particle, whose sum goes to fw, and the reactive row of particle lid into f.
+// TH (the sampled step): the pair terms are left summed per warp in s_wpart
+// (so that the accumulators are not live through the integrator).
+template <bool UNI, int X, bool TH>
+__device__ __forceinline__ void r_forces(const Dev<float>& d, const RunArgs& a, int P, const int4& fd, float& fx,
+                                         float& fy, float& fz)
 {
-    Acc<float> acc;
     typedef RStage RS;
-    const int t = threadIdx.x, B = blockDim.x;
-    const int P = s_ls.r_np, NQ = (P + s_ls.r_nhr + B - 1) / B * B;  // positions of the rows of S
-    const int pc = s_ls.pc;
-    int b0, b1;
-    block_range(d, b0, b1);
-    if (!s_ls.r_gathered) r_gather(d, pc);
-    cp_async_wait_all();
-    __syncthreads();
+    const int t = threadIdx.x;
     const PairP<float>* tab = stab<float>();
     const PairP<float>& ps = a.uf[0];
     const PairP<float>& pw = a.uf[1];
-    int4* lpos = RS::lpos();
-    float* lS = RS::lS();
-    for (int q = t; q < NQ; q += B) {
-        const int2 dsc = RS::sdesc()[q];
-        if (dsc.y < 0) continue;  // no row at this position
-        const int lid = dsc.y & 0xffff;
-        lS[lid] = r_row_s<UNI>(d, tab, ps, lpos, RS::sent() + dsc.x, (int)((unsigned)dsc.y >> 16), lpos[lid]);
-    }
-    __syncthreads();
+    const int4* lpos = RS::lpos();
+    const float* lS = RS::lS();
+    float* fw = RS::fw();
+    Acc<float> acc;
     if (TH)
 #pragma unroll
         for (int q = 0; q < kNQA; q++) acc.q[q] = 0.0f;
-    float dmax = 0.0f, kin = 0.0f;
-    float fx = 0.0f, fy = 0.0f, fz = 0.0f;
-    int4 pi = make_int4(0, 0, 0, 0);
-    int lid = 0;
-    float* fw = RS::fw();
     if (t < ((P + 31) & ~31)) {
-        const int4 fd = RS::fdesc()[t];
         const int nr = fd.z & 0xffff, nw = (int)((unsigned)fd.z >> 16);
         const int cw = (int)((unsigned)fd.w >> 16);
-        lid = fd.w & 0xffff;
         if (cw != 0xffff) {
-            // the other (purely two-body) row of particle cw: its sum goes to
-            // fw, for the thread that integrates cw
             const unsigned short* ew = RS::fent() + fd.y;
             const int4 pc_ = lpos[cw];
             float gx = 0.0f, gy = 0.0f, gz = 0.0f;
@@ -2615,7 +2724,7 @@ __device__ float r_step(const Dev<float>& d, const RunArgs& a, int flags, long l
             for (int k = 0; k < nw; k++) {
                 const int j = ew[32 * k];
                 float ex, ey, ez;
-                entry_force<float, UNI, false, TH>(d, tab, pc_, lpos[j], 0.0f, 0.0f, pw, acc, ex, ey, ez);
+                entry_force<float, UNI, X, false, TH>(d, tab, pc_, lpos[j], 0.0f, 0.0f, pw, acc, ex, ey, ez);
                 gx = __fadd_rn(gx, ex);
                 gy = __fadd_rn(gy, ey);
                 gz = __fadd_rn(gz, ez);
@@ -2625,26 +2734,23 @@ __device__ float r_step(const Dev<float>& d, const RunArgs& a, int flags, long l
             fw[2 * kBlock + cw] = gz;
         }
         if (t < P) {
-            // the reactive row of particle lid
+            const int lid = fd.w & 0xffff;
             const unsigned short* er = RS::fent() + fd.x;
-            pi = lpos[lid];
+            const int4 pi = lpos[lid];
             const float Si = lS[lid];
 #pragma unroll 2
             for (int k = 0; k < nr; k++) {
                 const int j = er[32 * k];
                 float ex, ey, ez;
-                entry_force<float, UNI, true, TH>(d, tab, pi, lpos[j], Si, lS[j], ps, acc, ex, ey, ez);
+                entry_force<float, UNI, X, true, TH>(d, tab, pi, lpos[j], Si, lS[j], ps, acc, ex, ey, ez);
                 fx = __fadd_rn(fx, ex);
                 fy = __fadd_rn(fy, ey);
                 fz = __fadd_rn(fz, ez);
             }
         }
     }
-    // the pair terms go to the warp partials now, so that the accumulators are
-    // not live through the integrator (the kinetic term follows it)
-    const bool rows = (t & ~31) < P;  // the warp holds rows (the same in all its lanes)
     if (TH) {
-        if (rows) {
+        if ((t & ~31) < P) {  // the warp holds rows (the same in all its lanes)
 #pragma unroll
             for (int q = 0; q < kNQA; q++)
                 if (q != Q_K) warp_part(acc.q[q], q);
@@ -2654,45 +2760,185 @@ __device__ float r_step(const Dev<float>& d, const RunArgs& a, int flags, long l
                 if (q != Q_K) s_wpart[q][t >> 5] = 0.0f;
         }
     }
-    __syncthreads();  // every row has read the old snapshots, and fw is complete
-    if (t < P) {
-        const int i = b0 + lid;
-        // the force: the reactive row's sum plus the other row's
-        fx = __fadd_rn(fx, fw[lid]);
-        fy = __fadd_rn(fy, fw[kBlock + lid]);
-        fz = __fadd_rn(fz, fw[2 * kBlock + lid]);
-        if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(&d.ctl->status, kStatusNonfinite);
-        if (flags & F_STORE) d.force[i] = make_float4(fx, fy, fz, 0.0f);
-        float4 v = RS::vel()[t];
-        long long q[3];
-        int w[3];
-#pragma unroll
-        for (int c = 0; c < 3; c++) q[c] = RS::xq()[3 * t + c];
-        int4 np = make_int4(0, 0, 0, 0);
-        dmax = advance_particle(d, a, fx, fy, fz, flags, step, pi.w, v, q, w, kin, np);
-        if (flags & F_OPENING) {
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                RS::xq()[3 * t + c] = q[c];
-                RS::img()[3 * t + c] += w[c];
-            }
-            d.pos[pc ^ 1][i] = np;  // the other blocks' halos read it
-            lpos[lid] = np;
+}
+
+// Resident steps until the run's last one is done (1), the list has to be
+// rebuilt before the next (2) or a wait ran out (0).  The loop's state is the
+// same in every thread.
+template <bool UNI, int X>
+static __device__ int r_run(const Dev<float>& d, const RunArgs& a)
+{
+    typedef RStage RS;
+    const int t = threadIdx.x, B = blockDim.x, warp = t >> 5, last_warp = (B >> 5) - 1;
+    const int P = s_ls.r_np, H = s_ls.r_nh, RB = s_ls.r_rb;
+    const int NQ = (P + s_ls.r_nhr + RB - 1) / RB * RB;  // positions of the rows of S
+    const bool spare = RB < B;                           // the last warp has no rows
+    int b0, b1;
+    block_range(d, b0, b1);
+    int pc = s_ls.pc, remaining = s_ls.remaining, k = 0;
+    long long step = s_ls.step;
+    unsigned epoch = s_ls.r_epoch;
+    int tl_left = s_ls.tlog_left, tl_slot = s_ls.tlog_slot, tl_n = 0;
+    const float skin_eff = (float)a.skin_eff;
+    int4* lpos = RS::lpos();
+    float* lS = RS::lS();
+    const int* hslot = RS::hslot();
+    double* lg = nullptr;  // record of the previous step, its warps' sums not yet added up
+    int result = 0;
+    for (;;) {
+        const bool more = remaining > 1, logged = tl_left == 1, th = !more || logged;
+        if (spare && k > 0 && warp == last_warp) {
+            asm volatile("bar.sync 2, %0;" ::"r"(B) : "memory");  // every row warp's maximum is in
+            if (t == B - 32) r_post(d, epoch);
         }
-        RS::vel()[t] = v;
+        // the halo's snapshots (complete at the first step)
+        const int4* pos = d.pos[pc];
+        const unsigned bit = r_bit(k), care = k > 0 ? 0x80000000u : 0u;
+        int4 v0 = make_int4(0, 0, 0, 0), v1 = v0;
+        bool w0 = t < RB && t < H, w1 = t < RB && t + RB < H;
+        if (w0) v0 = ld_snapshot(&pos[hslot[t]]);
+        if (w1) v1 = ld_snapshot(&pos[hslot[t + RB]]);
+        if (lg) {
+            __syncthreads();
+            warp_sums_to(lg, nullptr);
+            lg = nullptr;
+        }
+        int ok = 1;
+        for (int h = t; w0; h += 2 * RB) {
+            Patience wait;
+            for (;;) {
+                if (w0 && (((unsigned)v0.w ^ bit) & care) == 0) {
+                    v0.w &= 0x7fffffff;
+                    lpos[P + h] = v0;
+                    w0 = false;
+                }
+                if (w1 && (((unsigned)v1.w ^ bit) & care) == 0) {
+                    v1.w &= 0x7fffffff;
+                    lpos[P + h + RB] = v1;
+                    w1 = false;
+                }
+                if (!w0 && !w1) break;
+                if (!wait.more(d.ctl, a.timeout_ns, 23)) {
+                    ok = 0;
+                    break;
+                }
+                if (w0) v0 = ld_snapshot(&pos[hslot[h]]);
+                if (w1) v1 = ld_snapshot(&pos[hslot[h + RB]]);
+            }
+            w0 = ok && h + 2 * RB < H;
+            w1 = ok && h + 3 * RB < H;
+            if (w0) v0 = ld_snapshot(&pos[hslot[h + 2 * RB]]);
+            if (w1) v1 = ld_snapshot(&pos[hslot[h + 3 * RB]]);
+        }
+        if (!__syncthreads_and(ok)) break;
+        if (spare && k > 0 && t == B - 32) r_agree(d, a, epoch);
+        if (!spare && k > 0 && t == B - 32) r_post(d, epoch);
+        int4 fd = make_int4(0, 0, 0, -1);
+        float fx = 0.0f, fy = 0.0f, fz = 0.0f;
+        if (t < RB) {
+            const PairP<float>* tab = stab<float>();
+            for (int q = t; q < NQ; q += RB) {
+                const int2 dsc = RS::sdesc()[q];
+                if (dsc.y < 0) continue;  // no row at this position
+                const int lid = dsc.y & 0xffff;
+                lS[lid] = r_row_s<UNI, X>(d, tab, a.uf[0], lpos, RS::sent() + dsc.x, (int)((unsigned)dsc.y >> 16), lpos[lid]);
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(RB) : "memory");  // the row threads (whole warps)
+            if (t < ((P + 31) & ~31)) fd = RS::fdesc()[t];
+        }
+        if (th) r_forces<UNI, X, true>(d, a, P, fd, fx, fy, fz);
+        else if (t < RB) r_forces<UNI, X, false>(d, a, P, fd, fx, fy, fz);
+        if (!spare && k > 0 && t == B - 32) r_agree(d, a, epoch);
+        // the noise of the next step's start, while the agreement is on its way
+        float z[3] = {0.0f, 0.0f, 0.0f};
+        const int lid = fd.w & 0xffff;
+        if (t < P && more && a.langevin) normals3(a.seed, step + 1, (unsigned)(lpos[lid].w >> kTypeBits), z);
+        __syncthreads();  // every row has read the old snapshots, fw is complete, the displacement bound is known
+        if (k > 0) {
+            if (!s_ls.ok) break;
+            if (2.0f * s_ls.disp > skin_eff) {
+                result = 2;
+                break;
+            }
+        }
+        float kin = 0.0f, dmax = 0.0f;
+        if (t < P) {
+            const float* fw = RS::fw();
+            const int i = b0 + lid;
+            const int4 pi = lpos[lid];
+            // the force: the reactive row's sum plus the other row's
+            fx = __fadd_rn(fx, fw[lid]);
+            fy = __fadd_rn(fy, fw[kBlock + lid]);
+            fz = __fadd_rn(fz, fw[2 * kBlock + lid]);
+            if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(&d.ctl->status, kStatusNonfinite);
+            if (!more) d.force[i] = make_float4(fx, fy, fz, 0.0f);
+            float4 v = RS::vel()[t];
+            long long q[3];
+            int w[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) q[c] = RS::xq()[3 * t + c];
+            int4 np = make_int4(0, 0, 0, 0);
+            dmax = advance_particle(d, a, fx, fy, fz, F_CLOSING | (more ? F_OPENING : 0), z, pi.w, v, q, w, kin, np);
+            if (more) {
+                int4 pub = np;
+                pub.w |= (int)r_bit(k + 1);
+                st_snapshot(&d.pos[pc ^ 1][i], pub);
+                lpos[lid] = np;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    RS::xq()[3 * t + c] = q[c];
+                    if (w[c]) RS::img()[3 * t + c] += w[c];
+                }
+            }
+            RS::vel()[t] = v;
+        }
+        if (th) {
+            if ((t & ~31) < P)
+                warp_part(kin, Q_K);
+            else if ((t & 31) == 0)
+                s_wpart[Q_K][t >> 5] = 0.0f;
+        }
+        step++;
+        remaining--;
+        if (tl_left > 0) tl_left = logged ? a.tlog_every : tl_left - 1;
+        if (logged) {
+            lg = d.tlog + ((size_t)tl_slot * a.max_blocks + g_rank()) * kNQ;
+            if (t == 0 && g_rank() == 0) {
+                d.tlog_step[2 * tl_slot] = step;
+                d.tlog_step[2 * tl_slot + 1] = g_size();
+            }
+            tl_n++;
+            tl_slot = tl_slot + 1 == d.tlog_cap ? 0 : tl_slot + 1;
+        }
+        if (!more) {
+            thermo_partials(d, true, true, lg);
+            result = 1;
+            break;
+        }
+        if (t < RB) {
+            warp_max_disp(dmax);
+            if (spare) asm volatile("bar.arrive 2, %0;" ::"r"(B) : "memory");
+        }
+        k++;
+        epoch++;
+        pc ^= 1;
     }
-    if (TH) {
-        if (rows)
-            warp_part(kin, Q_K);
-        else if ((t & 31) == 0)
-            s_wpart[Q_K][t >> 5] = 0.0f;
-    }
+    __syncthreads();
     if (t == 0) {
-        s_ls.r_gathered = 0;
-        s_ls.r_steps++;
+        const int done = s_ls.remaining - remaining;
+        s_ls.step = step;
+        s_ls.remaining = remaining;
+        s_ls.done += done;
+        s_ls.r_steps += done;
+        s_ls.pc = pc;
+        s_ls.r_epoch = epoch;
+        s_ls.tlog_left = tl_left;
+        s_ls.tlog_slot = tl_slot;
+        s_ls.tlog_k += tl_n;
         s_ls.own_ok = 0;
     }
-    return dmax;
+    __syncthreads();
+    return result;
 }
 
 // Builds every block's resident structures and agrees on the mode: the step
@@ -2707,7 +2953,6 @@ static __device__ bool r_enter(const Dev<float>& d, const RunArgs& a)
         s_ls.r_valid = ld_relaxed(&d.ctl->rfail[round & 1]) == 0;
         s_ls.r_try = 0;  // tried again after the next list build
         s_ls.r_round = round + 1;
-        s_ls.r_gathered = 0;
         s_ls.own_ok = 0;  // the build overwrote the two-barrier path's staging
         // the next round's word: every block reads this round's word before it
         // arrives at the next barrier, and the next round comes after it
@@ -2751,7 +2996,9 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
         s_ls.own_ok = 0;
         s_ls.r_try = (kRes && a.resident && single_chunk(d)) ? 1 : 0;
         s_ls.r_valid = 0;
-        s_ls.r_gathered = 0;
+        s_ls.r_rb = 0;
+        s_ls.r_epoch = 0;
+        s_ls.ok = 1;
         s_ls.r_round = 0;
         s_ls.r_fail = 0;
         s_ls.r_np = s_ls.r_nh = s_ls.r_nhr = 0;
@@ -2815,27 +3062,17 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
             if (!grid_barrier(ctl, a.timeout_ns, 13, &ctl->dmax2[stp & 1])) return false;
             add_disp(ctl, stp);
         }
-        [[maybe_unused]] unsigned dm_pending = 0u;  // thread 0: the displacement maximum read after a resident barrier
         while (s_ls.rc == 0 && s_ls.state == 2) {
             const long long stp = s_ls.step;
-            if (threadIdx.x == 0 && g_rank() == 0) ctl->dmax2[(stp + 1) & 1] = 0u;
-#if SWP_HAS_RESIDENT
-            if constexpr (kRes) {
-                if (s_ls.r_gathered) {
-                    // the halo copies and the displacement read issued after the
-                    // last barrier were in flight together until here
-                    cp_async_wait_all();
-                    if (threadIdx.x == 0) s_ls.disp += sqrtf(__uint_as_float(dm_pending));
-                    __syncthreads();
-                }
-            }
-#endif
             if (s_ls.need_rb || 2.0f * s_ls.disp > skin_eff) {
-                // a resident gather issued for this step lands in memory the rebuild reuses
-                cp_async_wait_all();
 #if SWP_HAS_RESIDENT
                 if constexpr (kRes)
-                    if (s_ls.r_valid) r_flush(d, s_ls.ac);  // the build reorders the global state
+                    if (s_ls.r_valid) {
+                        // every block has read its halo; then the global state is
+                        // brought up to date for the build to reorder
+                        if (!grid_barrier(ctl, a.timeout_ns, 24)) return false;
+                        r_flush(d, s_ls.pc, s_ls.ac);
+                    }
 #endif
                 const int rc = run_rebuild(d, a);
                 if (rc == 2) return false;
@@ -2843,41 +3080,43 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
                     s_ls.need_rb = rc;
                     s_ls.rc = rc;
                     s_ls.r_valid = 0;
-                    s_ls.r_gathered = 0;
                     s_ls.r_try = (kRes && a.resident && single_chunk(d)) ? 1 : 0;
                 }
                 __syncthreads();
                 if (rc) break;
             }
+#if SWP_HAS_RESIDENT
+            if constexpr (kRes) {
+                if (s_ls.r_try)
+                    if (!r_enter(d, a)) return false;
+                if (s_ls.r_valid) {
+                    int rc = 0;
+                    expo_switch<UNI>(a, [&](auto x) { rc = r_run<UNI, decltype(x)::value>(d, a); });
+                    if (rc == 0) return false;
+                    if (rc == 1) {  // the last step is done: its partials are complete after the barrier
+                        if (!grid_barrier(ctl, a.timeout_ns, 21)) return false;
+                        if (threadIdx.x == 0) s_ls.state = 0;
+                        __syncthreads();
+                    }
+                    continue;
+                }
+            }
+#endif
             const bool more = s_ls.remaining > 1;
             // the thermo terms are summed on the launch's last step (the one a
             // launch reports) and on the logged steps only
             const bool logged = s_ls.tlog_left == 1;
             const bool th = !more || logged;
             const int flags = F_CLOSING | (more ? F_OPENING : F_STORE);
-            bool resident = false;
-#if SWP_HAS_RESIDENT
-            if constexpr (kRes) {
-                if (s_ls.r_try)
-                    if (!r_enter(d, a)) return false;
-                if (s_ls.r_valid) {
-                    const float dmax = th ? r_step<UNI, true>(d, a, flags, stp + 1)
-                                          : r_step<UNI, false>(d, a, flags, stp + 1);
-                    if (more) warp_max_disp(dmax);
-                    resident = true;
-                }
-            }
-#endif
-            if (!resident) {
-                run_s_pass<Real, UNI>(d, a, th);
-                if (!grid_barrier(ctl, a.timeout_ns, 20)) return false;
-                if (threadIdx.x == 0) s_ls.own_ok = single_chunk(d);
-                if (th)
-                    run_f_pass<Real, UNI, BONDS, true>(d, a, flags, stp + 1);
-                else
-                    run_f_pass<Real, UNI, BONDS, false>(d, a, flags, stp + 1);
-            }
-            if (threadIdx.x == 0) {  // every thread read `remaining` before the pass's barriers
+            if (threadIdx.x == 0 && g_rank() == 0) ctl->dmax2[(stp + 1) & 1] = 0u;
+            run_s_pass<Real, UNI>(d, a, th);
+            if (!grid_barrier(ctl, a.timeout_ns, 20)) return false;
+            if (threadIdx.x == 0) s_ls.own_ok = single_chunk(d);
+            if (th)
+                run_f_pass<Real, UNI, BONDS, true>(d, a, flags, stp + 1);
+            else
+                run_f_pass<Real, UNI, BONDS, false>(d, a, flags, stp + 1);
+            if (threadIdx.x == 0) {  // every thread read these before the passes' barrier
                 s_ls.step = stp + 1;
                 s_ls.remaining--;
                 s_ls.done++;
@@ -2888,44 +3127,15 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
                 d.tlog_step[2 * s_ls.tlog_slot] = stp + 1;
                 d.tlog_step[2 * s_ls.tlog_slot + 1] = g_size();
             }
-            // a logged resident step that is not the launch's last sums its
-            // warps' thermo terms while it waits at the barrier (the record is
-            // read after the launch); the launch's last step writes the
-            // partials the launch reduces, before its arrival
-            const bool late = resident && more;
-            if (th && !late) thermo_partials(d, resident, !more, lg);
-            unsigned* pub = more ? &ctl->dmax2[(stp + 1) & 1] : nullptr;
-            {
-                BarState bs;
-                bs.target = s_ls.bar_target;
-                bar_arrive(ctl, bs, pub, &s_ls.dmax_bits);
-                if (th && late) warp_sums_to(lg, nullptr);  // bar_arrive ordered the s_wpart writes
-                if (threadIdx.x == 0) s_ls.bar_target = bs.target;
-                if (!bar_wait(ctl, bs, a.timeout_ns, 21, &s_ls.ok)) return false;
-            }
+            if (th) thermo_partials(d, false, !more, lg);
+            if (!grid_barrier(ctl, a.timeout_ns, 21, more ? &ctl->dmax2[(stp + 1) & 1] : nullptr)) return false;
             if (logged && threadIdx.x == 0) {  // every thread used the slot before the barrier
                 s_ls.tlog_k++;
                 s_ls.tlog_slot = s_ls.tlog_slot + 1 == d.tlog_cap ? 0 : s_ls.tlog_slot + 1;
             }
             if (more) {
                 if (threadIdx.x == 0) s_ls.pc ^= 1;
-                __syncthreads();
-                bool gathered = false;
-#if SWP_HAS_RESIDENT
-                if constexpr (kRes) {
-                    if (s_ls.r_valid) {
-                        // the displacement read and the next step's copies
-                        // overlap; the read is used after the copies land (top
-                        // of the loop)
-                        if (threadIdx.x == 0) dm_pending = (unsigned)ld_relaxed((const int*)pub);
-                        r_gather(d, s_ls.pc);
-                        if (threadIdx.x == 0) s_ls.r_gathered = 1;
-                        __syncthreads();
-                        gathered = true;
-                    }
-                }
-#endif
-                if (!gathered) add_disp(ctl, stp + 1);
+                add_disp(ctl, stp + 1);
             } else {
                 if (threadIdx.x == 0) s_ls.state = 0;
                 __syncthreads();
@@ -2935,7 +3145,7 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
     cp_async_wait_all();  // copies issued for a step that did not come
 #if SWP_HAS_RESIDENT
     if constexpr (kRes)
-        if (s_ls.r_valid) r_flush(d, s_ls.ac);
+        if (s_ls.r_valid) r_flush(d, s_ls.pc, s_ls.ac);
 #endif
     if (s_ls.have_thermo) {
         // the partials were written before the arrival at the barrier that
@@ -3137,10 +3347,7 @@ __global__ void k_get_nlist(Dev<Real> d, int pc, int* rows, int* counts, int wid
 template <typename Real>
 __device__ __forceinline__ Real pair_x(const PairP<Real>& p, Real r2)
 {
-    const Real s2 = p.sig2 * recip(r2);
-    Real x = ipow(s2, p.nhalf);
-    if (p.odd) x *= sqrt(s2);
-    return x;
+    return pair_power<kExpoAny, true>(p, p.sig2 * recip(r2));
 }
 
 // The two passes give each particle kPgLanes consecutive lanes of a warp:

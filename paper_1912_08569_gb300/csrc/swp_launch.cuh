@@ -17,9 +17,8 @@ namespace swp {
 using single::Stage;
 
 template <typename Real>
-static void* run_fn(int uni, int bonds = 0)
+static void* run_fn(int uni)
 {
-    if (bonds) return uni ? (void*)single::k_run<Real, true, true> : (void*)single::k_run<Real, false, true>;
     return uni ? (void*)single::k_run<Real, true, false> : (void*)single::k_run<Real, false, false>;
 }
 
@@ -36,7 +35,7 @@ size_t run_smem_bytes()
 template <typename Real>
 static size_t launch_smem_bytes(const Dev<Real>& d, const RunArgs& a, int grid)
 {
-    const bool resident = a.resident && !d.has_bonds && (d.n + grid - 1) / grid <= kBlock;
+    const bool resident = a.resident && (d.n + grid - 1) / grid <= kBlock;
     return resident ? run_smem_bytes<Real>() : Stage<Real>::kBytes;
 }
 
@@ -51,7 +50,7 @@ static cudaError_t prepare_fn(void* fn)
 template <typename Real>
 cudaError_t launch_run(const Dev<Real>& d, const RunArgs& a, int grid, int block, cudaStream_t s)
 {
-    void* fn = run_fn<Real>(a.uni, d.has_bonds);
+    void* fn = run_fn<Real>(a.uni);
     cudaError_t e = prepare_fn<Real>(fn);
     if (e != cudaSuccess) return e;
     Dev<Real> dd = d;
@@ -65,8 +64,8 @@ cudaError_t run_occupancy(int block, int* blocks_per_sm)
 {
     int best = 1 << 30;
     cudaError_t e = cudaSuccess;
-    for (int v = 0; v < 4 && e == cudaSuccess; v++) {  // every (uniform, bonds) variant
-        void* fn = run_fn<Real>(v & 1, v >> 1);
+    for (int v = 0; v < 2 && e == cudaSuccess; v++) {  // uniform coefficients or not
+        void* fn = run_fn<Real>(v);
         int b = 0;
         e = prepare_fn<Real>(fn);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, block, run_smem_bytes<Real>());

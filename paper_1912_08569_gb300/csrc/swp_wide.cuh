@@ -14,16 +14,15 @@
 namespace swp {
 
 template <typename Real>
-static void* run_fn_wide(int uni, int bonds)
+static void* run_fn_wide(int uni)
 {
-    if (bonds) return uni ? (void*)wide::k_run<Real, true, true> : (void*)wide::k_run<Real, false, true>;
-    return uni ? (void*)wide::k_run<Real, true, false> : (void*)wide::k_run<Real, false, false>;
+    return uni ? (void*)wide::k_run<Real, true, true> : (void*)wide::k_run<Real, false, true>;
 }
 
 template <typename Real>
 cudaError_t launch_run_wide(const Dev<Real>& d, const RunArgs& a, int grid, cudaStream_t s)
 {
-    void* fn = run_fn_wide<Real>(a.uni, d.has_bonds);
+    void* fn = run_fn_wide<Real>(a.uni);
     const size_t sm = wide::Stage<Real>::kBytes;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -33,15 +32,15 @@ cudaError_t launch_run_wide(const Dev<Real>& d, const RunArgs& a, int grid, cuda
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kBlockWide), args, sm, s);
 }
 
-// Blocks per SM that every (uniform, bonds) variant reaches.
+// Blocks per SM that both variants (uniform coefficients or not) reach.
 template <typename Real>
 cudaError_t run_occupancy_wide(int* blocks_per_sm)
 {
     const int sm = (int)wide::Stage<Real>::kBytes;
     int best = 1 << 30;
     cudaError_t e = cudaSuccess;
-    for (int v = 0; v < 4 && e == cudaSuccess; v++) {
-        void* fn = run_fn_wide<Real>(v & 1, v >> 1);
+    for (int v = 0; v < 2 && e == cudaSuccess; v++) {
+        void* fn = run_fn_wide<Real>(v);
         int b = 0;
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kBlockWide, sm);
