@@ -2256,15 +2256,16 @@ struct RStage {
     static constexpr size_t O_IMG = O_XQ + (size_t)kBlock * 24;     // [3 kBlock] image counts
     static constexpr size_t kBytes = O_IMG + (size_t)kBlock * 12;
     // While building, the own-state area holds the hash table (keys, values),
-    // the sort histogram and the warp-block lengths; O_SENT holds the
-    // reactive first shell's table indices, O_LS the centres of the rows of S
-    // by position.
+    // the sorts' histograms and the warp-block lengths; O_SENT holds the reactive
+    // first shell's table indices, O_FENT the force rows' per-warp counts, O_LS
+    // the centres of the rows of S by position.
     static constexpr size_t B_KEY = O_VEL, B_VAL = B_KEY + (size_t)kHash * 4, B_HIST = B_VAL + (size_t)kHash * 4,
-                            B_WL = B_HIST + 256 * 4, B_END = B_WL + ((size_t)kRounds * 32 + 1) * 4;
+                            B_WL = B_HIST + 3 * 256 * 4, B_END = B_WL + ((size_t)(kRounds + 2) * 33) * 4;
     static_assert(B_END <= kBytes, "build scratch fits the own-state area");
     static_assert(kES <= 65536 && kEF <= 65536 && kL <= 65536, "16-bit local indices and offsets");
     static_assert(kBlock % 32 == 0 && kBlock / 32 <= 32, "whole warps, at most 32");
-    static_assert(kBlock >= 256 && kEF >= kBlock / 32 * 256, "force-row sort scratch (rank_desc) in O_FENT");
+    static_assert(kBlock >= 768 && kEF >= kBlock / 32 * 512, "force-row sort scratch in O_FENT");
+    static_assert(kES >= 2 * kHash, "the reactive first shell's table indices in O_SENT");
 
     static __device__ __forceinline__ int4* lpos() { return (int4*)(g_dyn + O_LPOS); }
     static __device__ __forceinline__ float* lS() { return (float*)(g_dyn + O_LS); }
@@ -2282,118 +2283,125 @@ static_assert(RStage::kBytes <= 227 * 1024 - 12 * 1024, "the resident layout fit
 
 __device__ __forceinline__ unsigned r_hash(int q) { return ((unsigned)q * 2654435761u) >> 20; }
 
-// Inserts slot q into the table (if absent); its index, or -1 when full.
-__device__ __forceinline__ int r_insert(int* key, int q)
+static __shared__ int s_nh, s_nhr;  // halo particles, halo rows of S (while building)
+
+// Inserts slot q into the table (if absent; a new one gets the next local index
+// after the P own particles); its place, or -1 when there is no room.  val:
+// bit 0 reactive partner of an own particle, then the rank in the halo.
+__device__ __forceinline__ int r_insert(int* key, int* val, int q, int P)
 {
     unsigned h = r_hash(q) & (RStage::kHash - 1);
     for (int probe = 0; probe < RStage::kHash; probe++) {
         const int old = atomicCAS(&key[h], -1, q);
+        if (old == -1) {
+            const int r = atomicAdd(&s_nh, 1);
+            if (P + r >= RStage::kL) return -1;
+            RStage::hslot()[r] = q;
+            atomicOr(&val[h], r << 1);
+        }
         if (old == -1 || old == q) return (int)h;
         h = (h + 1) & (RStage::kHash - 1);
     }
     return -1;
 }
 
-__device__ __forceinline__ int r_find(const int* key, int q)
-{
-    unsigned h = r_hash(q) & (RStage::kHash - 1);
-    for (int probe = 0; probe < RStage::kHash; probe++) {
-        const int k = key[h];
-        if (k == q) return (int)h;
-        if (k == -1) return -1;
-        h = (h + 1) & (RStage::kHash - 1);
-    }
-    return -1;
-}
-
-// Local index of global slot q: own particles first (q - b0), then the halo
-// (P + compact rank, kept in val >> 1).
-__device__ __forceinline__ int r_lid(const int* key, const int* val, int q, int b0, int b1, int P, int& fail)
+// Local index of global slot q: own particles first (q - b0), then the halo.
+__device__ __forceinline__ int r_lid(const int* key, const int* val, int q, int b0, int b1, int P)
 {
     if (q >= b0 && q < b1) return q - b0;
-    const int h = r_find(key, q);
-    if (h < 0) {
-        fail = 1;
-        return 0;
-    }
+    unsigned h = r_hash(q) & (RStage::kHash - 1);
+    for (int probe = 0; probe < RStage::kHash && key[h] != q; probe++) h = (h + 1) & (RStage::kHash - 1);
     return P + (val[h] >> 1);
 }
 
-// Counting sort, largest key first, of up to R items per thread (keys in
-// [0, 255], -1: no item); pos[r] gets item r's rank.  Equal keys keep the
-// order (thread, then round), so the result is the same on every run.
-template <int R>
-__device__ void r_sort_desc(const int (&key)[R], int (&pos)[R], int* hist)
+// Four entries of a row as local indices (padding: the row's own particle, in
+// the block or the halo like every partner).
+__device__ __forceinline__ void r_put_four(const Dev<float>& d, const int* key, const int* val, int b0, int b1, int P,
+                                           const int4& j, unsigned short* out, int n)
 {
-    const int t = threadIdx.x, B = blockDim.x;
-    for (int h = t; h < 256; h += B) hist[h] = 0;
-    __syncthreads();
+    const int q[4] = {j.x, j.y, j.z, j.w};
 #pragma unroll
-    for (int r = 0; r < R; r++)
-        if (key[r] >= 0) atomicAdd(&hist[key[r]], 1);
-    __syncthreads();
-    int base = 0;
-    for (int c = 255; c >= 0; c--) {
-        if (hist[c] == 0) continue;  // the same in every thread
-        int cl = 0;
+    for (int u = 0; u < 4; u++)
+        if (u < n) out[32 * u] = (unsigned short)r_lid(key, val, q[u], b0, b1, P);
+}
+
+// 256 counts -> the first rank of every key, keys in descending order (one warp).
+__device__ __forceinline__ void warp_desc_starts(int* hist)
+{
+    const int lane = threadIdx.x & 31;
+    int c[8], sum = 0;
 #pragma unroll
-        for (int r = 0; r < R; r++) cl += key[r] == c;
-        int tot;
-        int off = block_excl_scan(cl, s_int, &tot);
+    for (int i = 0; i < 8; i++) {
+        c[i] = hist[255 - 8 * lane - i];
+        sum += c[i];
+    }
+    int x = sum;
 #pragma unroll
-        for (int r = 0; r < R; r++)
-            if (key[r] == c) pos[r] = base + off++;
-        base += tot;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    x -= sum;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        hist[255 - 8 * lane - i] = x;
+        x += c[i];
     }
 }
 
-// Lays out warp blocks: rows by (thread, round r) with n[r] entries each (0: no
-// row); every warp block of 32 rows takes 32 x its
-// longest row, in order (round, warp).  Returns the total (entries), and in
-// first[r] the entry of row r's lane (entry k of the row at first + 32 k).
-template <int R>
-__device__ int r_warp_layout(const int (&n)[R], int (&first)[R], int* wl)
+// Adds the lanes with a key (-1: none) to counts[key], one atomic per key and
+// warp; the lane's place among them.
+__device__ __forceinline__ int warp_count(int key, int* counts)
 {
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const unsigned m = __match_any_sync(0xffffffffu, key);
+    const int leader = __ffs(m) - 1;
+    int base = 0;
+    if (key >= 0 && lane == leader) base = atomicAdd(&counts[key], __popc(m));
+    return __shfl_sync(0xffffffffu, base, leader) + __popc(m & ((1u << lane) - 1u));
+}
+
+// Lengths of n warp blocks (32 rows each) -> their first entries, in order; the
+// total goes behind them (one warp).
+__device__ __forceinline__ void warp_block_starts(int* wl, int n)
+{
+    const int lane = threadIdx.x & 31;
+    int base = 0;
+    for (int b = 0; b < n; b += 32) {
+        const int L = b + lane < n ? 32 * wl[b + lane] : 0;
+        int x = L;
 #pragma unroll
-    for (int r = 0; r < R; r++) {
-        const int L = __reduce_max_sync(0xffffffffu, n[r]);
-        if (lane == 0) wl[r * nw + warp] = L;
-    }
-    __syncthreads();
-    if (t == 0) {
-        int acc = 0;
-        for (int b = 0; b < R * nw; b++) {
-            const int L = wl[b];
-            wl[b] = acc;
-            acc += 32 * L;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
-        wl[R * nw] = acc;
+        if (b + lane < n) wl[b + lane] = base + x - L;
+        base += __shfl_sync(0xffffffffu, x, 31);
     }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < R; r++) first[r] = wl[r * nw + warp] + lane;
-    const int total = wl[R * nw];
-    __syncthreads();
-    return total;
+    if (lane == 0) wl[n] = base;
 }
 
 // Builds the block's resident structures from the global list and the
 // snapshots pos[pc].  Returns 1 when they fit (the same answer in every
-// thread of the block); 0 leaves nothing the step relies on.
+// thread of the block); 0 leaves nothing the step relies on.  Halo particles
+// and rows of S are numbered in the order in which threads find them: nothing
+// that is summed depends on it.  (With block-wide scans and sorts for the
+// numbering, one-thread layouts and one entry loaded at a time this took 26 us
+// at 4 particles per block and 50 us at 660, in every launch and after every list
+// build; now 11 and 28.)
 static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
 {
     typedef RStage RS;
     constexpr int RR = RS::kRounds;
     int4* lpos = RS::lpos();
     int* key = (int*)(g_dyn + RS::B_KEY);
-    int* val = (int*)(g_dyn + RS::B_VAL);  // bit 0: reactive partner of an own particle; then the rank << 1
-    int* hist = (int*)(g_dyn + RS::B_HIST);
-    int* wl = (int*)(g_dyn + RS::B_WL);
-    int* hr = (int*)RS::sent();   // table index of the k-th reactive first-shell particle
+    int* val = (int*)(g_dyn + RS::B_VAL);
+    int* hist = (int*)(g_dyn + RS::B_HIST);  // rows of S; reactive and other force rows
+    int* wl = (int*)(g_dyn + RS::B_WL);      // warp blocks of the rows of S; of the two kinds of force rows
+    int *wlr = wl + RR * 32 + 1, *wlo = wlr + 33;
+    int* hr = (int*)RS::sent();   // table place of the k-th reactive first-shell particle
     int* cen = (int*)RS::lS();    // centre (local index) of the row at each position
-    const int t = threadIdx.x, B = blockDim.x;
-    const int PER = (RS::kHash + B - 1) / B;
+    const int t = threadIdx.x, B = blockDim.x, lane = t & 31, warp = t >> 5, nw = B >> 5;
     int b0, b1;
     block_range(d, b0, b1);
     const int P = b1 - b0;
@@ -2402,55 +2410,53 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
         key[h] = -1;
         val[h] = 0;
     }
-    __syncthreads();
-    int fail = 0;
+    if (t == 0) s_nh = s_nhr = 0;
     int4 inf = make_int4(0, 0, 0, 0);
     if (t < P) inf = d.pinfo[b0 + t];
-    // 1. first shell: the partners of the own rows outside the block
-    for (int k = 0; k < inf.y + inf.w; k++) {
-        const bool react = k < inf.y;
-        const int q = d.ent_j[(unsigned)(react ? inf.x + k : inf.z + k - inf.y)];
-        if (q < b0 || q >= b1) {
-            const int h = r_insert(key, q);
-            if (h < 0) fail = 1;
-            else if (react) atomicOr(&val[h], 1);
+    __syncthreads();
+    int fail = inf.y > 255 || inf.w > 255;
+    // 1. first shell: the partners of the own rows outside the block (lanes that
+    // the particles leave share a row, four entries at a time)
+    {
+        int lg = 0;
+        while (lg < 5 && (P << (lg + 1)) <= B) lg++;
+        const int i = t >> lg, g = t & ((1 << lg) - 1);
+        if (i < P) {
+            const int4 f = d.pinfo[b0 + i];
+            const int cr = (f.y + 3) >> 2, cw = (f.w + 3) >> 2;
+            for (int c = g; c < cr + cw; c += 1 << lg) {
+                const bool react = c < cr;
+                const int4 j = load_four(d, react ? f.x : f.z, 4 * (react ? c : c - cr));
+                const int q[4] = {j.x, j.y, j.z, j.w};
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    if (q[u] >= b0 && q[u] < b1) continue;  // padding is the own slot
+                    const int h = r_insert(key, val, q[u], P);
+                    if (h < 0) fail = 1;
+                    else if (react && !(atomicOr(&val[h], 1) & 1)) hr[atomicAdd(&s_nhr, 1)] = h;
+                }
+            }
         }
     }
     if (__syncthreads_or(fail)) return 0;
-    // 2. its reactive part (their S is formed here too), in table order
-    const int h0 = min(t * PER, RS::kHash), h1 = min(h0 + PER, RS::kHash);
-    int c = 0;
-    for (int h = h0; h < h1; h++) c += val[h] & 1;
-    int Hr;
-    int off = block_excl_scan(c, s_int, &Hr);
-    if (P + Hr > RS::kL) return 0;  // Hr is the same in every thread
-    for (int h = h0; h < h1; h++)
-        if (val[h] & 1) hr[off++] = h;
-    __syncthreads();
-    // 3. second shell: the reactive partners of the reactive first shell
-    for (int k = t; k < Hr; k += B) {
-        const int4 fi = d.pinfo[key[hr[k]]];
-        for (int m = 0; m < fi.y; m++) {
-            const int q = d.ent_j[(unsigned)(fi.x + m)];
-            if ((q < b0 || q >= b1) && r_insert(key, q) < 0) fail = 1;
+    // 2. second shell: the reactive partners of the reactive first shell (whose S
+    // is formed here too)
+    const int Hr = s_nhr;
+    {
+        int lg = 0;
+        while (lg < 3 && (Hr << (lg + 1)) <= B) lg++;
+        for (int k = t >> lg; k < Hr; k += B >> lg) {
+            const int4 f = d.pinfo[key[hr[k]]];
+            for (int c = t & ((1 << lg) - 1); c < (f.y + 3) >> 2; c += 1 << lg) {
+                const int4 j = load_four(d, f.x, 4 * c);
+                const int q[4] = {j.x, j.y, j.z, j.w};
+#pragma unroll
+                for (int u = 0; u < 4; u++)
+                    if ((q[u] < b0 || q[u] >= b1) && r_insert(key, val, q[u], P) < 0) fail = 1;
+            }
         }
     }
-    if (__syncthreads_or(fail)) return 0;
-    // 4. compact the table: halo particle of rank r has local index P + r
-    c = 0;
-    for (int h = h0; h < h1; h++) c += key[h] != -1;
-    int H;
-    off = block_excl_scan(c, s_int, &H);
-    if (P + H > RS::kL) return 0;
-    for (int h = h0; h < h1; h++) {
-        if (key[h] != -1) {
-            RS::hslot()[off] = key[h];
-            val[h] = (val[h] & 1) | (off << 1);
-            off++;
-        }
-    }
-    __syncthreads();
-    // 5. rows of S (the own rows and the reactive first shell's), longest
+    // 3. rows of S (the own rows and the reactive first shell's), longest
     // first, dealt out over the RB row threads as a snake: rank s goes to round
     // s / RB, to thread s % RB in even rounds and RB - 1 - s % RB in odd ones, so
     // that a thread's second row is short when its first is long.  The force
@@ -2459,51 +2465,78 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
     // from warp 0, other rows longest first from the last warp, so that the
     // rows of a warp are alike in each loop and the warps' totals even out.
     const int NS = P + Hr;
-    // the rows leave the last warp free for the slots (r_run) where they can
+    if (NS > RS::kL) return 0;  // the same in every thread
+    // the rows leave the last warp free for the agreement (r_run) where they can
     const int RB = P <= B - 32 && NS <= RR * (B - 32) ? B - 32 : B;
-    const int rounds = (NS + RB - 1) / RB;
-    if (inf.y > 255 || inf.w > 255) fail = 1;
-    int skey[RR + 1], spos[RR + 1], hrow[RR], hcnt[RR];
+    const int rounds = (NS + RB - 1) / RB, W32 = (P + 31) & ~31;
+    int skey[RR + 1], hrow[RR];
     skey[0] = t < P ? min(inf.y, 255) : -1;
-    spos[0] = 0;
 #pragma unroll
     for (int r = 0; r < RR; r++) {
         const int k = t + r * B;
         skey[r + 1] = -1;
-        spos[r + 1] = 0;
-        hrow[r] = hcnt[r] = 0;
+        hrow[r] = 0;
         if (k < Hr) {
-            const int4 fi = d.pinfo[key[hr[k]]];
-            hrow[r] = fi.x;
-            hcnt[r] = fi.y;
-            if (fi.y > 255) fail = 1;
-            skey[r + 1] = min(fi.y, 255);
+            const int4 f = d.pinfo[key[hr[k]]];
+            hrow[r] = f.x;
+            if (f.y > 255) fail = 1;
+            skey[r + 1] = min(f.y, 255);
         }
     }
-    r_sort_desc<RR + 1>(skey, spos, hist);
-    const int W32 = (P + 31) & ~31;
-    const int rpos = rank_desc(t < P ? inf.y : -1, RS::fent(), hist, s_int);
-    const int wrank = rank_desc(t < P ? inf.w : -1, RS::fent(), hist, s_int);
-    const int wpos = W32 - 32 - (wrank & ~31) + (wrank & 31);  // rank chunk c -> warp W32/32 - 1 - c
+    // force rows are ranked in particle order among equal lengths (their threads
+    // sum the thermo terms): counts per warp and key, reactive then other
+    unsigned short* wh = RS::fent();
+    for (int k = t; k < nw * 256; k += B) ((int*)wh)[k] = 0;
+    for (int k = t; k < 3 * 256; k += B) hist[k] = 0;
     for (int q = t; q < rounds * RB; q += B) RS::sdesc()[q] = make_int2(0, -1);  // no row here
-    if (t < W32) RS::fdesc()[t] = make_int4(0, 0, 0, -1);  // no rows; centres 0xffff
+    if (t < W32) RS::fdesc()[t] = make_int4(0, 0, 0, -1);                        // no rows; centres 0xffff
+    if (__syncthreads_or(fail)) return 0;
+    const int H = s_nh;
+    const int krow = t < P ? inf.y : -1, kother = t < P ? inf.w : -1;
+    const unsigned mr = __match_any_sync(0xffffffffu, krow), mo = __match_any_sync(0xffffffffu, kother);
+    const int br = __popc(mr & ((1u << lane) - 1u)), bo = __popc(mo & ((1u << lane) - 1u));
+    if (t < P && br == 0) wh[warp * 512 + krow] = (unsigned short)__popc(mr);
+    if (t < P && bo == 0) wh[warp * 512 + 256 + kother] = (unsigned short)__popc(mo);
+#pragma unroll
+    for (int r = 0; r <= RR; r++)
+        if (r == 0 || (r - 1) * B < Hr) warp_count(skey[r], hist);
+    __syncthreads();
+    if (t >= 256) {
+        // per key: the counts of the warps before each warp, and the key's total
+        const int k = t - 256;  // 512 threads: the two kinds
+        int run = 0;
+        for (int w = 0; w < nw; w++) {
+            const int c = wh[w * 512 + k];
+            wh[w * 512 + k] = (unsigned short)run;
+            run += c;
+        }
+        hist[t] = run;
+    } else if (warp == 0) {
+        warp_desc_starts(hist);
+    }
+    __syncthreads();
+    if (warp < 2) warp_desc_starts(hist + 256 * (warp + 1));
     __syncthreads();
     // what each position needs: the centre and the row (start, count)
 #pragma unroll
     for (int r = 0; r <= RR; r++) {
+        if (r > 0 && (r - 1) * B >= Hr) continue;
+        const int sr = warp_count(skey[r], hist);
         if (skey[r] < 0) continue;
-        const int sr = spos[r], g = sr / RB, slot = sr - g * RB;
+        const int g = sr / RB, slot = sr - g * RB;
         const int q = g * RB + ((g & 1) ? RB - 1 - slot : slot);
         if (r == 0) {
             cen[q] = t;
             RS::sdesc()[q] = make_int2(inf.x, inf.y);
         } else {
-            const int k = t + (r - 1) * B;
-            cen[q] = P + (val[hr[k]] >> 1);
-            RS::sdesc()[q] = make_int2(hrow[r - 1], hcnt[r - 1]);
+            cen[q] = P + (val[hr[t + (r - 1) * B]] >> 1);
+            RS::sdesc()[q] = make_int2(hrow[r - 1], skey[r]);
         }
     }
     if (t < P) {
+        const int rpos = hist[256 + krow] + wh[warp * 512 + krow] + br;
+        const int wrank = hist[512 + kother] + wh[warp * 512 + 256 + kother] + bo;
+        const int wpos = W32 - 32 - (wrank & ~31) + (wrank & 31);  // rank chunk c -> warp W32/32 - 1 - c
         // 16-bit fields: (z, w) = (nr, nw, reactive centre, other centre)
         int4* fr = &RS::fdesc()[rpos];
         int4* fo = &RS::fdesc()[wpos];
@@ -2514,43 +2547,46 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
         ((unsigned short*)&fr->w)[0] = (unsigned short)t;
         ((unsigned short*)&fo->w)[1] = (unsigned short)t;
     }
-    if (__syncthreads_or(fail)) return 0;
-    // 6. warp-major layouts: the rows of S; the own rows' reactive parts, then
-    // their other parts
-    int n[RR], first[RR];
+    __syncthreads();
+    // 4. warp-major layouts: every warp block of 32 rows takes 32 x its longest
+    // row; the rows of S in order (round, warp); the own rows' reactive parts,
+    // then their other parts
+    int2 src[RR];
 #pragma unroll
     for (int r = 0; r < RR; r++) {
-        const int q = t + r * RB;
-        n[r] = r < rounds && t < RB ? max(RS::sdesc()[q].y, 0) : 0;
+        src[r] = r < rounds && t < RB ? RS::sdesc()[t + r * RB] : make_int2(0, -1);
+        const int L = __reduce_max_sync(0xffffffffu, max(src[r].y, 0));
+        if (lane == 0) wl[r * nw + warp] = L;
     }
-    const int ES = r_warp_layout<RR>(n, first, wl);
     const int4 fd = t < W32 ? RS::fdesc()[t] : make_int4(0, 0, 0, -1);
-    int nrc[1] = {fd.z & 0xffff}, nwc[1] = {(int)((unsigned)fd.z >> 16)}, rfirst[1], wfirst[1];
-    const int ER = r_warp_layout<1>(nrc, rfirst, wl);
-    const int EW = r_warp_layout<1>(nwc, wfirst, wl);
-    if (ES > RS::kES || ER + EW > RS::kEF) return 0;  // the same in every thread
-    // 7. the rows, partners as local indices
+    const int nrc = fd.z & 0xffff, nwc = (int)((unsigned)fd.z >> 16);
+    const int Lr = __reduce_max_sync(0xffffffffu, nrc), Lo = __reduce_max_sync(0xffffffffu, nwc);
+    if (lane == 0) {
+        wlr[warp] = Lr;
+        wlo[warp] = Lo;
+    }
+    __syncthreads();
+    if (warp == 0) warp_block_starts(wl, RR * nw);
+    else if (warp < 3) warp_block_starts(warp == 1 ? wlr : wlo, nw);
+    __syncthreads();
+    const int ER = wlr[nw];
+    if (wl[RR * nw] > RS::kES || ER + wlo[nw] > RS::kEF) return 0;  // the same in every thread
+    // 5. the rows, partners as local indices
 #pragma unroll
     for (int r = 0; r < RR; r++) {
-        const int q = t + r * RB;
-        if (r < rounds && t < RB) {
-            const int2 src = RS::sdesc()[q];
-            if (src.y >= 0) {
-                const int lid = cen[q];
-                for (int m = 0; m < src.y; m++)
-                    RS::sent()[first[r] + 32 * m] =
-                        (unsigned short)r_lid(key, val, d.ent_j[(unsigned)(src.x + m)], b0, b1, P, fail);
-                RS::sdesc()[q] = make_int2(first[r], lid | (src.y << 16));
-            }
-        }
+        if (r >= rounds || src[r].y < 0) continue;
+        const int q = t + r * RB, first = wl[r * nw + warp] + lane, n = src[r].y;
+        for (int m = 0; m < n; m += 4)
+            r_put_four(d, key, val, b0, b1, P, load_four(d, src[r].x, m), RS::sent() + first + 32 * m, n - m);
+        RS::sdesc()[q] = make_int2(first, cen[q] | (n << 16));
     }
     if (t < W32) {
-        unsigned short* fe = RS::fent();
-        for (int m = 0; m < nrc[0]; m++)
-            fe[rfirst[0] + 32 * m] = (unsigned short)r_lid(key, val, d.ent_j[(unsigned)(fd.x + m)], b0, b1, P, fail);
-        for (int m = 0; m < nwc[0]; m++)
-            fe[ER + wfirst[0] + 32 * m] = (unsigned short)r_lid(key, val, d.ent_j[(unsigned)(fd.y + m)], b0, b1, P, fail);
-        RS::fdesc()[t] = make_int4(rfirst[0], ER + wfirst[0], fd.z, fd.w);
+        const int first_r = wlr[warp] + lane, first_o = ER + wlo[warp] + lane;
+        for (int m = 0; m < nrc; m += 4)
+            r_put_four(d, key, val, b0, b1, P, load_four(d, fd.x, m), RS::fent() + first_r + 32 * m, nrc - m);
+        for (int m = 0; m < nwc; m += 4)
+            r_put_four(d, key, val, b0, b1, P, load_four(d, fd.y, m), RS::fent() + first_o + 32 * m, nwc - m);
+        RS::fdesc()[t] = make_int4(first_r, first_o, fd.z, fd.w);
     }
     if (t < P) {
         const int4 own = d.pos[pc][b0 + t];
@@ -2563,10 +2599,10 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
         s_ls.r_nh = H;
         s_ls.r_nhr = Hr;
     }
-    const int ok = __syncthreads_or(fail) ? 0 : 1;
-    // 8. the own particles' state by reactive-row position (over the table, now unused)
-    if (ok && t < P) {
-        const int i = b0 + (RS::fdesc()[t].w & 0xffff), n = d.n;
+    __syncthreads();
+    // 6. the own particles' state by reactive-row position (over the table, now unused)
+    if (t < P) {
+        const int i = b0 + (fd.w & 0xffff), n = d.n;
         RS::vel()[t] = d.vel[ac][i];
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -2575,7 +2611,7 @@ static __device__ int r_localize(const Dev<float>& d, int pc, int ac)
         }
     }
     __syncthreads();
-    return ok;
+    return 1;
 }
 
 // Writes the own particles' state back to the global arrays (snapshots to set
