@@ -96,6 +96,8 @@ struct swp_ctx {
     Dev<float> df;
     Dev<double> dd;
     Ctl hctl;
+    Ctl* mirror = nullptr;  // pinned: every launch is followed by a copy of the control block into it
+    bool pending = false;   // a launch since the last wait writes to the mirror
     std::vector<int> cell_rank;
     std::vector<unsigned char> table_host;
     std::string err;
@@ -290,6 +292,7 @@ size_t layout(swp_ctx* c, char* base, Dev<Real>* d)
         d->partials = partials;
         d->ctl = ctl;
         d->agree = ctl ? ctl->agree : nullptr;
+        d->mirror = c->mirror;
         d->io = io;
         d->io_int = io_int;
         d->table = table;
@@ -405,6 +408,8 @@ int ready(swp_ctx* c, bool need_state)
     return SWP_OK;
 }
 
+int mirror_ctl(swp_ctx* c);
+
 int map_status(swp_ctx* c)
 {
     int s = c->hctl.status;
@@ -421,11 +426,24 @@ int map_status(swp_ctx* c)
         k_clear_status_bits<<<1, 1, 0, c->stream>>>(dev_ctl(c), kStatusOverflow);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(c, e, "clear status");
+        const int rc = mirror_ctl(c);
+        if (rc) return rc;
         char buf[160];
         std::snprintf(buf, sizeof buf, "neighbour row of %d entries exceeds max_nn = %d",
                       c->hctl.max_row, c->max_nn);
         return fail(c, SWP_ERR_NLIST_OVERFLOW, buf);
     }
+    return SWP_OK;
+}
+
+// Enqueues the copy of the control block into the pinned mirror; every call that
+// changes the block ends with it, so that a synchronising call only has to wait
+// (also for replays of captured work: the copy is captured with it).
+int mirror_ctl(swp_ctx* c)
+{
+    if (!c->mirror) return SWP_OK;
+    c->pending = true;
+    SWP_CUDA(c, cudaMemcpyAsync(c->mirror, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
     return SWP_OK;
 }
 
@@ -436,8 +454,11 @@ int sync_ctl(swp_ctx* c)
         SWP_CUDA(c, cudaStreamSynchronize(c->stream));
         return SWP_OK;
     }
-    SWP_CUDA(c, cudaMemcpyAsync(&c->hctl, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
+    if (!c->mirror)
+        SWP_CUDA(c, cudaMemcpyAsync(&c->hctl, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
+    if (c->mirror) c->hctl = *c->mirror;
+    c->pending = false;
     return map_status(c);
 }
 
@@ -559,7 +580,7 @@ int run(swp_ctx* c, RunArgs a)
     SWP_CUDA(c, cudaMemsetAsync(d.ctl, 0, offsetof(Ctl, barrier) + sizeof(unsigned long long), c->stream));
     if (wide) SWP_CUDA(c, launch_run_wide<Real>(d, a, c->grid, c->stream));
     else SWP_CUDA(c, launch_run<Real>(d, a, c->grid, block, c->stream));
-    return SWP_OK;
+    return mirror_ctl(c);
 }
 
 int run_any(swp_ctx* c, RunArgs a)
@@ -572,8 +593,10 @@ int mark_stale(swp_ctx* c)
     if (!c->ws_bound || !c->state_set || c->n == 0) return SWP_OK;
     k_mark_stale<<<1, 1, 0, c->stream>>>(dev_ctl(c));
     SWP_CUDA(c, cudaGetLastError());
-    return SWP_OK;
+    return mirror_ctl(c);
 }
+
+bool aligned(const void* p, size_t a) { return ((uintptr_t)p & (a - 1)) == 0; }
 
 cudaMemcpyKind kind_to_dev(int where)
 {
@@ -824,7 +847,6 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
         uni &= args[r].uni;
         devs[r] = dev<Real>(c);
         bonds |= devs[r].has_bonds;
-        SWP_CUDA(c0, cudaMemsetAsync(&devs[r].ctl->barrier, 0, sizeof(unsigned long long), c0->stream));
     }
     for (int k = 0; k < B; k++)
         for (int it = plan.item_ofs[k]; it < plan.item_ofs[k + 1]; it++)
@@ -841,7 +863,10 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
                                  c0->stream));
     SWP_CUDA(c0, cudaMemcpyAsync(d_items, plan.items.data(), sizeof(int4) * plan.items.size(),
                                  cudaMemcpyHostToDevice, c0->stream));
+    SWP_CUDA(c0, launch_batch_begin<Real>(d_dev, m, c0->stream));
     SWP_CUDA(c0, launch_batch_shape<Real>(threads, d_dev, d_args, d_ofs, d_items, uni, bonds, B, c0->stream));
+    for (int r = 0; r < m; r++) cs[idx[r]]->pending = true;
+    SWP_CUDA(c0, launch_batch_end<Real>(d_dev, m, c0->stream));
     return SWP_OK;
 }
 
@@ -1026,6 +1051,10 @@ int swp_bind_workspace(swp_ctx* c, void* ptr, size_t bytes, void* stream)
     c->ws_bound = true;
     c->state_set = false;
     c->table_dirty = true;
+    if (!c->mirror && cudaHostAlloc((void**)&c->mirror, sizeof(Ctl), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();  // (during stream capture, say): synchronising calls copy the block themselves
+        c->mirror = nullptr;
+    }
     refresh_layout(c);
     SWP_CUDA(c, cudaMemcpyAsync((void*)(c->precision == SWP_FP64 ? c->dd.cell_rank : c->df.cell_rank),
                                 c->cell_rank.data(), sizeof(int) * 2 * c->ncell, cudaMemcpyHostToDevice,
@@ -1068,46 +1097,32 @@ int swp_set_state(swp_ctx* c, const double* x, const double* v, const int32_t* t
     }
     rc = upload_table(c);
     if (rc) return rc;
-    double* io;
-    int* io_int;
-    Ctl* ctl;
-    if (c->precision == SWP_FP64) {
-        io = c->dd.io;
-        io_int = c->dd.io_int;
-        ctl = c->dd.ctl;
-    } else {
-        io = c->df.io;
-        io_int = c->df.io_int;
-        ctl = c->df.ctl;
-    }
     std::memset(&c->hctl, 0, sizeof(Ctl));
     c->hctl.state = 1;
     c->hctl.need_rebuild = 1;
-    SWP_CUDA(c, cudaMemcpyAsync(ctl, &c->hctl, sizeof(Ctl), cudaMemcpyHostToDevice, c->stream));
-    // the cell build expects zeroed counts (it zeroes them itself after use)
-    SWP_CUDA(c, cudaMemsetAsync(c->precision == SWP_FP64 ? (void*)c->dd.cell_cnt : (void*)c->df.cell_cnt, 0,
-                                sizeof(int) * c->ncell, c->stream));
-    if (n == 0) {
-        c->state_set = true;
-        return SWP_OK;
-    }
-    SWP_CUDA(c, cudaMemcpyAsync(io, x, sizeof(double) * 3 * n, kind_to_dev(where), c->stream));
-    if (v) SWP_CUDA(c, cudaMemcpyAsync(io + 3 * n, v, sizeof(double) * 3 * n, kind_to_dev(where), c->stream));
-    else SWP_CUDA(c, cudaMemsetAsync(io + 3 * n, 0, sizeof(double) * 3 * n, c->stream));
-    if (mass) SWP_CUDA(c, cudaMemcpyAsync(io + 6 * n, mass, sizeof(double) * n, kind_to_dev(where), c->stream));
-    else {
-        std::vector<double> ones(n, 1.0);
-        SWP_CUDA(c, cudaMemcpyAsync(io + 6 * n, ones.data(), sizeof(double) * n, cudaMemcpyHostToDevice, c->stream));
-        SWP_CUDA(c, cudaStreamSynchronize(c->stream));
-    }
-    if (type) SWP_CUDA(c, cudaMemcpyAsync(io_int, type, sizeof(int) * n, kind_to_dev(where), c->stream));
-    else SWP_CUDA(c, cudaMemsetAsync(io_int, 0, sizeof(int) * n, c->stream));
-    if (img) SWP_CUDA(c, cudaMemcpyAsync(io_int + n, img, sizeof(int) * 3 * n, kind_to_dev(where), c->stream));
-    else SWP_CUDA(c, cudaMemsetAsync(io_int + n, 0, sizeof(int) * 3 * n, c->stream));
-    if (c->precision == SWP_FP64) SWP_CUDA(c, launch_set_state<double>(c->dd, c->stream));
-    else SWP_CUDA(c, launch_set_state<float>(c->df, c->stream));
+    SWP_CUDA(c, cudaMemsetAsync(dev_ctl(c), 0, sizeof(Ctl), c->stream));
     c->state_set = true;
-    return SWP_OK;
+    if (n == 0) return SWP_OK;
+    // aligned device arrays are read where they are; others through the staging area
+    const int32_t *ty = type, *im = img;
+    if (where == SWP_HOST || !aligned(x, 8) || !aligned(v, 8) || !aligned(mass, 8) || !aligned(type, 4) || !aligned(img, 4)) {
+        double* io = c->precision == SWP_FP64 ? c->dd.io : c->df.io;
+        int* io_int = c->precision == SWP_FP64 ? c->dd.io_int : c->df.io_int;
+        auto stage = [&](auto* dst, auto*& src, size_t count) {
+            if (!src) return cudaSuccess;
+            const cudaError_t e = cudaMemcpyAsync(dst, src, sizeof(*dst) * count, kind_to_dev(where), c->stream);
+            src = dst;
+            return e;
+        };
+        SWP_CUDA(c, stage(io, x, 3 * n));
+        SWP_CUDA(c, stage(io + 3 * n, v, 3 * n));
+        SWP_CUDA(c, stage(io + 6 * n, mass, n));
+        SWP_CUDA(c, stage(io_int, ty, n));
+        SWP_CUDA(c, stage(io_int + n, im, 3 * n));
+    }
+    if (c->precision == SWP_FP64) SWP_CUDA(c, launch_set_state<double>(c->dd, x, v, ty, mass, im, c->stream));
+    else SWP_CUDA(c, launch_set_state<float>(c->df, x, v, ty, mass, im, c->stream));
+    return mirror_ctl(c);
 }
 
 int swp_set_step(swp_ctx* c, int64_t step)
@@ -1119,8 +1134,9 @@ int swp_set_step(swp_ctx* c, int64_t step)
     static_assert(sizeof(long long) == sizeof(int64_t), "step width");
     long long s = (long long)step;
     SWP_CUDA(c, cudaMemcpyAsync(&dev_ctl(c)->step, &s, sizeof(s), cudaMemcpyHostToDevice, c->stream));
+    const int rm = mirror_ctl(c);
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
-    return SWP_OK;
+    return rm;
 }
 
 int swp_build_nlist(swp_ctx* c)
@@ -1286,15 +1302,10 @@ int swp_read_forces(swp_ctx* c, double* f, int where)
     rc = sync_ctl(c);
     if (rc) return rc;
     if (c->hctl.state != 0) return fail(c, SWP_ERR_STATE, "forces are not current: call swp_compute_forces");
-    double* io;
-    if (c->precision == SWP_FP64) {
-        SWP_CUDA(c, launch_get_forces<double>(c->dd, c->hctl.pos_cur, c->stream));
-        io = c->dd.io;
-    } else {
-        SWP_CUDA(c, launch_get_forces<float>(c->df, c->hctl.pos_cur, c->stream));
-        io = c->df.io;
-    }
-    SWP_CUDA(c, cudaMemcpyAsync(f, io, sizeof(double) * 3 * c->n, kind_from_dev(where), c->stream));
+    double* out = where == SWP_DEVICE && aligned(f, 8) ? f : c->precision == SWP_FP64 ? c->dd.io : c->df.io;
+    if (c->precision == SWP_FP64) SWP_CUDA(c, launch_get_forces<double>(c->dd, c->hctl.pos_cur, out, nullptr, c->stream));
+    else SWP_CUDA(c, launch_get_forces<float>(c->df, c->hctl.pos_cur, out, nullptr, c->stream));
+    if (out != f) SWP_CUDA(c, cudaMemcpyAsync(f, out, sizeof(double) * 3 * c->n, kind_from_dev(where), c->stream));
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
     return SWP_OK;
 }
@@ -1357,11 +1368,8 @@ int swp_eval_grad(swp_ctx* c, int ti, int tj, const double* theta_dev, const dou
     const double c_rmin = std::pow(2.0, 1.0 / p.n), c_rb = std::pow((1.0 - std::sqrt(0.5)) / 2.0, -1.0 / p.n);
     const bool f64 = c->precision == SWP_FP64;
     double* io = f64 ? c->dd.io : c->df.io;
-    SWP_CUDA(c, cudaMemsetAsync(f64 ? (void*)c->dd.cell_cnt : (void*)c->df.cell_cnt, 0, sizeof(int) * c->ncell,
-                                c->stream));
-    if (n > 0) SWP_CUDA(c, cudaMemcpyAsync(io, x_dev, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, c->stream));
-    if (f64) SWP_CUDA(c, launch_eval_prep<double>(c->dd, ti, tj, theta_dev, c_rmin, c_rb, p.rbond, type_dev, c->stream));
-    else SWP_CUDA(c, launch_eval_prep<float>(c->df, ti, tj, theta_dev, c_rmin, c_rb, p.rbond, type_dev, c->stream));
+    if (f64) SWP_CUDA(c, launch_eval_prep<double>(c->dd, ti, tj, theta_dev, c_rmin, c_rb, p.rbond, c->stream));
+    else SWP_CUDA(c, launch_eval_prep<float>(c->df, ti, tj, theta_dev, c_rmin, c_rb, p.rbond, c->stream));
     c->state_set = true;
     c->table_theta = true;
     if (n == 0) {
@@ -1369,8 +1377,12 @@ int swp_eval_grad(swp_ctx* c, int ti, int tj, const double* theta_dev, const dou
         if (dU_dev) SWP_CUDA(c, cudaMemsetAsync(dU_dev, 0, 3 * sizeof(double), c->stream));
         return SWP_OK;
     }
-    if (f64) SWP_CUDA(c, launch_set_state<double>(c->dd, c->stream));
-    else SWP_CUDA(c, launch_set_state<float>(c->df, c->stream));
+    if (!aligned(x_dev, 8)) {
+        SWP_CUDA(c, cudaMemcpyAsync(io, x_dev, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, c->stream));
+        x_dev = io;
+    }
+    if (f64) SWP_CUDA(c, launch_set_state<double>(c->dd, x_dev, nullptr, type_dev, nullptr, nullptr, c->stream));
+    else SWP_CUDA(c, launch_set_state<float>(c->df, x_dev, nullptr, type_dev, nullptr, nullptr, c->stream));
     // forces at the new positions: rebuild and evaluate, coefficients from the device table
     RunArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -1380,12 +1392,15 @@ int swp_eval_grad(swp_ctx* c, int ti, int tj, const double* theta_dev, const dou
     rc = run_any(c, a);
     c->table_only = 0;
     if (rc) return rc;
-    k_eval_energy<<<1, 1, 0, c->stream>>>(dev_ctl(c), U_dev);
-    SWP_CUDA(c, cudaGetLastError());
     if (F_dev) {
-        if (f64) SWP_CUDA(c, launch_get_forces<double>(c->dd, -1, c->stream));
-        else SWP_CUDA(c, launch_get_forces<float>(c->df, -1, c->stream));
-        SWP_CUDA(c, cudaMemcpyAsync(F_dev, io, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, c->stream));
+        double* out = aligned(F_dev, 8) ? F_dev : io;
+        if (f64) SWP_CUDA(c, launch_get_forces<double>(c->dd, -1, out, U_dev, c->stream));
+        else SWP_CUDA(c, launch_get_forces<float>(c->df, -1, out, U_dev, c->stream));
+        if (out != F_dev)
+            SWP_CUDA(c, cudaMemcpyAsync(F_dev, io, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, c->stream));
+    } else {
+        k_eval_energy<<<1, 1, 0, c->stream>>>(dev_ctl(c), U_dev);
+        SWP_CUDA(c, cudaGetLastError());
     }
     if (dU_dev || dF_dev) {
         double* part = f64 ? c->dd.partials : c->df.partials;
@@ -1405,20 +1420,19 @@ int swp_read_state(swp_ctx* c, double* x, double* v, int32_t* img, int where)
     rc = sync_ctl(c);
     if (rc && rc != SWP_ERR_NLIST_OVERFLOW) return rc;
     const size_t n = (size_t)c->n;
-    double* io;
-    int* io_int;
-    if (c->precision == SWP_FP64) {
-        SWP_CUDA(c, launch_get_state<double>(c->dd, c->hctl.pos_cur, c->hctl.arr_cur, c->stream));
-        io = c->dd.io;
-        io_int = c->dd.io_int;
-    } else {
-        SWP_CUDA(c, launch_get_state<float>(c->df, c->hctl.pos_cur, c->hctl.arr_cur, c->stream));
-        io = c->df.io;
-        io_int = c->df.io_int;
+    // straight into aligned device arrays; into others through the staging area
+    const bool dev = where == SWP_DEVICE && aligned(x, 8) && aligned(v, 8) && aligned(img, 4), f64 = c->precision == SWP_FP64;
+    double* io = f64 ? c->dd.io : c->df.io;
+    double *xo = !x || dev ? x : io, *vo = !v || dev ? v : io + 3 * n;
+    int* io_int = f64 ? c->dd.io_int : c->df.io_int;
+    int* mo = !img || dev ? img : io_int;
+    if (f64) SWP_CUDA(c, launch_get_state<double>(c->dd, c->hctl.pos_cur, c->hctl.arr_cur, xo, vo, mo, c->stream));
+    else SWP_CUDA(c, launch_get_state<float>(c->df, c->hctl.pos_cur, c->hctl.arr_cur, xo, vo, mo, c->stream));
+    if (!dev) {
+        if (x) SWP_CUDA(c, cudaMemcpyAsync(x, xo, sizeof(double) * 3 * n, kind_from_dev(where), c->stream));
+        if (v) SWP_CUDA(c, cudaMemcpyAsync(v, vo, sizeof(double) * 3 * n, kind_from_dev(where), c->stream));
+        if (img) SWP_CUDA(c, cudaMemcpyAsync(img, mo, sizeof(int) * 3 * n, kind_from_dev(where), c->stream));
     }
-    if (x) SWP_CUDA(c, cudaMemcpyAsync(x, io, sizeof(double) * 3 * n, kind_from_dev(where), c->stream));
-    if (v) SWP_CUDA(c, cudaMemcpyAsync(v, io + 3 * n, sizeof(double) * 3 * n, kind_from_dev(where), c->stream));
-    if (img) SWP_CUDA(c, cudaMemcpyAsync(img, io_int + n, sizeof(int) * 3 * n, kind_from_dev(where), c->stream));
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
     return rc;
 }
@@ -1500,6 +1514,8 @@ int swp_set_thermo_log(swp_ctx* c, int every, int64_t capacity, void* ring, size
     c->tlog_every = every;
     if (c->ws_bound) {
         SWP_CUDA(c, cudaMemsetAsync(&dev_ctl(c)->tlog_n, 0, sizeof(long long), c->stream));
+        const int rm = mirror_ctl(c);
+        if (rm) return rm;
     }
     return SWP_OK;
 }
@@ -1537,6 +1553,18 @@ const char* swp_last_error(const swp_ctx* c) { return c ? c->err.c_str() : "null
 
 int swp_destroy(swp_ctx* c)
 {
+    if (c && c->mirror) {
+        // launches that nobody waited for may still write to it (the stream
+        // itself may be gone by now)
+        int dev = -1;
+        if (c->pending && cudaGetDevice(&dev) == cudaSuccess) {
+            if (dev != c->device) cudaSetDevice(c->device);
+            cudaDeviceSynchronize();
+            if (dev != c->device) cudaSetDevice(dev);
+        }
+        cudaFreeHost(c->mirror);
+        cudaGetLastError();  // (the process may be ending)
+    }
     delete c;
     return SWP_OK;
 }
@@ -1570,19 +1598,6 @@ static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBy
 // Device address of g_static_scratch per device (host code sees only a
 // stand-in symbol; the address comes from cudaGetSymbolAddress).
 static void* g_static_addr[kMaxStaticDevices];
-
-__global__ void k_static_stage(const double* x, const int32_t* type, double* io, int* io_int, int n)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        for (int c = 0; c < 3; c++) {
-            io[3 * i + c] = x[3 * i + c];
-            io[3 * n + 3 * i + c] = 0.0;  // velocities
-            io_int[n + 3 * i + c] = 0;    // images
-        }
-        io[6 * n + i] = 1.0;  // masses
-        io_int[i] = type ? type[i] : 0;
-    }
-}
 
 template <typename Real>
 int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, double* thermo,
@@ -1627,10 +1642,7 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
     h.state = 1;
     h.need_rebuild = 1;
     SWP_CUDA(c, cudaMemcpyAsync(d.ctl, &h, sizeof(h), cudaMemcpyHostToDevice, s));
-    SWP_CUDA(c, cudaMemsetAsync(d.cell_cnt, 0, sizeof(int) * c->ncell, s));
-    k_static_stage<<<(c->n + 255) / 256, 256, 0, s>>>(x, type, d.io, d.io_int, c->n);
-    SWP_CUDA(c, cudaGetLastError());
-    SWP_CUDA(c, launch_set_state<Real>(d, s));
+    SWP_CUDA(c, launch_set_state<Real>(d, x, nullptr, type, nullptr, nullptr, s));
 
     int bps = 0;
     const int block = sizeof(Real) == 4 ? kBlock : kBlock64;
@@ -1656,8 +1668,7 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
                       c->max_nn);
         return fail(c, SWP_ERR_NLIST_OVERFLOW, buf);
     }
-    SWP_CUDA(c, launch_get_forces<Real>(d, h.pos_cur, s));
-    SWP_CUDA(c, cudaMemcpyAsync(f, d.io, sizeof(double) * 3 * c->n, cudaMemcpyDeviceToDevice, s));
+    SWP_CUDA(c, launch_get_forces<Real>(d, h.pos_cur, f, nullptr, s));
     if (thermo) {
         // [U2, U3, W xx yy zz xy xz yz, n_bonds]
         SWP_CUDA(c, cudaMemcpyAsync(thermo, &d.ctl->thermo[Q_U2], 2 * sizeof(double),

@@ -155,6 +155,7 @@ struct Dev {
     double* partials;  // [max_blocks][kNQ]
     Ctl* ctl;
     unsigned long long* agree;  // resident steps: ctl->agree
+    Ctl* mirror;     // pinned host memory: the control block after the last launch (null: none)
     double* io;        // host-exchange staging: [3n] x, [3n] v, [n] mass
     int* io_int;       // staging: [n] types, [3n] images
     const PairP<Real>* table;  // [ntypes * ntypes]
@@ -237,13 +238,18 @@ cudaError_t launch_param_grad(const Dev<Real>& d, int pc, double* sd, double* pa
                               double* out, double* total, double* dU, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_eval_prep(const Dev<Real>& d, int ti, int tj, const double* theta, double c_rmin, double c_rb,
-                             double rbond, const int* type, cudaStream_t s);
+                             double rbond, cudaStream_t s);
 template <typename Real>
-cudaError_t launch_set_state(const Dev<Real>& d, cudaStream_t s);
+cudaError_t launch_set_state(const Dev<Real>& d, const double* x, const double* v, const int* type, const double* mass,
+                             const int* img, cudaStream_t s);
 template <typename Real>
-cudaError_t launch_get_state(const Dev<Real>& d, int pc, int ac, cudaStream_t s);
+cudaError_t launch_get_state(const Dev<Real>& d, int pc, int ac, double* x, double* v, int* img, cudaStream_t s);
 template <typename Real>
-cudaError_t launch_get_forces(const Dev<Real>& d, int pc, cudaStream_t s);
+cudaError_t launch_get_forces(const Dev<Real>& d, int pc, double* f, double* U, cudaStream_t s);
+template <typename Real>
+cudaError_t launch_batch_begin(const Dev<Real>* devs, int m, cudaStream_t s);
+template <typename Real>
+cudaError_t launch_batch_end(const Dev<Real>* devs, int m, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_get_nlist(const Dev<Real>& d, int pc, int* rows, int* counts, int width,
                              cudaStream_t s);

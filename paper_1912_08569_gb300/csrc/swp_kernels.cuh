@@ -3259,19 +3259,28 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_batch(const Dev<Real>*
 // ---------------------------------------------------------------------------
 // Host-exchange kernels (user order <-> slot order).
 
+// A new state from user-order arrays in device memory (v, type, mass, img null:
+// zero, 0, one, zero), read where they are; also zeroes the cell counts and marks
+// the control block (cleared before) for forces to be computed on a new list.
 template <typename Real>
-__global__ void k_set_state(Dev<Real> d)
+__global__ void k_set_state(Dev<Real> d, const double* x_in, const double* v_in, const int* type, const double* mass,
+                            const int* img)
 {
     typedef typename Dev<Real>::R4 R4;
     typedef typename Dev<Real>::P4 P4;
-    const int n = d.n;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int n = d.n, t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    if (t == 0) {
+        d.ctl->state = 1;
+        d.ctl->need_rebuild = 1;
+    }
+    for (int c = t; c < d.ncell; c += nt) d.cell_cnt[c] = 0;
+    for (int i = t; i < n; i += nt) {
         long long qs[3];
         for (int c = 0; c < 3; c++) {
             // wrap into [0, L) and round to the fixed-point grid: one rounding per
             // operation (no contraction), so the conversion is reproducible
             double L = (double)d.Lq[c] * kInvFix;
-            double x = d.io[3 * i + c];
+            double x = x_in[3 * i + c];
             double fl = floor(__ddiv_rn(x, L));
             int im = (int)fl;
             double xw = __dsub_rn(x, __dmul_rn(fl, L));
@@ -3285,10 +3294,10 @@ __global__ void k_set_state(Dev<Real> d)
                 im--;
             }
             d.xq[0][c * n + i] = q;
-            d.img[0][c * n + i] = im + d.io_int[n + 3 * i + c];
+            d.img[0][c * n + i] = im + (img ? img[3 * i + c] : 0);
             qs[c] = q;
         }
-        int ty = d.io_int[i];
+        int ty = type ? type[i] : 0;
         if ((unsigned)ty >= (unsigned)d.ntypes) {  // (device input is not checked on the host)
             atomicOr(&d.ctl->status, kStatusBadType);
             ty = 0;
@@ -3300,47 +3309,51 @@ __global__ void k_set_state(Dev<Real> d)
         p.w = snap_bits((i << kTypeBits) | ty, d);
         d.pos[0][i] = p;
         R4 v;
-        v.x = (Real)d.io[3 * n + 3 * i + 0];
-        v.y = (Real)d.io[3 * n + 3 * i + 1];
-        v.z = (Real)d.io[3 * n + 3 * i + 2];
-        v.w = (Real)(1.0 / d.io[6 * n + i]);
+        v.x = v_in ? (Real)v_in[3 * i + 0] : Real(0);
+        v.y = v_in ? (Real)v_in[3 * i + 1] : Real(0);
+        v.z = v_in ? (Real)v_in[3 * i + 2] : Real(0);
+        v.w = mass ? (Real)(1.0 / mass[i]) : Real(1);
         d.vel[0][i] = v;
     }
 }
 
+// The state in user order into x, v, img (each may be null), device memory.
 template <typename Real>
-__global__ void k_get_state(Dev<Real> d, int pc, int ac)
+__global__ void k_get_state(Dev<Real> d, int pc, int ac, double* x, double* v_out, int* img)
 {
     typedef typename Dev<Real>::R4 R4;
     const int n = d.n;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-        const int bits = pos_bits(d.pos[pc][q]);
-        int tag = bits >> kTypeBits;
-        R4 v = d.vel[ac][q];
+        const size_t tag = pos_bits(d.pos[pc][q]) >> kTypeBits;
+        const R4 v = d.vel[ac][q];
         for (int c = 0; c < 3; c++) {
-            d.io[3 * tag + c] = (double)d.xq[ac][c * n + q] * kInvFix;
-            d.io_int[n + 3 * tag + c] = d.img[ac][c * n + q];
+            if (x) x[3 * tag + c] = (double)d.xq[ac][c * n + q] * kInvFix;
+            if (img) img[3 * tag + c] = d.img[ac][c * n + q];
         }
-        d.io[3 * n + 3 * tag + 0] = (double)v.x;
-        d.io[3 * n + 3 * tag + 1] = (double)v.y;
-        d.io[3 * n + 3 * tag + 2] = (double)v.z;
-        d.io_int[tag] = bits & ((1 << kTypeBits) - 1);
+        if (v_out) {
+            v_out[3 * tag + 0] = (double)v.x;
+            v_out[3 * tag + 1] = (double)v.y;
+            v_out[3 * tag + 2] = (double)v.z;
+        }
     }
 }
 
-// pc < 0: the current snapshot set as the control block records it.
+// Forces in user order into f (device memory).  pc < 0: the current snapshot set
+// as the control block records it.  U (may be null): the potential energy of the
+// thermo record.
 template <typename Real>
-__global__ void k_get_forces(Dev<Real> d, int pc)
+__global__ void k_get_forces(Dev<Real> d, int pc, double* f_out, double* U)
 {
     typedef typename Dev<Real>::R4 R4;
     const int n = d.n;
     if (pc < 0) pc = d.ctl->pos_cur;
+    if (U && blockIdx.x == 0 && threadIdx.x == 0) U[0] = d.ctl->thermo[Q_U2] + d.ctl->thermo[Q_U3];
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
-        int tag = pos_bits(d.pos[pc][q]) >> kTypeBits;
-        R4 f = d.force[q];
-        d.io[3 * tag + 0] = (double)f.x;
-        d.io[3 * tag + 1] = (double)f.y;
-        d.io[3 * tag + 2] = (double)f.z;
+        const size_t tag = pos_bits(d.pos[pc][q]) >> kTypeBits;
+        const R4 f = d.force[q];
+        f_out[3 * tag + 0] = (double)f.x;
+        f_out[3 * tag + 1] = (double)f.y;
+        f_out[3 * tag + 2] = (double)f.z;
     }
 }
 
@@ -3556,25 +3569,18 @@ static __global__ void k_pgrad_total(const double* part, int nblocks, double* to
     }
 }
 
-// Start of one device-driven evaluation (swp_eval_grad): resets the control
-// block as a new state does (forces stale, list to be rebuilt), writes the
-// reactive pair's coefficients from theta = (lambda, eps, sigma) in device
-// memory into both (ti, tj) entries of the device pair table (the
-// theta-dependent ones; the same arithmetic as the host table), and fills
-// the state staging: velocities 0, masses 1, images 0, types from type.
-// c_rmin = 2^(1/n), c_rb = ((1 - sqrt(1/2)) / 2)^(-1/n) (host constants),
-// rbond > 0: the bond radius as given.
+// Start of one device-driven evaluation (swp_eval_grad), one warp: clears the
+// control block (k_set_state follows) and writes the reactive pair's coefficients
+// from theta = (lambda, eps, sigma) in device memory into both (ti, tj) entries
+// of the device pair table (the theta-dependent ones; the same arithmetic as the
+// host table).  c_rmin = 2^(1/n), c_rb = ((1 - sqrt(1/2)) / 2)^(-1/n) (host
+// constants), rbond > 0: the bond radius as given.
 template <typename Real>
-__global__ void k_eval_prep(Dev<Real> d, int ti, int tj, const double* theta, double c_rmin, double c_rb,
-                            double rbond, const int* type)
+__global__ void k_eval_prep(Dev<Real> d, int ti, int tj, const double* theta, double c_rmin, double c_rb, double rbond)
 {
-    const int n = d.n;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        Ctl* ctl = d.ctl;
-        int* w = (int*)ctl;
-        for (int k = 0; k < (int)(sizeof(Ctl) / sizeof(int)); k++) w[k] = 0;
-        ctl->state = 1;
-        ctl->need_rebuild = 1;
+    int* w = (int*)d.ctl;
+    for (int k = threadIdx.x; k < (int)(sizeof(Ctl) / sizeof(int)); k += 32) w[k] = 0;
+    if (threadIdx.x == 0) {
         const double lam = theta[0], eps = theta[1], sig = theta[2];
         PairP<Real>* tab = (PairP<Real>*)d.table;
         PairP<Real> e = tab[ti * d.ntypes + tj];
@@ -3589,14 +3595,27 @@ __global__ void k_eval_prep(Dev<Real> d, int ti, int tj, const double* theta, do
         tab[ti * d.ntypes + tj] = e;
         tab[tj * d.ntypes + ti] = e;
     }
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        for (int c = 0; c < 3; c++) {
-            d.io[3 * n + 3 * i + c] = 0.0;
-            d.io_int[n + 3 * i + c] = 0;
-        }
-        d.io[6 * n + i] = 1.0;
-        d.io_int[i] = type ? type[i] : 0;
-    }
+}
+
+// Before a batched launch: every system's barrier counter starts at zero.
+template <typename Real>
+__global__ void k_batch_begin(const Dev<Real>* devs, int m)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < m) devs[r].ctl->barrier = 0;
+}
+
+// After it: every system's control block into its mirror in host memory (one
+// warp per system), so that the systems' next synchronising calls need no copy
+// of their own (96 systems: one launch for 96 copies of 8 us).
+template <typename Real>
+__global__ void k_batch_end(const Dev<Real>* devs, int m)
+{
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (r >= m || !devs[r].mirror) return;
+    const int* src = (const int*)devs[r].ctl;
+    int* dst = (int*)devs[r].mirror;
+    for (int k = lane; k < (int)(sizeof(Ctl) / sizeof(int)); k += 32) dst[k] = src[k];
 }
 
 #endif  // SWP_HAS_RESIDENT

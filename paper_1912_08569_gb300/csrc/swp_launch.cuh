@@ -78,26 +78,41 @@ cudaError_t run_occupancy(int block, int* blocks_per_sm)
 static inline int io_grid(int n) { return n > 0 ? (n + 255) / 256 : 1; }
 
 template <typename Real>
-cudaError_t launch_set_state(const Dev<Real>& d, cudaStream_t s)
+cudaError_t launch_set_state(const Dev<Real>& d, const double* x, const double* v, const int* type, const double* mass,
+                             const int* img, cudaStream_t s)
 {
     if (d.n == 0) return cudaSuccess;
-    single::k_set_state<Real><<<io_grid(d.n), 256, 0, s>>>(d);
+    single::k_set_state<Real><<<io_grid(d.n), 256, 0, s>>>(d, x, v, type, mass, img);
     return cudaGetLastError();
 }
 
 template <typename Real>
-cudaError_t launch_get_state(const Dev<Real>& d, int pc, int ac, cudaStream_t s)
+cudaError_t launch_get_state(const Dev<Real>& d, int pc, int ac, double* x, double* v, int* img, cudaStream_t s)
 {
     if (d.n == 0) return cudaSuccess;
-    single::k_get_state<Real><<<io_grid(d.n), 256, 0, s>>>(d, pc, ac);
+    single::k_get_state<Real><<<io_grid(d.n), 256, 0, s>>>(d, pc, ac, x, v, img);
     return cudaGetLastError();
 }
 
 template <typename Real>
-cudaError_t launch_get_forces(const Dev<Real>& d, int pc, cudaStream_t s)
+cudaError_t launch_get_forces(const Dev<Real>& d, int pc, double* f, double* U, cudaStream_t s)
 {
     if (d.n == 0) return cudaSuccess;
-    single::k_get_forces<Real><<<io_grid(d.n), 256, 0, s>>>(d, pc);
+    single::k_get_forces<Real><<<io_grid(d.n), 256, 0, s>>>(d, pc, f, U);
+    return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t launch_batch_begin(const Dev<Real>* devs, int m, cudaStream_t s)
+{
+    single::k_batch_begin<Real><<<(m + 127) / 128, 128, 0, s>>>(devs, m);
+    return cudaGetLastError();
+}
+
+template <typename Real>
+cudaError_t launch_batch_end(const Dev<Real>* devs, int m, cudaStream_t s)
+{
+    single::k_batch_end<Real><<<(m + 7) / 8, 256, 0, s>>>(devs, m);
     return cudaGetLastError();
 }
 
@@ -133,24 +148,27 @@ cudaError_t launch_param_grad(const Dev<Real>& d, int pc, double* sd, double* pa
 
 template <typename Real>
 cudaError_t launch_eval_prep(const Dev<Real>& d, int ti, int tj, const double* theta, double c_rmin, double c_rb,
-                             double rbond, const int* type, cudaStream_t s)
+                             double rbond, cudaStream_t s)
 {
-    single::k_eval_prep<Real><<<io_grid(d.n), 256, 0, s>>>(d, ti, tj, theta, c_rmin, c_rb, rbond, type);
+    single::k_eval_prep<Real><<<1, 32, 0, s>>>(d, ti, tj, theta, c_rmin, c_rb, rbond);
     return cudaGetLastError();
 }
 
 #define SWP_INSTANTIATE(R)                                                                       \
     template cudaError_t launch_run<R>(const Dev<R>&, const RunArgs&, int, int, cudaStream_t);   \
     template cudaError_t run_occupancy<R>(int, int*);                                            \
-    template cudaError_t launch_set_state<R>(const Dev<R>&, cudaStream_t);                       \
-    template cudaError_t launch_get_state<R>(const Dev<R>&, int, int, cudaStream_t);             \
-    template cudaError_t launch_get_forces<R>(const Dev<R>&, int, cudaStream_t);                 \
+    template cudaError_t launch_set_state<R>(const Dev<R>&, const double*, const double*, const int*, const double*, \
+                                             const int*, cudaStream_t);                          \
+    template cudaError_t launch_get_state<R>(const Dev<R>&, int, int, double*, double*, int*, cudaStream_t); \
+    template cudaError_t launch_get_forces<R>(const Dev<R>&, int, double*, double*, cudaStream_t); \
+    template cudaError_t launch_batch_begin<R>(const Dev<R>*, int, cudaStream_t);                \
+    template cudaError_t launch_batch_end<R>(const Dev<R>*, int, cudaStream_t);                  \
     template cudaError_t launch_get_nlist<R>(const Dev<R>&, int, int*, int*, int, cudaStream_t); \
     SWP_BATCH_DEFINE(R)                                                                          \
     template cudaError_t launch_param_grad<R>(const Dev<R>&, int, double*, double*, const double*, double*, \
                                               double*, double*, cudaStream_t);                            \
     template cudaError_t launch_eval_prep<R>(const Dev<R>&, int, int, const double*, double, double, double, \
-                                             const int*, cudaStream_t);                                  \
+                                             cudaStream_t);                                              \
     template size_t run_smem_bytes<R>();
 
 }  // namespace swp
