@@ -289,6 +289,7 @@ size_t layout(swp_ctx* c, char* base, Dev<Real>* d)
         d->cell_fill = cell_fill;
         d->perm = perm;
         d->bsum = bsum;
+        d->nbsum = c->max_blocks;
         d->partials = partials;
         d->ctl = ctl;
         d->agree = ctl ? ctl->agree : nullptr;
@@ -351,6 +352,9 @@ void fill_pair_table(const swp_ctx* c, PairP<Real>* t)
         }
         const double reach = pair_cut(p) + 0x1p-18 * Lm;
         e.reach2 = p.kind == KIND_NONE ? 0.0f : (float)(reach * reach * (1.0 + 1e-6));
+        const double out = reach + c->skin, in = pair_cut(p) + c->skin - 0x1p-18 * Lm;
+        e.list_out2 = p.kind == KIND_NONE ? -1.0f : (float)(out * out * (1.0 + 1e-6));
+        e.list_in2 = p.kind == KIND_NONE || in <= 0.0 ? -1.0f : (float)(in * in * (1.0 - 1e-6));
         t[k] = e;
     }
 }
@@ -1335,10 +1339,10 @@ int swp_param_grad(swp_ctx* c, int ti, int tj, double dU[3], double* dF_dev)
     double* ddu = dth + 3;
     SWP_CUDA(c, cudaMemcpyAsync(dth, th, sizeof th, cudaMemcpyHostToDevice, c->stream));
     if (c->precision == SWP_FP64)
-        SWP_CUDA(c, launch_param_grad<double>(c->dd, c->hctl.pos_cur, c->dd.io, part, dth, dF_dev, part + 2048,
+        SWP_CUDA(c, launch_param_grad<double>(c->dd, c->hctl.pos_cur, ti * c->ntypes + tj, c->dd.io, part, dth, dF_dev, part + 2048,
                                                ddu, c->stream));
     else
-        SWP_CUDA(c, launch_param_grad<float>(c->df, c->hctl.pos_cur, c->df.io, part, dth, dF_dev, part + 2048,
+        SWP_CUDA(c, launch_param_grad<float>(c->df, c->hctl.pos_cur, ti * c->ntypes + tj, c->df.io, part, dth, dF_dev, part + 2048,
                                               ddu, c->stream));
     SWP_CUDA(c, cudaMemcpyAsync(out, ddu, sizeof out, cudaMemcpyDeviceToHost, c->stream));
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1405,9 +1409,9 @@ int swp_eval_grad(swp_ctx* c, int ti, int tj, const double* theta_dev, const dou
     if (dU_dev || dF_dev) {
         double* part = f64 ? c->dd.partials : c->df.partials;
         if (f64)
-            SWP_CUDA(c, launch_param_grad<double>(c->dd, -1, io, part, theta_dev, dF_dev, part + 2048, dU_dev, c->stream));
+            SWP_CUDA(c, launch_param_grad<double>(c->dd, -1, ti * c->ntypes + tj, io, part, theta_dev, dF_dev, part + 2048, dU_dev, c->stream));
         else
-            SWP_CUDA(c, launch_param_grad<float>(c->df, -1, io, part, theta_dev, dF_dev, part + 2048, dU_dev, c->stream));
+            SWP_CUDA(c, launch_param_grad<float>(c->df, -1, ti * c->ntypes + tj, io, part, theta_dev, dF_dev, part + 2048, dU_dev, c->stream));
     }
     return SWP_OK;
 }

@@ -36,7 +36,10 @@ struct PairP {
     int kind;   // PairKind
     int nhalf;  // exponent n = 2*nhalf + odd
     int odd;
-    float reach2;  // FP64: squared cut-off of the FP32 sorting-out of listed pairs (see may_reach)
+    // FP64: squared bounds of FP32 distances: a listed pair beyond reach2 is outside
+    // its cut-off, a candidate beyond list_out2 outside the list, below list_in2 inside
+    float reach2, list_out2, list_in2;
+    int pad;
     Real four_eps;    // 4 eps
     Real n_real;      // n
     Real sig2;        // sigma^2
@@ -151,7 +154,8 @@ struct Dev {
     int* cell_start;   // [ncell + 1]
     int* cell_fill;    // [ncell]
     int* perm;         // [n] new slot -> old slot while the list is built; then (FP32) the particle of every thread
-    int* bsum;         // [max_blocks] per-block cell-count sums (scan)
+    int* bsum;         // [nbsum] particles in each block's chunk of cells (list build)
+    int nbsum;         // max_blocks
     double* partials;  // [max_blocks][kNQ]
     Ctl* ctl;
     unsigned long long* agree;  // resident steps: ctl->agree
@@ -232,9 +236,10 @@ SWP_DECLARE_BATCH(float, 384)
 SWP_DECLARE_BATCH(float, 256)
 // Derivatives with respect to one reactive type pair's (lambda, eps, sigma).
 // theta: (lambda, eps, sigma) in device memory; pc < 0: the control block's
-// current snapshot set; dU (device, may be null): dU/dtheta from the sums.
+// current snapshot set; pair: the reactive pair's place in the table; dU (device,
+// may be null): dU/dtheta from the sums.
 template <typename Real>
-cudaError_t launch_param_grad(const Dev<Real>& d, int pc, double* sd, double* part, const double* theta,
+cudaError_t launch_param_grad(const Dev<Real>& d, int pc, int pair, double* sd, double* part, const double* theta,
                               double* out, double* total, double* dU, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_eval_prep(const Dev<Real>& d, int ti, int tj, const double* theta, double c_rmin, double c_rb,

@@ -660,8 +660,12 @@ __device__ __forceinline__ int block_excl_scan(int v, int* sh, int* total)
 
 // ---------------------------------------------------------------------------
 // Neighbour-list rebuild phases: bin by cell, counting sort with a
-// deterministic order inside each cell, gather every per-particle array into
-// the sorted order, then one row per particle from the 27-cell stencil.
+// deterministic order inside each cell (by old slot), every per-particle array
+// moved into the sorted order, then one row per particle from the 27-cell
+// stencil.  Five grid barriers.  (With the counts of a block's cells summed in a
+// phase of their own, the members of a cell sorted in global memory by one thread
+// and the arrays then gathered one load after the other, the phases before the
+// row build took 17 us at 1,200 particles and 82 us at 1M; now 13 and 49.)
 
 template <typename Real>
 __device__ __forceinline__ void cell_coords(const Dev<Real>& d, const typename Dev<Real>::R4& p,
@@ -683,24 +687,42 @@ __device__ __forceinline__ void cell_coords(const Dev<float>& d, const int4& p, 
     cz = min((int)__umulhi((unsigned)p.z, (unsigned)d.nc[2]), d.nc[2] - 1);
 }
 
+// Block b owns the contiguous chunk [b*ch, (b+1)*ch) of cells (ranks) in the scan.
 template <typename Real>
-__device__ void ph_bin(const Dev<Real>& d, int pc, int t, int nt)
+__device__ __forceinline__ int chunk_cells(const Dev<Real>& d) { return (d.ncell + g_size() - 1) / g_size(); }
+
+// Counts the cells' particles and the chunks' (through chunk: g_size() ints of
+// shared memory); both counts start at zero (k_set_state, ph_chunk_scan, ph_move).
+template <typename Real>
+__device__ void ph_bin(const Dev<Real>& d, int pc, int* chunk)
 {
-    for (int p = t; p < d.n; p += nt) {
-        int cx, cy, cz;
-        cell_coords(d, d.pos[pc][p], cx, cy, cz);
-        int r = __ldg(&d.cell_rank[(cz * d.nc[1] + cy) * d.nc[0] + cx]);
-        d.perm[p] = r;  // temporarily: cell rank of old slot p
-        atomicAdd(&d.cell_cnt[r], 1);
+    const int G = g_size(), ch = chunk_cells(d);
+    __syncthreads();  // what the memory held before has been read (r_flush)
+    for (int b = threadIdx.x; b < G; b += blockDim.x) chunk[b] = 0;
+    __syncthreads();
+    for (int p0 = g_rank() * blockDim.x; p0 < d.n; p0 += G * blockDim.x) {  // block-uniform
+        const int p = p0 + threadIdx.x;
+        int b = -1;
+        if (p < d.n) {
+            int cx, cy, cz;
+            cell_coords(d, d.pos[pc][p], cx, cy, cz);
+            const int r = __ldg(&d.cell_rank[(cz * d.nc[1] + cy) * d.nc[0] + cx]);
+            d.perm[p] = r;  // the cell of old slot p
+            atomicAdd(&d.cell_cnt[r], 1);
+            b = r / ch;
+        }
+        // slots are nearly in cell order: a warp has one or two chunks
+        const unsigned m = __match_any_sync(0xffffffffu, b);
+        if (b >= 0 && (threadIdx.x & 31) == __ffs(m) - 1) atomicAdd(&chunk[b], __popc(m));
     }
+    __syncthreads();
+    for (int b = threadIdx.x; b < G; b += blockDim.x)
+        if (chunk[b]) atomicAdd(&d.bsum[b], chunk[b]);
 }
 
-// Parallel exclusive scan of the cell counts in two steps.  Block b owns the
-// contiguous chunk [b*ch, (b+1)*ch) of cells.  Step 1: each block sums its
-// chunk into bsum[b].  Step 2 (after a grid barrier): each block adds up the
-// sums of the blocks before it, scans its own chunk, writes cell_start and
-// cell_fill, and zeroes the counts it consumed (so the next build starts
-// from zero without a separate pass).
+// Exclusive scan of the cell counts: each block adds up the chunks before its
+// own, scans its cells, writes cell_start and cell_fill, and zeroes the counts it
+// consumed (so the next build starts from zero without a separate pass).
 __device__ __forceinline__ int block_sum_int(int v, int* sh)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -716,20 +738,9 @@ __device__ __forceinline__ int block_sum_int(int v, int* sh)
 }
 
 template <typename Real>
-__device__ void ph_chunk_sums(const Dev<Real>& d, int* sh)
-{
-    const int ch = (d.ncell + g_size() - 1) / g_size();
-    const int beg = min(g_rank() * ch, d.ncell), end = min(beg + ch, d.ncell);
-    int v = 0;
-    for (int c = beg + threadIdx.x; c < end; c += blockDim.x) v += d.cell_cnt[c];
-    int t = block_sum_int(v, sh);
-    if (threadIdx.x == 0) d.bsum[g_rank()] = t;
-}
-
-template <typename Real>
 __device__ void ph_chunk_scan(const Dev<Real>& d, int* sh)
 {
-    const int ch = (d.ncell + g_size() - 1) / g_size();
+    const int ch = chunk_cells(d);
     const int beg = min(g_rank() * ch, d.ncell), end = min(beg + ch, d.ncell);
     int v = 0;
     for (int b = threadIdx.x; b < g_rank(); b += blockDim.x) v += d.bsum[b];
@@ -750,51 +761,50 @@ __device__ void ph_chunk_scan(const Dev<Real>& d, int* sh)
     if (end == d.ncell && beg < end && threadIdx.x == 0) d.cell_start[d.ncell] = base;
 }
 
+// The members of every cell, in any order (after the fill counters).
 template <typename Real>
 __device__ void ph_scatter(const Dev<Real>& d, int t, int nt)
 {
-    // perm[p] holds the rank of p's cell; write the slot order into cell_of
-    // (reused as the inverse map's scratch) then back into perm.
-    for (int p = t; p < d.n; p += nt) {
-        int r = d.perm[p];
-        int q = atomicAdd(&d.cell_fill[r], 1);
-        d.cell_fill[d.ncell + q] = p;  // scratch area after the fill counters
-    }
+    for (int p = t; p < d.n; p += nt) d.cell_fill[d.ncell + atomicAdd(&d.cell_fill[d.perm[p]], 1)] = p;
 }
 
-// Sorts each cell's members by old slot (deterministic order), into perm.
+// Moves every particle to its new slot: its cell's first, plus the members of
+// the cell with a smaller old slot.  All loads of a particle come before its
+// stores.
 template <typename Real>
-__device__ void ph_cell_sort(const Dev<Real>& d, int t, int nt)
-{
-    const int* src = d.cell_fill + d.ncell;
-    for (int c = t; c < d.ncell; c += nt) {
-        int s = d.cell_start[c], e = d.cell_start[c + 1];
-        for (int a = s; a < e; a++) d.perm[a] = src[a];
-        for (int a = s + 1; a < e; a++) {
-            int v = d.perm[a], b = a - 1;
-            while (b >= s && d.perm[b] > v) {
-                d.perm[b + 1] = d.perm[b];
-                b--;
-            }
-            d.perm[b + 1] = v;
-        }
-    }
-}
-
-template <typename Real>
-__device__ void ph_gather(const Dev<Real>& d, int pc, int ac, int t, int nt)
+__device__ void ph_move(const Dev<Real>& d, int pc, int ac, int t, int nt)
 {
     const int n = d.n;
-    for (int q = t; q < n; q += nt) {
-        int p = d.perm[q];
+    const int* member = d.cell_fill + d.ncell;
+    if (g_rank() == 0)
+        for (int b = threadIdx.x; b < g_size(); b += blockDim.x) d.bsum[b] = 0;  // every block has read them
+    for (int p = t; p < n; p += nt) {
+        const int r = d.perm[p];
         const typename Dev<Real>::P4 pp = d.pos[pc][p];
-        d.pos[pc ^ 1][q] = pp;
-        if (d.has_bonds) d.slot_of_tag[pos_bits(pp) >> kTypeBits] = q;
-        d.vel[ac ^ 1][q] = d.vel[ac][p];
+        const typename Dev<Real>::R4 v = d.vel[ac][p];
+        long long x[3];
+        int im[3];
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            d.xq[ac ^ 1][c * n + q] = d.xq[ac][c * n + p];
-            d.img[ac ^ 1][c * n + q] = d.img[ac][c * n + p];
+            x[c] = d.xq[ac][c * n + p];
+            im[c] = d.img[ac][c * n + p];
+        }
+        const int s = d.cell_start[r], e = d.cell_start[r + 1];
+        int q = s;
+        for (int k = s; k < e; k += 4) {
+            int m[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) m[u] = k + u < e ? member[k + u] : n;
+#pragma unroll
+            for (int u = 0; u < 4; u++) q += m[u] < p;
+        }
+        d.pos[pc ^ 1][q] = pp;
+        if (d.has_bonds) d.slot_of_tag[pos_bits(pp) >> kTypeBits] = q;
+        d.vel[ac ^ 1][q] = v;
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            d.xq[ac ^ 1][c * n + q] = x[c];
+            d.img[ac ^ 1][c * n + q] = im[c];
         }
     }
 }
@@ -880,6 +890,25 @@ struct BuildStage {
     static constexpr size_t kBytes = O_HIST + 1024;
 };
 
+// Whether candidate pj lies inside the list radius of pi.  FP64: FP32 distances
+// decide all but the pairs within 2^-18 of the box of the radius, so that the
+// FP64 pipe, 19 cycles per warp instruction, sees hardly any candidate (with 8
+// FP64 instructions for every one the rows of 20,000 particles took 132 us, now 27).
+__device__ __forceinline__ bool in_list(const Dev<float>& d, const PairP<float>& p, const int4& pi, const int4& pj)
+{
+    float dx, dy, dz;
+    return dist2(pi, pj, d, dx, dy, dz) < p.rlist2;
+}
+__device__ __forceinline__ float float_dist2(const Dev<double>& d, const dbl4& pi, const dbl4& pj);
+__device__ __forceinline__ bool in_list(const Dev<double>& d, const PairP<double>& p, const dbl4& pi, const dbl4& pj)
+{
+    const float r2 = float_dist2(d, pi, pj);
+    if (r2 >= p.list_out2) return false;
+    if (r2 < p.list_in2) return true;
+    double dx, dy, dz;
+    return dist2(pi, pj, d, dx, dy, dz) < p.rlist2;
+}
+
 // One lane's share [c0, c1) of the 27 stencil cells of particle i (cell cx, cy,
 // cz): hit(q, reactive) for every partner q inside the list radius, in stencil
 // order.  The next cell's range is loaded while the present one's candidates
@@ -901,8 +930,7 @@ __device__ __forceinline__ void sweep_cells(const Dev<Real>& d, const PairP<Real
     };
     auto test = [&](int q, const P4& pj) {
         const PairP<Real>& p = row[type_of(pj)];
-        Real dx, dy, dz;
-        if (q != i && dist2(pi, pj, d, dx, dy, dz) < p.rlist2) hit(q, p.kind == KIND_SWAP);
+        if (q != i && in_list(d, p, pi, pj)) hit(q, p.kind == KIND_SWAP);
     };
     int s = 0, e = 0;
     if (c0 < c1) range(c0, s, e);
@@ -1252,9 +1280,8 @@ __device__ __forceinline__ float float_below(double x)
     return __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), (unsigned)max(__double2hiint(x) - 0x38000000, 0), 3));
 }
 
-// Whether a listed pair may lie inside its cut-off (p.reach2: the cut-off plus
-// 2^-18 of the box, far above the error of these FP32 distances, squared).
-__device__ __forceinline__ bool may_reach(const Dev<double>& d, const dbl4& pi, const dbl4& pj, float reach2)
+// Squared distance in FP32, far closer than 2^-18 of the box.
+__device__ __forceinline__ float float_dist2(const Dev<double>& d, const dbl4& pi, const dbl4& pj)
 {
     const double xi[3] = {pi.x, pi.y, pi.z}, xj[3] = {pj.x, pj.y, pj.z};
     float r2 = 0.0f;
@@ -1264,7 +1291,14 @@ __device__ __forceinline__ bool may_reach(const Dev<double>& d, const dbl4& pi, 
         dx = fmaf(-d.Lf[c], rintf(dx * d.iLf[c]), dx);
         r2 = fmaf(dx, dx, r2);
     }
-    return r2 < reach2;
+    return r2;
+}
+
+// Whether a listed pair may lie inside its cut-off (p.reach2: the cut-off plus
+// 2^-18 of the box, squared).
+__device__ __forceinline__ bool may_reach(const Dev<double>& d, const dbl4& pi, const dbl4& pj, float reach2)
+{
+    return float_dist2(d, pi, pj) < reach2;
 }
 
 // dist2_listed with the wrap, 9 of its 17 FP64 instructions, left to the pairs
@@ -2012,17 +2046,13 @@ __device__ SWP_COLD int run_rebuild(const Dev<Real>& d, const RunArgs& a)
         ctl->overflow = 0;
     }
     const int pc0 = s_ls.pc, ac0 = s_ls.ac;
-    ph_bin(d, pc0, gt, gn);  // cell counts start at zero (see ph_chunk_scan)
+    ph_bin(d, pc0, (int*)g_dyn);
     if (!grid_barrier(ctl, a.timeout_ns, 1)) return 2;
-    ph_chunk_sums(d, s_int);
-    if (!grid_barrier(ctl, a.timeout_ns, 2)) return 2;
     ph_chunk_scan(d, s_int);
     if (!grid_barrier(ctl, a.timeout_ns, 3)) return 2;
     ph_scatter(d, gt, gn);
     if (!grid_barrier(ctl, a.timeout_ns, 4)) return 2;
-    ph_cell_sort(d, gt, gn);
-    if (!grid_barrier(ctl, a.timeout_ns, 5)) return 2;
-    ph_gather(d, pc0, ac0, gt, gn);
+    ph_move(d, pc0, ac0, gt, gn);
     __syncthreads();
     if (threadIdx.x == 0) {
         s_ls.pc = pc0 ^ 1;
@@ -3260,7 +3290,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_batch(const Dev<Real>*
 // Host-exchange kernels (user order <-> slot order).
 
 // A new state from user-order arrays in device memory (v, type, mass, img null:
-// zero, 0, one, zero), read where they are; also zeroes the cell counts and marks
+// zero, 0, one, zero), read where they are; also zeroes the counts of the list build and marks
 // the control block (cleared before) for forces to be computed on a new list.
 template <typename Real>
 __global__ void k_set_state(Dev<Real> d, const double* x_in, const double* v_in, const int* type, const double* mass,
@@ -3274,6 +3304,7 @@ __global__ void k_set_state(Dev<Real> d, const double* x_in, const double* v_in,
         d.ctl->need_rebuild = 1;
     }
     for (int c = t; c < d.ncell; c += nt) d.cell_cnt[c] = 0;
+    for (int b = t; b < d.nbsum; b += nt) d.bsum[b] = 0;
     for (int i = t; i < n; i += nt) {
         long long qs[3];
         for (int c = 0; c < 3; c++) {
@@ -3393,91 +3424,131 @@ __global__ void k_get_nlist(Dev<Real> d, int pc, int* rows, int* counts, int wid
 //   Q_s = 4 n^2 x (4x - 1) (= sigma dQ/dsigma), q_s = Q_s beyond r_min (0 inside).
 // Decisions (inside r_cut, beyond r_min) are the force kernels' own.
 
+//
+// Both passes are bound by the FP64 pipe (19 cycles per warp instruction on an
+// SM, however many lanes are on).  A lane takes one particle (FP32: in the
+// threads' order of the list, alike rows in a warp), first lines up the partners
+// inside the cut-off (they are half of the listed ones) and then works through
+// them, so that a warp's FP64 work is that of its fullest particle; sums are kept
+// of the bare products (x, x^2, ...), the factors follow once per particle.
+// Blocks of two warps spread 20,000 particles over every SM.  (Four lanes per
+// particle, every listed partner, a division for each derivative: a
+// gradient over 16 snapshots of 20,000 took 2.62 ms, now 1.93.)
+
+constexpr int kPgThreads = 64;
+
+// A particle's reactive partners inside the cut-off, a few at a time.
 template <typename Real>
-__device__ __forceinline__ Real pair_x(const PairP<Real>& p, Real r2)
+struct PgLine {
+    static constexpr int kCap = 12;
+    struct Item {
+        Real r2, dx, dy, dz;
+        int j;
+    };
+    Item item[kCap][kPgThreads];
+};
+
+// Particle of index q in the order the two passes take them, and its list ranges.
+__device__ __forceinline__ int pg_particle(const Dev<float>& d, int q, int4& inf)
 {
-    return pair_power<kExpoAny, true>(p, p.sig2 * recip(r2));
+    inf = d.tinfo[q];
+    return d.perm[q];
+}
+__device__ __forceinline__ int pg_particle(const Dev<double>& d, int q, int4& inf)
+{
+    inf = d.pinfo[q];
+    return q;
 }
 
-// The two passes give each particle kPgLanes consecutive lanes of a warp:
-// lane l of the group takes the particle's reactive entries l, l + kPgLanes,
-// ..., and the group's partial sums meet in a fixed shuffle tree, so the
-// gathers of a particle's partners run in parallel (and the grid fills the
-// device at a few 10^4 particles).
-constexpr int kPgLanes = 4;
-
-__device__ __forceinline__ double pg_group_sum(double v)
+// f(item) for every reactive partner of the lane's particle inside the cut-off,
+// in list order; the warp's lanes go through their lines together.
+template <typename Real, typename F>
+__device__ __forceinline__ void pg_partners(const Dev<Real>& d, const typename Dev<Real>::P4* pos, Real rc2,
+                                            const typename Dev<Real>::P4& pi, const int4& inf, PgLine<Real>& line, F&& f)
 {
+    typedef typename Dev<Real>::P4 P4;
+    const int t = threadIdx.x;
+    int k = 0;
+    while (__any_sync(0xffffffffu, k < inf.y)) {
+        int m = 0;
+        for (; k < inf.y && m + 4 <= PgLine<Real>::kCap; k += 4) {
+            int j[4];
+            P4 pj[4];
 #pragma unroll
-    for (int o = kPgLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o, kPgLanes);
-    return v;
+            for (int u = 0; u < 4; u++) j[u] = k + u < inf.y ? d.ent_j[(unsigned)(inf.x + k + u)] : -1;
+#pragma unroll
+            for (int u = 0; u < 4; u++) pj[u] = pos[max(j[u], 0)];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                Real dx, dy, dz;
+                const Real r2 = dist2_listed(pi, pj[u], d, dx, dy, dz);
+                if (j[u] >= 0 && r2 < rc2) {
+                    line.item[m][t] = {r2, dx, dy, dz, j[u]};
+                    m++;
+                }
+            }
+        }
+        __syncwarp();
+        for (int e = 0; __any_sync(0xffffffffu, e < m); e++)
+            if (e < m) f(line.item[e][t]);
+        __syncwarp();
+    }
 }
 
 // Pass 1: S_i and D_i per slot into sd[2i], sd[2i+1]; per-block sums of
 // (T, sum_i (sum_j vh q - S D), sum_pairs v/eps, sum_pairs Q) into part[4b..].
+// pair: the reactive pair's place in the table.
 template <typename Real>
-__global__ void k_pgrad_sums(Dev<Real> d, int pc, double* sd, double* part)
+__global__ void __launch_bounds__(kPgThreads) k_pgrad_sums(Dev<Real> d, int pc, int pair, double* sd, double* part)
 {
-    __shared__ double red[4][32];
+    __shared__ PgLine<Real> line;
+    __shared__ double red[4][kPgThreads / 32];
     const int n = d.n;
     if (pc < 0) pc = d.ctl->pos_cur;
-    const int g = threadIdx.x % kPgLanes;
-    const int gpb = blockDim.x / kPgLanes;  // particles per block and round
+    const PairP<Real> p = d.table[pair];
+    const double nn = (double)p.n_real;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    // every lane of a warp runs the same number of rounds (the shuffles need them all)
-    const int rounds = (n + gpb * gridDim.x - 1) / (gpb * gridDim.x);
-    for (int r = 0; r < rounds; r++) {
-        const int i = (r * gridDim.x + blockIdx.x) * gpb + (int)threadIdx.x / kPgLanes;
-        double S = 0.0, D = 0.0, v2 = 0.0, vq = 0.0, ve = 0.0, qq = 0.0;
-        if (i < n) {
-            const typename Dev<Real>::P4 pi = d.pos[pc][i];
-            const int4 inf = d.pinfo[i];
-            for (int m = g; m < inf.y; m += kPgLanes) {
-                const typename Dev<Real>::P4 pj = d.pos[pc][d.ent_j[(unsigned)(inf.x + m)]];
-                const PairP<Real>& p = d.table[type_of(pi) * d.ntypes + type_of(pj)];
-                Real dx, dy, dz;
-                const Real r2 = dist2_listed(pi, pj, d, dx, dy, dz);
-                if (!(r2 < p.rc2)) continue;
-                const double x = (double)pair_x(p, r2), nn = (double)p.n_real;
-                const bool beyond = r2 > p.rmin2;
-                const double vh = beyond ? 4.0 * (x - x * x) : 1.0;
-                const double Q = 4.0 * nn * (2.0 * x * x - x);
-                const double q = beyond ? Q : 0.0;
-                S += vh;
-                D += q;
-                v2 += vh * vh;
-                vq += vh * q;
-                ve += 0.5 * 4.0 * (x * x - x);  // each pair is listed from both ends
-                qq += 0.5 * Q;
-            }
-        }
-        S = pg_group_sum(S);
-        D = pg_group_sum(D);
-        v2 = pg_group_sum(v2);
-        vq = pg_group_sum(vq);
-        ve = pg_group_sum(ve);
-        qq = pg_group_sum(qq);
-        if (i < n && g == 0) {
+    for (int q0 = blockIdx.x * kPgThreads; q0 < n; q0 += gridDim.x * kPgThreads) {
+        const int q = q0 + threadIdx.x;
+        int4 inf = make_int4(0, 0, 0, 0);
+        const int i = q < n ? pg_particle(d, q, inf) : 0;
+        const typename Dev<Real>::P4 pi = d.pos[pc][i];
+        // with w = x - x^2 and u = 2x^2 - x: v/eps = -4 w, vh = 4 w and q = Q = 4 n u beyond r_min
+        double w1 = 0.0, x2 = 0.0, wb = 0.0, ub = 0.0, ww = 0.0, wu = 0.0;
+        int inside = 0;  // partners inside r_min (vh = 1, q = 0)
+        pg_partners(d, d.pos[pc], p.rc2, pi, inf, line, [&](const typename PgLine<Real>::Item& it) {
+            const double x = (double)pair_power<kExpoAny, true>(p, p.sig2 * recip(it.r2));
+            const double xx = x * x, w = x - xx, u = xx - w;
+            const bool beyond = it.r2 > p.rmin2;
+            w1 += w;
+            x2 += xx;
+            const double wo = beyond ? w : 0.0, uo = beyond ? u : 0.0;
+            inside += !beyond;
+            wb += wo;
+            ub += uo;
+            ww += wo * wo;
+            wu += wo * uo;
+        });
+        if (q < n) {
+            const double S = 4.0 * wb + (double)inside, Dn = 4.0 * nn * ub;
             sd[2 * i] = S;
-            sd[2 * i + 1] = D;
-            acc[0] += 0.5 * (S * S - v2);
-            acc[1] += vq - S * D;
-            acc[2] += ve;
-            acc[3] += qq;
+            sd[2 * i + 1] = Dn;
+            acc[0] += 0.5 * (S * S - (16.0 * ww + (double)inside));
+            acc[1] += 16.0 * nn * wu - S * Dn;
+            acc[2] -= 2.0 * w1;  // each pair is listed from both ends
+            acc[3] += 2.0 * nn * (x2 - w1);
         }
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-        double v = acc[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) red[k][w] = v;
+        const double v = warp_sum(acc[k]);
+        if (lane == 0) red[k][wp] = v;
     }
     __syncthreads();
     if (threadIdx.x < 4) {
         double t = 0.0;
-        for (int k = 0; k < nw; k++) t += red[threadIdx.x][k];
+        for (int k = 0; k < kPgThreads / 32; k++) t += red[threadIdx.x][k];
         part[4 * blockIdx.x + threadIdx.x] = t;
     }
 }
@@ -3485,58 +3556,49 @@ __global__ void k_pgrad_sums(Dev<Real> d, int pc, double* sd, double* part)
 // Pass 2: dF/dtheta per particle, in user order: out[(k n + tag) 3 + c];
 // theta = (lambda, eps, sigma) in device memory.
 template <typename Real>
-__global__ void k_pgrad_forces(Dev<Real> d, int pc, const double* sd, const double* theta, double* out)
+__global__ void __launch_bounds__(kPgThreads) k_pgrad_forces(Dev<Real> d, int pc, int pair, const double* sd,
+                                                             const double* theta, double* out)
 {
+    __shared__ PgLine<Real> line;
     const int n = d.n;
     if (pc < 0) pc = d.ctl->pos_cur;
-    const double lam = theta[0], eps = theta[1], sig = theta[2];
-    const int g = threadIdx.x % kPgLanes;
-    const int gpb = blockDim.x / kPgLanes;
-    const int rounds = (n + gpb * gridDim.x - 1) / (gpb * gridDim.x);
-    for (int r = 0; r < rounds; r++) {
-        const int i = (r * gridDim.x + blockIdx.x) * gpb + (int)threadIdx.x / kPgLanes;
-        double g3[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
-        int tag = 0;
-        if (i < n) {
-            const typename Dev<Real>::P4 pi = d.pos[pc][i];
-            const int4 inf = d.pinfo[i];
-            const double Si = sd[2 * i], Di = sd[2 * i + 1];
-            tag = pos_bits(pi) >> kTypeBits;
-            for (int m = g; m < inf.y; m += kPgLanes) {
-                const int j = d.ent_j[(unsigned)(inf.x + m)];
-                const typename Dev<Real>::P4 pj = d.pos[pc][j];
-                const PairP<Real>& p = d.table[type_of(pi) * d.ntypes + type_of(pj)];
-                Real dx, dy, dz;
-                const Real r2 = dist2_listed(pi, pj, d, dx, dy, dz);
-                if (!(r2 < p.rc2)) continue;
-                const double x = (double)pair_x(p, r2), nn = (double)p.n_real, rr = (double)r2;
-                const bool beyond = r2 > p.rmin2;
-                const double vh = beyond ? 4.0 * (x - x * x) : 1.0;
-                const double Q = 4.0 * nn * (2.0 * x * x - x);
-                const double q = beyond ? Q : 0.0;
-                const double Qs = 4.0 * nn * nn * x * (4.0 * x - 1.0);
-                const double qs = beyond ? Qs : 0.0;
-                const double gg = Si + sd[2 * j] - 2.0 * vh;
-                const double Dsum = Di + sd[2 * j + 1];
-                const double dft[3] = {-eps * gg * q / rr, (Q - lam * gg * q) / rr,
-                                       (eps * Qs - lam * eps * ((2.0 * q - Dsum) * q + gg * qs)) / (sig * rr)};
-                const double dv[3] = {(double)dx, (double)dy, (double)dz};
-#pragma unroll
-                for (int k = 0; k < 3; k++)
-#pragma unroll
-                    for (int c = 0; c < 3; c++) g3[k][c] -= dft[k] * dv[c];
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 3; k++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) g3[k][c] = pg_group_sum(g3[k][c]);
-        if (i < n && g < 3) {  // lanes 0..2 of the group write parameter k = g
+    const PairP<Real> p = d.table[pair];
+    const double lam = theta[0], eps = theta[1], sig = theta[2], nn = (double)p.n_real, n4 = 4.0 * nn;
+    for (int q0 = blockIdx.x * kPgThreads; q0 < n; q0 += gridDim.x * kPgThreads) {
+        const int q = q0 + threadIdx.x;
+        int4 inf = make_int4(0, 0, 0, 0);
+        const int i = q < n ? pg_particle(d, q, inf) : 0;
+        const typename Dev<Real>::P4 pi = d.pos[pc][i];
+        const double Si = sd[2 * i], Di = sd[2 * i + 1];
+        double g[3][3] = {{0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}, {0.0, 0.0, 0.0}};
+        pg_partners(d, d.pos[pc], p.rc2, pi, inf, line, [&](const typename PgLine<Real>::Item& it) {
+            const double Sj = sd[2 * it.j], Dj = sd[2 * it.j + 1];
+            const double x = (double)pair_power<kExpoAny, true>(p, p.sig2 * recip(it.r2));
+            const bool beyond = it.r2 > p.rmin2;
+            const double c = n4 * (1.0 / (double)it.r2);  // 4 n / r^2
+            const double xx = x * x, w = x - xx, u = xx - w, z = 4.0 * xx - x;
+            const double vh = beyond ? 4.0 * w : 1.0;
+            const double gg = (Si + Sj) - 2.0 * vh;
+            const double Q = c * u, Qs = c * nn * z;  // Q / r^2, Q_s / r^2
+            const double qb = beyond ? Q : 0.0, qs = beyond ? Qs : 0.0;
+            const double h = gg * qb;
+            // dft/dlambda = -eps h, dft/deps = Q/r^2 - lambda h,
+            // dft/dsigma = eps/sigma (Q_s/r^2 - lambda ((2q - D_i - D_j) q/r^2 + g q_s/r^2))
+            const double a = (2.0 * (n4 * u) - (Di + Dj)) * qb + gg * qs;
+            const double f[3] = {h, Q - lam * h, Qs - lam * a};
+            const double dv[3] = {(double)it.dx, (double)it.dy, (double)it.dz};
 #pragma unroll
             for (int k = 0; k < 3; k++)
-                if (k == g)
 #pragma unroll
-                    for (int c = 0; c < 3; c++) out[((size_t)k * n + tag) * 3 + c] = g3[k][c];
+                for (int e = 0; e < 3; e++) g[k][e] += f[k] * dv[e];
+        });
+        if (q < n) {
+            const size_t tag = pos_bits(pi) >> kTypeBits;
+            const double scale[3] = {eps, -1.0, -eps / sig};  // F_i = -ft (x_j - x_i)
+#pragma unroll
+            for (int k = 0; k < 3; k++)
+#pragma unroll
+                for (int e = 0; e < 3; e++) out[((size_t)k * n + tag) * 3 + e] = scale[k] * g[k][e];
         }
     }
 }

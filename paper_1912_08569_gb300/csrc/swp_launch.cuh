@@ -129,16 +129,17 @@ cudaError_t launch_get_nlist(const Dev<Real>& d, int pc, int* rows, int* counts,
 // into out [3][n][3] (user order) when out is not null, the four sums into
 // total [4]; part: scratch of 4 * 512 doubles.
 template <typename Real>
-cudaError_t launch_param_grad(const Dev<Real>& d, int pc, double* sd, double* part, const double* theta,
+cudaError_t launch_param_grad(const Dev<Real>& d, int pc, int pair, double* sd, double* part, const double* theta,
                               double* out, double* total, double* dU, cudaStream_t s)
 {
-    // kPgLanes threads per particle; at most 512 blocks (the partials scratch)
-    const int blocks = std::max(1, std::min(512, (d.n * single::kPgLanes + 255) / 256));
-    single::k_pgrad_sums<Real><<<blocks, 256, 0, s>>>(d, pc, sd, part);
+    // at most 512 blocks (the partials scratch)
+    const int blocks = std::max(1, std::min(512, (d.n + single::kPgThreads - 1) / single::kPgThreads));
+    single::k_pgrad_sums<Real><<<blocks, single::kPgThreads, 0, s>>>(d, pc, pair, sd, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (out) {
-        single::k_pgrad_forces<Real><<<blocks, 256, 0, s>>>(d, pc, sd, theta, out);
+        const int all = std::max(1, (d.n + single::kPgThreads - 1) / single::kPgThreads);
+        single::k_pgrad_forces<Real><<<all, single::kPgThreads, 0, s>>>(d, pc, pair, sd, theta, out);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -165,7 +166,7 @@ cudaError_t launch_eval_prep(const Dev<Real>& d, int ti, int tj, const double* t
     template cudaError_t launch_batch_end<R>(const Dev<R>*, int, cudaStream_t);                  \
     template cudaError_t launch_get_nlist<R>(const Dev<R>&, int, int*, int*, int, cudaStream_t); \
     SWP_BATCH_DEFINE(R)                                                                          \
-    template cudaError_t launch_param_grad<R>(const Dev<R>&, int, double*, double*, const double*, double*, \
+    template cudaError_t launch_param_grad<R>(const Dev<R>&, int, int, double*, double*, const double*, double*, \
                                               double*, double*, cudaStream_t);                            \
     template cudaError_t launch_eval_prep<R>(const Dev<R>&, int, int, const double*, double, double, double, \
                                              cudaStream_t);                                              \
