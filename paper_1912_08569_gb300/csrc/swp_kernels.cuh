@@ -1526,7 +1526,7 @@ __device__ __forceinline__ float advance_particle(const Dev<Real>& d, const RunA
         Real ddx = hdt * v.x, ddy = hdt * v.y, ddz = hdt * v.z;
         if (a.langevin) {
             const Real c1 = pick(Real(0), a.c1_f, a.c1_d);
-            const Real sd = pick(Real(0), a.c2_f, a.c2_d) * sqrt(im);
+            const Real sd = pick(Real(0), a.c2_f, a.c2_d) * (im == Real(1) ? Real(1) : sqrt(im));
             v.x = c1 * v.x + sd * z[0];
             v.y = c1 * v.y + sd * z[1];
             v.z = c1 * v.z + sd * z[2];
@@ -1578,9 +1578,16 @@ __device__ __forceinline__ float integrate_one(const Dev<Real>& d, const RunArgs
     return disp2;
 }
 
+// What a thread's FP32 thermo terms are multiplied by when they are folded: half
+// of a pair to each end, and the virial's sign (the force is on the owner).
+__device__ __forceinline__ float th_scale(int q)
+{
+    return q == Q_K ? 1.0f : q >= Q_W0 && q < Q_BONDS ? -0.5f : 0.5f;
+}
+
 // One entry's pair force on its owner (returned as the components of
-// f (x_i - x_j)), with the entry's share of energies, virial and bond count
-// when TH (the sampled step of a launch).  REACT: a reactive pair (two-body
+// f (x_i - x_j)), with the pair's energies, virial and bond count when TH (the
+// sampled step of a launch), bare: th_scale holds the factors.  REACT: a reactive pair (two-body
 // plus the three-body factor); else a purely two-body pair.
 template <typename Real, bool UNI, int X, bool REACT, bool TH>
 __device__ __forceinline__ void entry_force(const Dev<Real>& d, const PairP<Real>* tab,
@@ -1597,15 +1604,16 @@ __device__ __forceinline__ void entry_force(const Dev<Real>& d, const PairP<Real
     const bool in = r2 < p.rc2;
     Real v, ft;
     lj_eval<X, REACT>(p, r2, v, ft);
-    if (TH) acc.q[Q_U2] += in ? Real(0.5) * (v + p.ushift) : Real(0);
+    if (TH) acc.q[Q_U2] += in ? v + p.ushift : Real(0);
     if (REACT) {
         const bool beyond = r2 > p.rmin2;
         const Real vh = beyond ? (p.vshift - v) * p.inv_epshat : Real(1);
         const Real h = p.a * (Si + Sj - Real(2) * p.a * vh);
         ft = beyond ? ft * (Real(1) - h * p.inv_epshat) : ft;
         if (TH) {
-            acc.q[Q_U3] += in ? Real(0.5) * p.a * vh * (Si - p.a * vh) : Real(0);
-            acc.q[Q_BONDS] += (in && r2 < p.rbond2) ? Real(0.5) : Real(0);
+            const Real av = p.a * vh;
+            acc.q[Q_U3] += in ? av * (Si - av) : Real(0);
+            acc.q[Q_BONDS] += (in && r2 < p.rbond2) ? Real(1) : Real(0);
         }
     }
     ft = in ? ft : Real(0);
@@ -1613,13 +1621,12 @@ __device__ __forceinline__ void entry_force(const Dev<Real>& d, const PairP<Real
     fy = -ft * dy;
     fz = -ft * dz;
     if (!TH) return;
-    const Real hf = Real(0.5) * ft;
-    acc.q[Q_W0 + 0] += hf * dx * dx;
-    acc.q[Q_W0 + 1] += hf * dy * dy;
-    acc.q[Q_W0 + 2] += hf * dz * dz;
-    acc.q[Q_W0 + 3] += hf * dx * dy;
-    acc.q[Q_W0 + 4] += hf * dx * dz;
-    acc.q[Q_W0 + 5] += hf * dy * dz;
+    acc.q[Q_W0 + 0] += fx * dx;
+    acc.q[Q_W0 + 1] += fy * dy;
+    acc.q[Q_W0 + 2] += fz * dz;
+    acc.q[Q_W0 + 3] += fx * dy;
+    acc.q[Q_W0 + 4] += fx * dz;
+    acc.q[Q_W0 + 5] += fy * dz;
 }
 
 // The harmonic bonds of particle pi (vitrimer chains): F_i = k (r - r0) (x_j -
@@ -1643,8 +1650,9 @@ __device__ __forceinline__ void bond_forces(const Dev<Real>& d, const typename D
         fy += g * dy;
         fz += g * dz;
         if (!TH) continue;
-        acc.q[Q_U2] += Real(0.25) * d.bond_k * dr * dr;
-        const Real hf = Real(-0.5) * g;
+        // (FP32 terms are scaled when they are folded, th_scale)
+        acc.q[Q_U2] += (sizeof(Real) == 4 ? Real(0.5) : Real(0.25)) * d.bond_k * dr * dr;
+        const Real hf = sizeof(Real) == 4 ? g : Real(-0.5) * g;
         acc.q[Q_W0 + 0] += hf * dx * dx;
         acc.q[Q_W0 + 1] += hf * dy * dy;
         acc.q[Q_W0 + 2] += hf * dz * dz;
@@ -1760,7 +1768,7 @@ __device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const
 #pragma unroll
             for (int q = 0; q < kNQA; q++)
                 if (q != Q_K) {
-                    const float x = warp_sum(acc.q[q]);
+                    const float x = warp_sum(acc.q[q] * th_scale(q));
                     if (lane == q) run += (double)x;
                 }
         if (qn < b1) {
@@ -2115,9 +2123,8 @@ __device__ __forceinline__ void run_s_pass(const Dev<Real>& d, const RunArgs& a,
 // shared atomic per warp); the barrier arrival publishes it.
 __device__ __forceinline__ void warp_max_disp(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0 && v > 0.0f) atomicMax(&s_ls.dmax_bits, __float_as_uint(v));
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(v));  // (v >= 0: the bits order like the values)
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(&s_ls.dmax_bits, m);
 }
 
 template <typename Real, bool UNI, bool BONDS, bool TH>
@@ -2819,7 +2826,7 @@ __device__ __forceinline__ void r_forces(const Dev<float>& d, const RunArgs& a, 
         if ((t & ~31) < P) {  // the warp holds rows (the same in all its lanes)
 #pragma unroll
             for (int q = 0; q < kNQA; q++)
-                if (q != Q_K) warp_part(acc.q[q], q);
+                if (q != Q_K) warp_part(acc.q[q] * th_scale(q), q);
         } else if ((t & 31) == 0) {
 #pragma unroll
             for (int q = 0; q < kNQA; q++)
@@ -2918,7 +2925,16 @@ static __device__ int r_run(const Dev<float>& d, const RunArgs& a)
         // the noise of the next step's start, while the agreement is on its way
         float z[3] = {0.0f, 0.0f, 0.0f};
         const int lid = fd.w & 0xffff;
-        if (t < P && more && a.langevin) normals3(a.seed, step + 1, (unsigned)(lpos[lid].w >> kTypeBits), z);
+        int4 pi = make_int4(0, 0, 0, 0);
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 1.0f);
+        long long q[3] = {0, 0, 0};
+        if (t < P) {
+            pi = lpos[lid];
+            v = RS::vel()[t];
+#pragma unroll
+            for (int c = 0; c < 3; c++) q[c] = RS::xq()[3 * t + c];
+            if (more && a.langevin) normals3(a.seed, step + 1, (unsigned)(pi.w >> kTypeBits), z);
+        }
         __syncthreads();  // every row has read the old snapshots, fw is complete, the displacement bound is known
         if (k > 0) {
             if (!s_ls.ok) break;
@@ -2931,18 +2947,13 @@ static __device__ int r_run(const Dev<float>& d, const RunArgs& a)
         if (t < P) {
             const float* fw = RS::fw();
             const int i = b0 + lid;
-            const int4 pi = lpos[lid];
             // the force: the reactive row's sum plus the other row's
             fx = __fadd_rn(fx, fw[lid]);
             fy = __fadd_rn(fy, fw[kBlock + lid]);
             fz = __fadd_rn(fz, fw[2 * kBlock + lid]);
             if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(&d.ctl->status, kStatusNonfinite);
             if (!more) d.force[i] = make_float4(fx, fy, fz, 0.0f);
-            float4 v = RS::vel()[t];
-            long long q[3];
             int w[3];
-#pragma unroll
-            for (int c = 0; c < 3; c++) q[c] = RS::xq()[3 * t + c];
             int4 np = make_int4(0, 0, 0, 0);
             dmax = advance_particle(d, a, fx, fy, fz, F_CLOSING | (more ? F_OPENING : 0), z, pi.w, v, q, w, kin, np);
             if (more) {
