@@ -1273,8 +1273,8 @@ __device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc
 static __shared__ int s_nlist;  // entries lined up
 static __shared__ int s_nkeep;  // reactive pairs whose values the S pass kept (-1: not kept)
 
-// The float below a non-negative double, from its bits (the conversion
-// instruction runs on the FP64 pipe).
+// A non-negative double cut off to a float, from its bits (the conversion
+// instruction runs on the FP64 pipe).  Values below 2^-126 come out below it too.
 __device__ __forceinline__ float float_below(double x)
 {
     return __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), (unsigned)max(__double2hiint(x) - 0x38000000, 0), 3));
@@ -3204,8 +3204,17 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
                 d.tlog_step[2 * s_ls.tlog_slot] = stp + 1;
                 d.tlog_step[2 * s_ls.tlog_slot + 1] = g_size();
             }
-            if (th) thermo_partials(d, false, !more, lg);
-            if (!grid_barrier(ctl, a.timeout_ns, 21, more ? &ctl->dmax2[(stp + 1) & 1] : nullptr)) return false;
+            // a logged step that is not the launch's last adds its terms up while
+            // it waits (the record is read after the launch); the last step writes
+            // the partials that the launch reduces before its arrival
+            const bool late = th && more;
+            if (th && !late) thermo_partials(d, false, true, lg);
+            BarState bs;
+            bs.target = s_ls.bar_target;
+            bar_arrive(ctl, bs, more ? &ctl->dmax2[(stp + 1) & 1] : nullptr, &s_ls.dmax_bits);
+            if (late) thermo_partials(d, false, false, lg);
+            if (threadIdx.x == 0) s_ls.bar_target = bs.target;
+            if (!bar_wait(ctl, bs, a.timeout_ns, 21, &s_ls.ok)) return false;
             if (logged && threadIdx.x == 0) {  // every thread used the slot before the barrier
                 s_ls.tlog_k++;
                 s_ls.tlog_slot = s_ls.tlog_slot + 1 == d.tlog_cap ? 0 : s_ls.tlog_slot + 1;
@@ -3321,11 +3330,18 @@ __global__ void k_set_state(Dev<Real> d, const double* x_in, const double* v_in,
         for (int c = 0; c < 3; c++) {
             // wrap into [0, L) and round to the fixed-point grid: one rounding per
             // operation (no contraction), so the conversion is reproducible
-            double L = (double)d.Lq[c] * kInvFix;
-            double x = x_in[3 * i + c];
-            double fl = floor(__ddiv_rn(x, L));
-            int im = (int)fl;
-            double xw = __dsub_rn(x, __dmul_rn(fl, L));
+            const double L = (double)d.Lq[c] * kInvFix, x = x_in[3 * i + c];
+            double xw = x;
+            int im = 0;
+            // inside the box already (the bits of non-negative doubles order like
+            // their values): the quotient below is less than 1 and its floor 0, so
+            // nothing changes, and the division, most of this kernel's FP64 work
+            // (7 of the 200 us of a force call on 100,000 particles), is left out
+            if (!((unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(L))) {
+                const double fl = floor(__ddiv_rn(x, L));
+                im = (int)fl;
+                xw = __dsub_rn(x, __dmul_rn(fl, L));
+            }
             long long q = __double2ll_rn(__dmul_rn(xw, kFix));
             if (q >= d.Lq[c]) {
                 q -= d.Lq[c];

@@ -1,0 +1,193 @@
+"""The list build, the passes, the resident step and the device-array entry
+points at the sizes where they can go wrong: edges of sub-chunks, rows longer
+than what a lane or a wave of entries holds, odd and large exponents, blocks
+whose rows leave no spare warp, unaligned arrays, positions on the box faces.
+
+Forces, energies and bond counts against the oracle at the tolerances of the
+parity tests (FP32 1e-5, FP64 1e-12 of the oracle's error scales, from the
+arithmetic); two ways of computing the same thing are held to the same bits.
+"""
+import numpy as np
+import pytest
+
+from gpu_helpers import TOL, assert_forces_match, assert_thermo_match, make_gpu, oracle_pairs
+from paper_1912_08569_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1912_08569_gb300.build import build
+
+    build()
+
+
+def _wl(count, density=0.5, lam=1.0, seed=11, **pair):
+    wl = inputs.workload("mix2k", lambda3=lam, n=count, density=density, seed=seed)
+    if pair:
+        wl["pairs"] = inputs.swap_pairs(lambda3=lam, **pair)
+    return wl
+
+
+def _check(orc, wl, precision, s):
+    s.compute_forces()
+    ref = orc.forces(wl["x"], wl["types"], wl["n_types"], oracle_pairs(orc, wl), wl["box"], fp32=precision == "fp32")
+    assert_forces_match(s.forces(), ref, TOL[precision], precision)
+    assert_thermo_match(s.thermo(), ref, TOL[precision], precision)
+
+
+# ten blocks: 768 (FP32) and 512 (FP64) particles fill a sub-chunk
+@pytest.mark.parametrize("precision,n", [("fp32", 7680), ("fp32", 7681), ("fp32", 15370),
+                                         ("fp64", 5120), ("fp64", 5121)])
+def test_sub_chunk_edges(orc, precision, n):
+    wl = _wl(n)
+    s = make_gpu(wl, precision)
+    s.set_grid(10)
+    _check(orc, wl, precision, s)
+
+
+# r_cut = 2.4: about 34 reactive and 3 other partners, more than a lane of the
+# build holds; on ten blocks of 300 FP64 particles several waves of entries
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("grid", [0, 10])
+def test_long_rows(orc, precision, grid):
+    wl = _wl(3000, n=10, rcut=2.4)
+    s = make_gpu(wl, precision)
+    if grid:
+        s.set_grid(grid)
+    _check(orc, wl, precision, s)
+
+
+# reactive and other exponents: short products, selected squarings, odd powers
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,wca_n", [(10, 6), (12, 6), (9, 5), (1, 7), (100, 12), (128, 127)])
+def test_exponents(orc, precision, n, wca_n):
+    wl = _wl(900, density=0.3, n=n, wca_n=wca_n)
+    if n >= 100:  # no overlaps on the steep walls
+        wl["x"] = inputs.rsa_positions(900, wl["box"], 1.0, seed=4)
+    _check(orc, wl, precision, make_gpu(wl, precision))
+
+
+@pytest.mark.parametrize("n,density", [(90, 0.2), (114_000, 0.4)])  # empty blocks; rows in every warp
+def test_resident_equals_two_barrier_path_at_the_ends(n, density):
+    wl = _wl(n, density, seed=5)
+    wl["v"] = inputs.maxwell_velocities(n, 0.2, 1.0, seed=6)
+    a, b = make_gpu(wl, "fp32"), make_gpu(wl, "fp32")
+    b.set_resident(False)
+    logs = []
+    for s in (a, b):
+        s.set_thermo_log(7, 20)
+        s.run(120, 0.001, 0.2, 1.0)
+        logs.append(s.thermo_log())
+    assert a.thermo()["resident_steps"] == 120 and b.thermo()["resident_steps"] == 0
+    for p, q in zip(a.state(), b.state()):
+        assert np.array_equal(p, q)
+    assert np.array_equal(logs[0]["step"], logs[1]["step"])
+    assert np.array_equal(logs[0]["n_bonds"], logs[1]["n_bonds"])
+    # FP32 terms, summed in another order: 1e-5 as for the energies against the oracle
+    for k in ("U2", "U3", "K"):
+        np.testing.assert_allclose(logs[0][k], logs[1][k], rtol=1e-5)
+
+
+class _At:
+    """A device address inside a buffer, as the binding takes it."""
+
+    def __init__(self, buf, offset):
+        self.buf, self.offset = buf, offset
+
+    def data_ptr(self):
+        return self.buf.data_ptr() + self.offset
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_unaligned_device_arrays(precision):
+    import torch
+    from paper_1912_08569_gb300 import _abi as A
+
+    wl = _wl(1000, 0.3)
+    n = wl["n"]
+
+    def at4(a):  # the same bytes four bytes off an 8-byte boundary
+        raw = torch.from_numpy(np.ascontiguousarray(a).view(np.uint8).reshape(-1)).cuda()
+        buf = torch.zeros(raw.numel() + 16, dtype=torch.uint8, device="cuda")
+        buf[4:4 + raw.numel()] = raw
+        return _At(buf, 4)
+
+    got = []
+    for shift in (False, True):
+        s = make_gpu(wl, precision)
+        if shift:
+            A.swp_set_state(s.ctx, at4(wl["x"]), at4(wl["v"]), at4(wl["types"].astype(np.int32)), None, None, where=A.SWP_DEVICE)
+        s.run(20, 0.001, 0.1, 1.0)
+        if shift:
+            bufs = [torch.zeros(24 * n + 16, dtype=torch.uint8, device="cuda") for _ in range(3)]
+            A.swp_read_forces(s.ctx, _At(bufs[0], 4), where=A.SWP_DEVICE)
+            A.swp_read_state(s.ctx, _At(bufs[1], 4), _At(bufs[2], 4), None, where=A.SWP_DEVICE)
+            got.append([b[4:4 + 24 * n].cpu().numpy().view(np.float64).reshape(n, 3) for b in bufs])
+        else:
+            x, v, _ = s.state()
+            got.append([s.forces(), x, v])
+    for p, q in zip(*got):
+        assert np.array_equal(p, q)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("device", [False, True])
+def test_positions_on_and_outside_the_faces(precision, device):
+    import torch
+    from paper_1912_08569_gb300 import _abi as A, SwapSystem
+
+    L = 16.0
+    below = float(np.nextafter(L, 0.0))
+    edge = [0.0, -0.0, below, L, -L, 3.25 * L, -0.5, 1e-30, 2.0 ** -48, L - 2.0 ** -49, 7.5]
+    x = np.array([[v, 0.5 + k, 15.5 - k] for k, v in enumerate(edge)])
+    s = SwapSystem(len(x), 1, [L] * 3, {}, precision=precision)
+    xs = torch.from_numpy(x).cuda() if device else x
+    s.set_state(xs)
+    got, _, img = s.state()
+    q = np.array([round((v - np.floor(v / L) * L) * 2.0 ** 48) for v in edge], dtype=object)  # exact: L is a power of two
+    im = np.array([int(np.floor(v / L)) for v in edge])
+    for k in range(len(edge)):
+        if q[k] >= 2 ** 52:
+            q[k], im[k] = q[k] - 2 ** 52, im[k] + 1
+    assert np.array_equal(got[:, 0], np.array([float(v) * 2.0 ** -48 for v in q]))
+    assert np.array_equal(img[:, 0], im)
+    assert np.array_equal(got[:, 1:], x[:, 1:])
+
+
+# r_cut = 2.4: about 26 partners inside the cut-off, more than the derivative
+# passes line up at once.  Central differences of the oracle, h = 1e-4: the
+# truncation is below 1e-4 of the derivative (FP64), FP32 terms allow 1e-3.
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-4), ("fp32", 1e-3)])
+def test_parameter_derivatives_of_long_rows(orc, precision, tol):
+    import torch
+    from paper_1912_08569_gb300 import _abi as A
+
+    wl = _wl(1501, 0.5, n=10, rcut=2.4)
+    s = make_gpu(wl, precision)
+    s.compute_forces()
+    dF = torch.empty((3, wl["n"], 3), dtype=torch.float64, device=s.device)
+    dU = A.swp_param_grad(s.ctx, 0, 1, dF)
+    h, theta = 1e-4, (1.0, 1.0, 1.0)
+    x, L = wl["x"], wl["box"]
+    d = x[None] - x[:, None]
+    d -= L * np.round(d / L)
+    r = np.sqrt((d * d).sum(-1))
+    near = (wl["types"][:, None] != wl["types"][None]) & (np.abs(r - 2.0 ** 0.1) < 4 * h)
+    keep = ~near.any(1)  # vh is only once differentiable where a partner crosses r_min
+    for k in range(3):
+        r = []
+        for sg in (1, -1):
+            p = {q: dict(v) for q, v in wl["pairs"].items()}
+            th = list(theta)
+            th[k] += sg * h
+            p[(0, 1)]["lambda3"], p[(0, 1)]["eps"], p[(0, 1)]["sigma"] = th
+            r.append(orc.forces(x, wl["types"], 2, orc.pair_table(2, p), L, fp32=precision == "fp32"))
+        fd = ((r[0]["U2"] + r[0]["U3"]) - (r[1]["U2"] + r[1]["U3"])) / (2 * h)
+        assert abs(dU[k] - fd) <= tol * (abs(fd) + 1.0)
+        ref = (r[0]["F"] - r[1]["F"])[keep] / (2 * h)
+        assert np.linalg.norm(dF[k].cpu().numpy()[keep] - ref) <= tol * np.linalg.norm(ref)
