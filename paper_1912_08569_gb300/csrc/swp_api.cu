@@ -98,6 +98,7 @@ struct swp_ctx {
     Ctl hctl;
     Ctl* mirror = nullptr;  // pinned: every launch is followed by a copy of the control block into it
     bool pending = false;   // a launch since the last wait writes to the mirror
+    bool captured = false;  // launches of this context were captured (see capturing)
     std::vector<int> cell_rank;
     std::vector<unsigned char> table_host;
     std::string err;
@@ -440,12 +441,24 @@ int map_status(swp_ctx* c)
     return SWP_OK;
 }
 
+// Whether the context's stream is being captured.  Captured work changes the
+// control block at every replay, unseen from here, and may be replayed after the
+// context is gone: it does not write to the mirror, and from then on the context's
+// synchronising calls copy the block themselves.
+bool capturing(swp_ctx* c)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+    if (st == cudaStreamCaptureStatusNone) return false;
+    c->captured = true;
+    return true;
+}
+
 // Enqueues the copy of the control block into the pinned mirror; every call that
-// changes the block ends with it, so that a synchronising call only has to wait
-// (also for replays of captured work: the copy is captured with it).
+// changes the block ends with it, so that a synchronising call only has to wait.
 int mirror_ctl(swp_ctx* c)
 {
-    if (!c->mirror) return SWP_OK;
+    if (!c->mirror || c->captured || capturing(c)) return SWP_OK;
     c->pending = true;
     SWP_CUDA(c, cudaMemcpyAsync(c->mirror, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
     return SWP_OK;
@@ -458,10 +471,10 @@ int sync_ctl(swp_ctx* c)
         SWP_CUDA(c, cudaStreamSynchronize(c->stream));
         return SWP_OK;
     }
-    if (!c->mirror)
-        SWP_CUDA(c, cudaMemcpyAsync(&c->hctl, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
+    const bool copy = !c->mirror || c->captured;
+    if (copy) SWP_CUDA(c, cudaMemcpyAsync(&c->hctl, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (c->mirror) c->hctl = *c->mirror;
+    if (!copy) c->hctl = *c->mirror;
     c->pending = false;
     return map_status(c);
 }
@@ -869,8 +882,12 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
                                  cudaMemcpyHostToDevice, c0->stream));
     SWP_CUDA(c0, launch_batch_begin<Real>(d_dev, m, c0->stream));
     SWP_CUDA(c0, launch_batch_shape<Real>(threads, d_dev, d_args, d_ofs, d_items, uni, bonds, B, c0->stream));
-    for (int r = 0; r < m; r++) cs[idx[r]]->pending = true;
-    SWP_CUDA(c0, launch_batch_end<Real>(d_dev, m, c0->stream));
+    bool end = true;
+    for (int r = 0; r < m; r++) end &= !capturing(cs[idx[r]]);
+    if (end) {
+        for (int r = 0; r < m; r++) cs[idx[r]]->pending = true;
+        SWP_CUDA(c0, launch_batch_end<Real>(d_dev, m, c0->stream));
+    }
     return SWP_OK;
 }
 

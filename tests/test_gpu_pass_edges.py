@@ -135,6 +135,34 @@ def test_unaligned_device_arrays(precision):
         assert np.array_equal(p, q)
 
 
+def test_replayed_launches_are_seen():
+    """Steps captured into a graph: every replay advances the state, and the next
+    synchronising call reports what the replays did."""
+    import torch
+
+    wl = _wl(1500, 0.4)
+    a = make_gpu(wl, "fp32")
+    a.run(10, 0.001, 0.1, 1.0)
+    a.run(10, 0.001, 0.1, 1.0)
+    a.run(10, 0.001, 0.1, 1.0)
+    st = torch.cuda.Stream()
+    from paper_1912_08569_gb300 import SwapSystem
+    b = SwapSystem(wl["n"], 2, wl["box"], wl["pairs"], precision="fp32", seed=wl.get("seed", 0), skin=wl["skin"], stream=st)
+    b.set_state(wl["x"], wl["v"], wl["types"], wl["mass"])
+    b.run(10, 0.001, 0.1, 1.0)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        b.run(10, 0.001, 0.1, 1.0, sync=False)
+    with torch.cuda.stream(st):
+        g.replay()
+    assert b.thermo()["step"] == 20
+    with torch.cuda.stream(st):
+        g.replay()
+    assert b.thermo()["step"] == 30
+    for p, q in zip(a.state(), b.state()):
+        assert np.array_equal(p, q)
+
+
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("device", [False, True])
 def test_positions_on_and_outside_the_faces(precision, device):
