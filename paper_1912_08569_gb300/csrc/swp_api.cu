@@ -569,11 +569,10 @@ int run(swp_ctx* c, RunArgs a)
     if (c->bps_req > 0) bps = std::min(bps, c->bps_req);
     bps = std::min(bps, c->max_blocks / std::max(c->num_sms, 1));
     c->grid = step_grid(c, bps);
-    // a bonded network runs the 1024-thread kernel (two-barrier step: more
-    // warps hide its global gathers; 434 against 500 us per step on the 2M-bead
-    // network), everything else the 768-thread one (the resident step where it
-    // applies; at 1M-2M unbonded particles the two shapes are within 3 %, the
-    // 768-thread one ahead)
+    // a bonded network runs the 1024-thread kernel (its bonds' chains of gathers
+    // want more warps; a 768-thread block took 500 against 434 us per step on the
+    // 2M-bead network when this was chosen), everything else the 768-thread one
+    // (FP64: 512): at 1M unbonded particles the two shapes are within 2 %
     const bool wide = !c->bond_host.empty();
     if (wide) {
         int bw = 0;

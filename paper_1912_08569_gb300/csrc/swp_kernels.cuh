@@ -1195,6 +1195,12 @@ __device__ __forceinline__ int4 load_four(const Dev<float>& d, int first, int k)
     return __ldcs((const int4*)&d.ent_j[(unsigned)first + (unsigned)k]);  // streamed: keep L2 for the snapshots
 }
 
+// The 1024-thread shapes (64 registers) gather two partners at a time and load the
+// next row's ranges late: with four at a time and the ranges held through the row
+// they spilled (2M-bead network, 10 steps 2.36 -> 2.30 ms; sweep of 96 systems, 50
+// steps 6.81 -> 6.61 ms).
+constexpr bool kLean = kThreads >= 1024;
+
 // FP32.  staged: the block has one sub-chunk and the shared copies of its
 // positions and list ranges are current (kept by the previous force pass), so
 // they are not loaded again; its S values also stay in shared memory for the
@@ -1231,7 +1237,7 @@ __device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc
         const int qn = q + kThreads;
         int4 tn = make_int4(0, 0, 0, 0);
         int in = i;
-        if (qn < b1) {
+        if (!kLean && qn < b1) {
             tn = d.tinfo[qn];
             in = d.perm[qn];
         }
@@ -1241,8 +1247,27 @@ __device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc
         for (int k = 0; k < cnt; k += 4) {
             const int4 j = jn;
             if (k + 4 < cnt) jn = load_four(d, ti.x, k + 4);
-            const int4 p0 = pos[j.x], p1 = pos[j.y], p2 = pos[j.z], p3 = pos[j.w];  // padding: the own slot
-            const float w0 = s_term<float, UNI, X>(d, tab, ps, pi, p0);
+            const int4 p0 = pos[j.x], p1 = pos[j.y];  // padding: the own slot
+            int4 p2, p3;
+            float w0;
+            if (kLean) {
+                w0 = s_term<float, UNI, X>(d, tab, ps, pi, p0);
+                const float w1 = s_term<float, UNI, X>(d, tab, ps, pi, p1);
+                p2 = pos[j.z];
+                p3 = pos[j.w];
+                const float w2 = s_term<float, UNI, X>(d, tab, ps, pi, p2);
+                if (k + 4 <= cnt) {
+                    s += (w0 + w1) + (w2 + s_term<float, UNI, X>(d, tab, ps, pi, p3));
+                } else {
+                    s += w0;
+                    if (k + 1 < cnt) s += w1;
+                    if (k + 2 < cnt) s += w2;
+                }
+                continue;
+            }
+            p2 = pos[j.z];
+            p3 = pos[j.w];
+            w0 = s_term<float, UNI, X>(d, tab, ps, pi, p0);
             if (k + 4 <= cnt) {
                 const float w1 = s_term<float, UNI, X>(d, tab, ps, pi, p1);
                 const float w2 = s_term<float, UNI, X>(d, tab, ps, pi, p2);
@@ -1257,8 +1282,8 @@ __device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc
         d.S[i] = s;
         if (single) SM::S()[t] = s;
         if (qn < b1) {
-            ti = tn;
-            i = in;
+            ti = kLean ? d.tinfo[qn] : tn;
+            i = kLean ? d.perm[qn] : in;
             pi = pos[i];
             if (ti.y > 0) jn = load_four(d, ti.x, 0);
             // the row after that, into L2
@@ -1710,7 +1735,7 @@ __device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const
             } else {
                 pi = pos[i];
                 Si = d.S[i];
-                if (qn < b1) {
+                if (!kLean && qn < b1) {
                     tn = d.tinfo[qn];
                     in = d.perm[qn];
                 }
@@ -1739,8 +1764,21 @@ __device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const
         for (int k = 0; k < ti.y; k += 4) {
             const int4 j = jn;
             if (k + 4 < ti.y) jn = load_four(d, ti.x, k + 4);
-            const int4 p0 = pos[j.x], p1 = pos[j.y], p2 = pos[j.z], p3 = pos[j.w];  // padding: the own slot
-            const float s0 = d.S[j.x], s1 = d.S[j.y], s2 = d.S[j.z], s3 = d.S[j.w];
+            const int4 p0 = pos[j.x], p1 = pos[j.y];  // padding: the own slot
+            const float s0 = d.S[j.x], s1 = d.S[j.y];
+            if (kLean) {
+                reactive(p0, s0);
+                if (k + 1 < ti.y) reactive(p1, s1);
+                if (k + 2 < ti.y) {
+                    const int4 p2 = pos[j.z], p3 = pos[j.w];
+                    const float s2 = d.S[j.z], s3 = d.S[j.w];
+                    reactive(p2, s2);
+                    if (k + 3 < ti.y) reactive(p3, s3);
+                }
+                continue;
+            }
+            const int4 p2 = pos[j.z], p3 = pos[j.w];
+            const float s2 = d.S[j.z], s3 = d.S[j.w];
             reactive(p0, s0);
             if (k + 1 < ti.y) reactive(p1, s1);
             if (k + 2 < ti.y) reactive(p2, s2);
@@ -1772,7 +1810,13 @@ __device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const
                     if (lane == q) run += (double)x;
                 }
         if (qn < b1) {
-            if (tn.y > 0) jn = load_four(d, tn.x, 0);
+            if (kLean) {
+                tn = d.tinfo[qn];
+                in = d.perm[qn];
+                prefetch_row(d, tn.x);
+            } else if (tn.y > 0) {
+                jn = load_four(d, tn.x, 0);
+            }
             if (tn.w > 0) prefetch_row(d, tn.z);
         }
         float kin = 0.0f;
@@ -1793,6 +1837,7 @@ __device__ float f_pass_rows(const Dev<float>& d, const PairP<float>* tab, const
         }
         ti = tn;
         i = in;
+        if (kLean && ti.y > 0) jn = load_four(d, ti.x, 0);
     }
     if (TH && lane < kNQA) s_wacc[t >> 5][lane] = run;
     return dmax;
