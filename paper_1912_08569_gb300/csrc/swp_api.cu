@@ -573,7 +573,11 @@ int run(swp_ctx* c, RunArgs a)
     // want more warps; a 768-thread block took 500 against 434 us per step on the
     // 2M-bead network when this was chosen), everything else the 768-thread one
     // (FP64: 512): at 1M unbonded particles the two shapes are within 2 %
-    const bool wide = !c->bond_host.empty();
+    // either; FP32 blocks of 769 to 1,024 particles are one row per thread there and
+    // two in turn for some warps here (120,000 particles x 60 steps 1501 -> 1156 us,
+    // 150,000 logged 1923 -> 1621, 131,072 dumbbells x 61 1090 -> 878)
+    const int Pb = (c->n + c->grid - 1) / c->grid;
+    const bool wide = !c->bond_host.empty() || (sizeof(Real) == 4 && Pb > kBlock && Pb <= kBlockWide);
     if (wide) {
         int bw = 0;
         SWP_CUDA(c, run_occupancy_wide<Real>(&bw));

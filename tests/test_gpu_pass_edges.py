@@ -40,8 +40,9 @@ def _check(orc, wl, precision, s):
     assert_thermo_match(s.thermo(), ref, TOL[precision], precision)
 
 
-# ten blocks: 768 (FP32) and 512 (FP64) particles fill a sub-chunk
-@pytest.mark.parametrize("precision,n", [("fp32", 7680), ("fp32", 7681), ("fp32", 15370),
+# ten blocks: 768 (FP32; up to 1,024 in the wide kernel) and 512 (FP64) particles
+# fill a sub-chunk
+@pytest.mark.parametrize("precision,n", [("fp32", 7680), ("fp32", 7681), ("fp32", 10240), ("fp32", 10241), ("fp32", 15370),
                                          ("fp64", 5120), ("fp64", 5121)])
 def test_sub_chunk_edges(orc, precision, n):
     wl = _wl(n)
