@@ -351,7 +351,8 @@ SWP_API int swp_set_timeout(swp_ctx* ctx, int64_t ns);
  * that other blocks own) with partners as local indices; a step then copies
  * the halo's new positions in once, forms S (Eq. 3bp via S_i) for its own
  * particles and the reactive halo itself, and the forces and the integrator
- * from shared memory, with one grid barrier per step instead of two.  Blocks
+ * from shared memory, the blocks following one another's published positions
+ * instead of meeting at two grid barriers.  Blocks
  * whose structures exceed the shared-memory capacity (3,072 local particles,
  * 16,384 local entries, rows of 255 entries) make the whole run fall back to
  * the two-barrier path until the next list build.  Forces and trajectories are
