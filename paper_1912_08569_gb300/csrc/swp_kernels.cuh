@@ -1468,6 +1468,8 @@ __device__ void s_pass_waves(const Dev<double>& d, const PairP<double>* tab, int
             d.S[q0 + t] = s[0];
             if (single) SM::S()[t] = s[0];
         }
+        // the staging is free (a sub-chunk without a reactive pair has run no wave)
+        if (!single) __syncthreads();
     }
 }
 

@@ -51,6 +51,23 @@ def test_sub_chunk_edges(orc, precision, n):
     _check(orc, wl, precision, s)
 
 
+# several FP64 sub-chunks per block, all or some of them without a reactive pair: the
+# S pass runs no wave of entries there, and the staging is filled again at once
+@pytest.mark.parametrize("some", [False, True])
+@pytest.mark.parametrize("n", [5121, 12_300])
+def test_sub_chunks_without_reactive_pairs(orc, n, some):
+    wl = _wl(n)
+    wl["n_types"] = 3
+    wca = wl["pairs"][(0, 0)]
+    wl["types"] = np.where(wl["x"][:, 0] < (0.3 if some else 0.0) * wl["box"][0], wl["types"], 2).astype(np.int32)
+    wl["pairs"] = {k: wl["pairs"].get(k, wca) for k in ((0, 0), (0, 1), (0, 2), (1, 1), (1, 2), (2, 2))}
+    if not some:
+        wl["pairs"][(0, 1)] = wca
+    s = make_gpu(wl, "fp64")
+    s.set_grid(10)
+    _check(orc, wl, "fp64", s)
+
+
 # r_cut = 2.4: about 34 reactive and 3 other partners, more than a lane of the
 # build holds; on ten blocks of 300 FP64 particles several waves of entries
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
