@@ -385,6 +385,26 @@ int refresh_layout(swp_ctx* c)
     return SWP_OK;
 }
 
+// A new cell grid on a bound workspace: the arrays from the cell list on move, the
+// grid's order is uploaded, and the counts that every list build expects to be
+// zero (k_set_state, or the build before) are cleared where they are now.
+template <typename Real>
+int move_cells_of(swp_ctx* c, const Dev<Real>& d)
+{
+    SWP_CUDA(c, cudaMemcpyAsync((void*)d.cell_rank, c->cell_rank.data(), sizeof(int) * 2 * c->ncell,
+                                cudaMemcpyHostToDevice, c->stream));
+    SWP_CUDA(c, cudaMemsetAsync(d.cell_cnt, 0, sizeof(int) * c->ncell, c->stream));
+    SWP_CUDA(c, cudaMemsetAsync(d.bsum, 0, sizeof(int) * d.nbsum, c->stream));
+    return SWP_OK;
+}
+
+int move_cells(swp_ctx* c)
+{
+    const int rc = refresh_layout(c);
+    if (rc) return rc;
+    return c->precision == SWP_FP64 ? move_cells_of(c, c->dd) : move_cells_of(c, c->df);
+}
+
 Ctl* dev_ctl(swp_ctx* c) { return c->precision == SWP_FP64 ? c->dd.ctl : c->df.ctl; }
 
 int upload_table(swp_ctx* c)
@@ -980,10 +1000,8 @@ int swp_set_pair(swp_ctx* c, int ti, int tj, int kind, double eps, double sigma,
             c->state_set = false;
             return fail(c, SWP_ERR_STATE, "cell grid grew: workspace too small, bind a larger one");
         }
-        refresh_layout(c);
-        SWP_CUDA(c, cudaMemcpyAsync((void*)(c->precision == SWP_FP64 ? c->dd.cell_rank : c->df.cell_rank),
-                                    c->cell_rank.data(), sizeof(int) * 2 * c->ncell,
-                                    cudaMemcpyHostToDevice, c->stream));
+        rc = move_cells(c);
+        if (rc) return rc;
     }
     return mark_stale(c);
 }
@@ -1042,10 +1060,8 @@ int swp_set_nlist(swp_ctx* c, double skin, int max_nn)
             c->state_set = false;
             return fail(c, SWP_ERR_STATE, "cell grid grew: workspace too small, bind a larger one");
         }
-        refresh_layout(c);
-        SWP_CUDA(c, cudaMemcpyAsync((void*)(c->precision == SWP_FP64 ? c->dd.cell_rank : c->df.cell_rank),
-                                    c->cell_rank.data(), sizeof(int) * 2 * c->ncell,
-                                    cudaMemcpyHostToDevice, c->stream));
+        rc = move_cells(c);
+        if (rc) return rc;
     }
     return mark_stale(c);
 }

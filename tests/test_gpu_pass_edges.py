@@ -111,6 +111,26 @@ def test_resident_equals_two_barrier_path_at_the_ends(n, density):
         np.testing.assert_allclose(logs[0][k], logs[1][k], rtol=1e-5)
 
 
+# r_cut and the skin move the cell grid, and with it the arrays of the list build
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_a_new_cell_grid_on_a_live_state(orc, precision):
+    from paper_1912_08569_gb300 import _abi as A
+
+    wl = _wl(4000, 0.4)
+    s = make_gpu(wl, precision)
+    s.run(20, 0.001, 0.1, 1.0)
+    for rcut, skin in ((2.0, 0.3), (1.5, 0.3), (1.5, 0.6), (1.3, 0.5)):  # (more cells than at first need a larger workspace)
+        wl["pairs"] = inputs.swap_pairs(lambda3=1.0, rcut=rcut)
+        for (ti, tj), p in wl["pairs"].items():
+            A.swp_set_pair(s.ctx, ti, tj, p["kind"], p["eps"], p["sigma"], p["n"], p.get("rcut", 0.0),
+                           p.get("lambda3", 0.0), p.get("shift", 0), p.get("rbond", 0.0))
+        s.skin = skin
+        A.swp_set_nlist(s.ctx, skin, s.max_nn)
+        s.run(5, 0.001, 0.1, 1.0)
+        wl["x"] = s.state()[0]
+        _check(orc, wl, precision, s)
+
+
 class _At:
     """A device address inside a buffer, as the binding takes it."""
 
