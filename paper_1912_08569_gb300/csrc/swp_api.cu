@@ -96,9 +96,8 @@ struct swp_ctx {
     Dev<float> df;
     Dev<double> dd;
     Ctl hctl;
-    Ctl* mirror = nullptr;  // pinned: every launch is followed by a copy of the control block into it
-    bool pending = false;   // a launch since the last wait writes to the mirror
-    bool captured = false;  // launches of this context were captured (see capturing)
+    bool ctl_known = false;  // hctl is the control block after everything enqueued so far
+    bool captured = false;   // launches of this context were captured (see ctl_changes)
     std::vector<int> cell_rank;
     std::vector<unsigned char> table_host;
     std::string err;
@@ -294,7 +293,6 @@ size_t layout(swp_ctx* c, char* base, Dev<Real>* d)
         d->partials = partials;
         d->ctl = ctl;
         d->agree = ctl ? ctl->agree : nullptr;
-        d->mirror = c->mirror;
         d->io = io;
         d->io_int = io_int;
         d->table = table;
@@ -433,7 +431,7 @@ int ready(swp_ctx* c, bool need_state)
     return SWP_OK;
 }
 
-int mirror_ctl(swp_ctx* c);
+void ctl_changes(swp_ctx* c);
 
 int map_status(swp_ctx* c)
 {
@@ -448,11 +446,10 @@ int map_status(swp_ctx* c)
     if (s & kStatusNonfinite) return fail(c, SWP_ERR_NONFINITE, "non-finite force; set the state again");
     if (s & kStatusOverflow) {
         cudaError_t e = cudaSuccess;
+        ctl_changes(c);
         k_clear_status_bits<<<1, 1, 0, c->stream>>>(dev_ctl(c), kStatusOverflow);
         e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(c, e, "clear status");
-        const int rc = mirror_ctl(c);
-        if (rc) return rc;
         char buf[160];
         std::snprintf(buf, sizeof buf, "neighbour row of %d entries exceeds max_nn = %d",
                       c->hctl.max_row, c->max_nn);
@@ -461,27 +458,15 @@ int map_status(swp_ctx* c)
     return SWP_OK;
 }
 
-// Whether the context's stream is being captured.  Captured work changes the
-// control block at every replay, unseen from here, and may be replayed after the
-// context is gone: it does not write to the mirror, and from then on the context's
-// synchronising calls copy the block themselves.
-bool capturing(swp_ctx* c)
+// Comes before everything that enqueues a change of the control block: the host
+// copy is out of date until the next wait.  Captured work changes the block at every
+// replay, unseen from here: from then on every wait copies it.
+void ctl_changes(swp_ctx* c)
 {
+    c->ctl_known = false;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
-    if (st == cudaStreamCaptureStatusNone) return false;
-    c->captured = true;
-    return true;
-}
-
-// Enqueues the copy of the control block into the pinned mirror; every call that
-// changes the block ends with it, so that a synchronising call only has to wait.
-int mirror_ctl(swp_ctx* c)
-{
-    if (!c->mirror || c->captured || capturing(c)) return SWP_OK;
-    c->pending = true;
-    SWP_CUDA(c, cudaMemcpyAsync(c->mirror, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
-    return SWP_OK;
+    if (st != cudaStreamCaptureStatusNone) c->captured = true;
 }
 
 // Waits for the stream and refreshes the host copy of the control block.
@@ -491,11 +476,12 @@ int sync_ctl(swp_ctx* c)
         SWP_CUDA(c, cudaStreamSynchronize(c->stream));
         return SWP_OK;
     }
-    const bool copy = !c->mirror || c->captured;
-    if (copy) SWP_CUDA(c, cudaMemcpyAsync(&c->hctl, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
+    if (!c->ctl_known || c->captured) {
+        c->ctl_known = false;
+        SWP_CUDA(c, cudaMemcpyAsync(&c->hctl, dev_ctl(c), sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
+    }
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
-    if (!copy) c->hctl = *c->mirror;
-    c->pending = false;
+    c->ctl_known = true;
     return map_status(c);
 }
 
@@ -616,11 +602,12 @@ int run(swp_ctx* c, RunArgs a)
     a.withhold = c->withhold;
     a.tlog_every = d.tlog ? c->tlog_every : 0;
     c->withhold = 0;  // one launch consumes the request
+    ctl_changes(c);
     // the agreement words and the barrier counter, the control block's first
     SWP_CUDA(c, cudaMemsetAsync(d.ctl, 0, offsetof(Ctl, barrier) + sizeof(unsigned long long), c->stream));
     if (wide) SWP_CUDA(c, launch_run_wide<Real>(d, a, c->grid, c->stream));
     else SWP_CUDA(c, launch_run<Real>(d, a, c->grid, block, c->stream));
-    return mirror_ctl(c);
+    return SWP_OK;
 }
 
 int run_any(swp_ctx* c, RunArgs a)
@@ -631,9 +618,10 @@ int run_any(swp_ctx* c, RunArgs a)
 int mark_stale(swp_ctx* c)
 {
     if (!c->ws_bound || !c->state_set || c->n == 0) return SWP_OK;
+    ctl_changes(c);
     k_mark_stale<<<1, 1, 0, c->stream>>>(dev_ctl(c));
     SWP_CUDA(c, cudaGetLastError());
-    return mirror_ctl(c);
+    return SWP_OK;
 }
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p & (a - 1)) == 0; }
@@ -903,14 +891,9 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
                                  c0->stream));
     SWP_CUDA(c0, cudaMemcpyAsync(d_items, plan.items.data(), sizeof(int4) * plan.items.size(),
                                  cudaMemcpyHostToDevice, c0->stream));
+    for (int r = 0; r < m; r++) ctl_changes(cs[idx[r]]);
     SWP_CUDA(c0, launch_batch_begin<Real>(d_dev, m, c0->stream));
     SWP_CUDA(c0, launch_batch_shape<Real>(threads, d_dev, d_args, d_ofs, d_items, uni, bonds, B, c0->stream));
-    bool end = true;
-    for (int r = 0; r < m; r++) end &= !capturing(cs[idx[r]]);
-    if (end) {
-        for (int r = 0; r < m; r++) cs[idx[r]]->pending = true;
-        SWP_CUDA(c0, launch_batch_end<Real>(d_dev, m, c0->stream));
-    }
     return SWP_OK;
 }
 
@@ -1091,10 +1074,6 @@ int swp_bind_workspace(swp_ctx* c, void* ptr, size_t bytes, void* stream)
     c->ws_bound = true;
     c->state_set = false;
     c->table_dirty = true;
-    if (!c->mirror && cudaHostAlloc((void**)&c->mirror, sizeof(Ctl), cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();  // (during stream capture, say): synchronising calls copy the block themselves
-        c->mirror = nullptr;
-    }
     refresh_layout(c);
     SWP_CUDA(c, cudaMemcpyAsync((void*)(c->precision == SWP_FP64 ? c->dd.cell_rank : c->df.cell_rank),
                                 c->cell_rank.data(), sizeof(int) * 2 * c->ncell, cudaMemcpyHostToDevice,
@@ -1140,6 +1119,7 @@ int swp_set_state(swp_ctx* c, const double* x, const double* v, const int32_t* t
     std::memset(&c->hctl, 0, sizeof(Ctl));
     c->hctl.state = 1;
     c->hctl.need_rebuild = 1;
+    ctl_changes(c);
     SWP_CUDA(c, cudaMemsetAsync(dev_ctl(c), 0, sizeof(Ctl), c->stream));
     c->state_set = true;
     if (n == 0) return SWP_OK;
@@ -1162,7 +1142,7 @@ int swp_set_state(swp_ctx* c, const double* x, const double* v, const int32_t* t
     }
     if (c->precision == SWP_FP64) SWP_CUDA(c, launch_set_state<double>(c->dd, x, v, ty, mass, im, c->stream));
     else SWP_CUDA(c, launch_set_state<float>(c->df, x, v, ty, mass, im, c->stream));
-    return mirror_ctl(c);
+    return SWP_OK;
 }
 
 int swp_set_step(swp_ctx* c, int64_t step)
@@ -1173,10 +1153,10 @@ int swp_set_step(swp_ctx* c, int64_t step)
     if (c->n == 0) return SWP_OK;
     static_assert(sizeof(long long) == sizeof(int64_t), "step width");
     long long s = (long long)step;
+    ctl_changes(c);
     SWP_CUDA(c, cudaMemcpyAsync(&dev_ctl(c)->step, &s, sizeof(s), cudaMemcpyHostToDevice, c->stream));
-    const int rm = mirror_ctl(c);
     SWP_CUDA(c, cudaStreamSynchronize(c->stream));
-    return rm;
+    return SWP_OK;
 }
 
 int swp_build_nlist(swp_ctx* c)
@@ -1408,6 +1388,7 @@ int swp_eval_grad(swp_ctx* c, int ti, int tj, const double* theta_dev, const dou
     const double c_rmin = std::pow(2.0, 1.0 / p.n), c_rb = std::pow((1.0 - std::sqrt(0.5)) / 2.0, -1.0 / p.n);
     const bool f64 = c->precision == SWP_FP64;
     double* io = f64 ? c->dd.io : c->df.io;
+    ctl_changes(c);
     if (f64) SWP_CUDA(c, launch_eval_prep<double>(c->dd, ti, tj, theta_dev, c_rmin, c_rb, p.rbond, c->stream));
     else SWP_CUDA(c, launch_eval_prep<float>(c->df, ti, tj, theta_dev, c_rmin, c_rb, p.rbond, c->stream));
     c->state_set = true;
@@ -1553,9 +1534,8 @@ int swp_set_thermo_log(swp_ctx* c, int every, int64_t capacity, void* ring, size
     c->df.tlog_cap = c->dd.tlog_cap = cap;
     c->tlog_every = every;
     if (c->ws_bound) {
+        ctl_changes(c);
         SWP_CUDA(c, cudaMemsetAsync(&dev_ctl(c)->tlog_n, 0, sizeof(long long), c->stream));
-        const int rm = mirror_ctl(c);
-        if (rm) return rm;
     }
     return SWP_OK;
 }
@@ -1593,18 +1573,6 @@ const char* swp_last_error(const swp_ctx* c) { return c ? c->err.c_str() : "null
 
 int swp_destroy(swp_ctx* c)
 {
-    if (c && c->mirror) {
-        // launches that nobody waited for may still write to it (the stream
-        // itself may be gone by now)
-        int dev = -1;
-        if (c->pending && cudaGetDevice(&dev) == cudaSuccess) {
-            if (dev != c->device) cudaSetDevice(c->device);
-            cudaDeviceSynchronize();
-            if (dev != c->device) cudaSetDevice(dev);
-        }
-        cudaFreeHost(c->mirror);
-        cudaGetLastError();  // (the process may be ending)
-    }
     delete c;
     return SWP_OK;
 }

@@ -159,7 +159,6 @@ struct Dev {
     double* partials;  // [max_blocks][kNQ]
     Ctl* ctl;
     unsigned long long* agree;  // resident steps: ctl->agree
-    Ctl* mirror;     // pinned host memory: the control block after the last launch (null: none)
     double* io;        // host-exchange staging: [3n] x, [3n] v, [n] mass
     int* io_int;       // staging: [n] types, [3n] images
     const PairP<Real>* table;  // [ntypes * ntypes]
@@ -253,8 +252,6 @@ template <typename Real>
 cudaError_t launch_get_forces(const Dev<Real>& d, int pc, double* f, double* U, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_batch_begin(const Dev<Real>* devs, int m, cudaStream_t s);
-template <typename Real>
-cudaError_t launch_batch_end(const Dev<Real>* devs, int m, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_get_nlist(const Dev<Real>& d, int pc, int* rows, int* counts, int width,
                              cudaStream_t s);

@@ -3741,19 +3741,6 @@ __global__ void k_batch_begin(const Dev<Real>* devs, int m)
     if (r < m) devs[r].ctl->barrier = 0;
 }
 
-// After it: every system's control block into its mirror in host memory (one
-// warp per system), so that the systems' next synchronising calls need no copy
-// of their own (96 systems: one launch for 96 copies of 8 us).
-template <typename Real>
-__global__ void k_batch_end(const Dev<Real>* devs, int m)
-{
-    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (r >= m || !devs[r].mirror) return;
-    const int* src = (const int*)devs[r].ctl;
-    int* dst = (int*)devs[r].mirror;
-    for (int k = lane; k < (int)(sizeof(Ctl) / sizeof(int)); k += 32) dst[k] = src[k];
-}
-
 #endif  // SWP_HAS_RESIDENT
 
 }  // namespace single / wide / SWP_BATCH_NS

@@ -201,6 +201,49 @@ def test_replayed_launches_are_seen():
         assert np.array_equal(p, q)
 
 
+def test_binding_another_workspace_and_stream():
+    """Work that is still waiting on the stream bound before changes nothing of
+    what the calls on the new binding report."""
+    import torch
+    from paper_1912_08569_gb300 import _abi as A
+
+    wl = _wl(1500, 0.4)
+    a = make_gpu(wl, "fp32")
+    a.run(30, 0.001, 0.1, 1.0)
+    s = make_gpu(wl, "fp32", stream=torch.cuda.Stream())
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s.stream):
+        torch.cuda._sleep(1_000_000_000)  # about half a second
+    s.run(7, 0.001, 0.1, 1.0, sync=False)
+    ws, nl, st = torch.empty_like(s.workspace), torch.empty_like(s.nlist_buf), torch.cuda.Stream()
+    A.swp_bind_workspace(s.ctx, ws.data_ptr(), ws.numel(), st.cuda_stream)
+    A.swp_bind_nlist(s.ctx, nl.data_ptr(), nl.numel())
+    s.set_state(wl["x"], wl["v"], wl["types"], wl["mass"])
+    s.run(30, 0.001, 0.1, 1.0)
+    first = s.state()
+    torch.cuda.synchronize()  # the seven steps on the old binding, too
+    assert s.thermo()["step"] == 30
+    for p, q, r in zip(a.state(), first, s.state()):
+        assert np.array_equal(p, q) and np.array_equal(p, r)
+
+
+def test_destroying_a_context_is_host_work():
+    """A context may go while another stream is captured and its own work still runs."""
+    import torch
+
+    wl = _wl(1500, 0.4)
+    s = make_gpu(wl, "fp32", stream=torch.cuda.Stream())
+    s.run(7, 0.001, 0.1, 1.0, sync=False)
+    y = torch.zeros(8, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        y += 1.0
+        s.close()
+    g.replay()
+    torch.cuda.synchronize()
+    assert y.tolist() == [1.0] * 8
+
+
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("device", [False, True])
 def test_positions_on_and_outside_the_faces(precision, device):
