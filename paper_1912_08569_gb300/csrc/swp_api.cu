@@ -5,10 +5,12 @@
 #include "swapmd.h"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <mutex>
 #include <string>
 #include <utility>
 #include <type_traits>
@@ -98,6 +100,7 @@ struct swp_ctx {
     Ctl hctl;
     bool ctl_known = false;  // hctl is the control block after everything enqueued so far
     bool captured = false;   // launches of this context were captured (see ctl_changes)
+    int slot = -1;           // its place in g_slots: a batched launch returns the control block there
     std::vector<int> cell_rank;
     std::vector<unsigned char> table_host;
     std::string err;
@@ -293,6 +296,8 @@ size_t layout(swp_ctx* c, char* base, Dev<Real>* d)
         d->partials = partials;
         d->ctl = ctl;
         d->agree = ctl ? ctl->agree : nullptr;
+        d->slot = nullptr;  // (set per batched launch)
+        d->ticket = 0;
         d->io = io;
         d->io_int = io_int;
         d->table = table;
@@ -458,12 +463,79 @@ int map_status(swp_ctx* c)
     return SWP_OK;
 }
 
+// Pinned places into which a batched launch returns its systems' control blocks
+// (one kernel, k_batch_end, for a copy of 7 us per system: 50 steps of 96 systems and
+// their read-outs 7275 -> 6617 us).  A context holds a place from such a launch until
+// its next wait or change; the launch may still be running when the place is let
+// go (the context destroyed, bound to another stream), so a place is given out again
+// only once the ticket of its last launch has arrived in it.  Any thread; without a
+// place left the block is copied like everybody's.
+struct Slots {
+    static constexpr int kCount = 512;  // 128 KB, kept until the process ends
+    std::mutex lock;
+    CtlSlot* at = nullptr;
+    bool tried = false;
+    int last = 0;
+    unsigned long long next = 0, want[kCount] = {};
+    bool held[kCount] = {}, open[kCount] = {};  // given out; let go before its launch was seen to end
+
+    bool arrived(int k) const { return ((const volatile CtlSlot*)at)[k].ticket == want[k]; }
+
+    int take()
+    {
+        std::lock_guard<std::mutex> g(lock);
+        if (!tried) {
+            tried = true;
+            // the allocation must not disturb a capture that goes on elsewhere
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            void* p = nullptr;
+            if (cudaHostAlloc(&p, sizeof(CtlSlot) * kCount, cudaHostAllocPortable) == cudaSuccess) {
+                std::memset(p, 0, sizeof(CtlSlot) * kCount);
+                at = (CtlSlot*)p;
+            } else {
+                cudaGetLastError();
+            }
+            cudaThreadExchangeStreamCaptureMode(&mode);
+        }
+        for (int i = 0; at && i < kCount; i++) {
+            const int k = (last + i) % kCount;
+            if (held[k] || (open[k] && !arrived(k))) continue;
+            held[k] = true;
+            want[k] = ++next;
+            last = k + 1;
+            return k;
+        }
+        return -1;
+    }
+
+    void give_back(int k, bool ended)
+    {
+        std::lock_guard<std::mutex> g(lock);
+        held[k] = false;
+        open[k] = !ended;
+    }
+};
+
+Slots& slots()
+{
+    static Slots* s = new Slots();  // (contexts may outlive static objects)
+    return *s;
+}
+
+void let_go(swp_ctx* c, bool ended = false)
+{
+    if (c->slot >= 0) slots().give_back(c->slot, ended);
+    c->slot = -1;
+}
+
 // Comes before everything that enqueues a change of the control block: the host
 // copy is out of date until the next wait.  Captured work changes the block at every
 // replay, unseen from here: from then on every wait copies it.
 void ctl_changes(swp_ctx* c)
 {
     c->ctl_known = false;
+    let_go(c);
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
     if (st != cudaStreamCaptureStatusNone) c->captured = true;
@@ -475,6 +547,16 @@ int sync_ctl(swp_ctx* c)
     if (c->n == 0 || !c->state_set) {
         SWP_CUDA(c, cudaStreamSynchronize(c->stream));
         return SWP_OK;
+    }
+    if (c->slot >= 0) {
+        SWP_CUDA(c, cudaStreamSynchronize(c->stream));
+        if (slots().arrived(c->slot)) {
+            std::atomic_thread_fence(std::memory_order_acquire);
+            c->hctl = slots().at[c->slot].ctl;
+            c->ctl_known = true;
+        }
+        let_go(c, c->ctl_known);
+        if (c->ctl_known) return map_status(c);
     }
     if (!c->ctl_known || c->captured) {
         c->ctl_known = false;
@@ -879,6 +961,14 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
     for (int k = 0; k < B; k++)
         for (int it = plan.item_ofs[k]; it < plan.item_ofs[k + 1]; it++)
             cs[idx[plan.items[it].x]]->grid = plan.items[it].z;
+    for (int r = 0; r < m; r++) ctl_changes(cs[idx[r]]);
+    for (int r = 0; r < m && !c0->captured; r++) {
+        swp_ctx* c = cs[idx[r]];
+        c->slot = slots().take();
+        if (c->slot < 0) break;
+        devs[r].slot = &slots().at[c->slot];
+        devs[r].ticket = slots().want[c->slot];
+    }
     char* base = (char*)ws;
     Dev<Real>* d_dev = (Dev<Real>*)base;
     RunArgs* d_args = (RunArgs*)(base + align256(sizeof(Dev<Real>) * m));
@@ -891,9 +981,9 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
                                  c0->stream));
     SWP_CUDA(c0, cudaMemcpyAsync(d_items, plan.items.data(), sizeof(int4) * plan.items.size(),
                                  cudaMemcpyHostToDevice, c0->stream));
-    for (int r = 0; r < m; r++) ctl_changes(cs[idx[r]]);
     SWP_CUDA(c0, launch_batch_begin<Real>(d_dev, m, c0->stream));
     SWP_CUDA(c0, launch_batch_shape<Real>(threads, d_dev, d_args, d_ofs, d_items, uni, bonds, B, c0->stream));
+    if (cs[idx[0]]->slot >= 0) SWP_CUDA(c0, launch_batch_end<Real>(d_dev, m, c0->stream));
     return SWP_OK;
 }
 
@@ -1074,6 +1164,7 @@ int swp_bind_workspace(swp_ctx* c, void* ptr, size_t bytes, void* stream)
     c->ws_bound = true;
     c->state_set = false;
     c->table_dirty = true;
+    let_go(c);
     refresh_layout(c);
     SWP_CUDA(c, cudaMemcpyAsync((void*)(c->precision == SWP_FP64 ? c->dd.cell_rank : c->df.cell_rank),
                                 c->cell_rank.data(), sizeof(int) * 2 * c->ncell, cudaMemcpyHostToDevice,
@@ -1573,6 +1664,7 @@ const char* swp_last_error(const swp_ctx* c) { return c ? c->err.c_str() : "null
 
 int swp_destroy(swp_ctx* c)
 {
+    if (c) let_go(c);
     delete c;
     return SWP_OK;
 }

@@ -115,6 +115,12 @@ struct PosVec<double> {
     typedef dbl4 type;
 };
 
+// A control block returned to pinned host memory, then the launch's ticket.
+struct alignas(256) CtlSlot {
+    Ctl ctl;
+    unsigned long long ticket;
+};
+
 // Pointers and sizes of one context's device state (passed by value).
 template <typename Real>
 struct Dev {
@@ -159,6 +165,8 @@ struct Dev {
     double* partials;  // [max_blocks][kNQ]
     Ctl* ctl;
     unsigned long long* agree;  // resident steps: ctl->agree
+    CtlSlot* slot;   // pinned host memory that a batched launch returns the control block to (null: none)
+    unsigned long long ticket;  // and what marks it as this launch's
     double* io;        // host-exchange staging: [3n] x, [3n] v, [n] mass
     int* io_int;       // staging: [n] types, [3n] images
     const PairP<Real>* table;  // [ntypes * ntypes]
@@ -252,6 +260,8 @@ template <typename Real>
 cudaError_t launch_get_forces(const Dev<Real>& d, int pc, double* f, double* U, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_batch_begin(const Dev<Real>* devs, int m, cudaStream_t s);
+template <typename Real>
+cudaError_t launch_batch_end(const Dev<Real>* devs, int m, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_get_nlist(const Dev<Real>& d, int pc, int* rows, int* counts, int width,
                              cudaStream_t s);

@@ -3741,6 +3741,21 @@ __global__ void k_batch_begin(const Dev<Real>* devs, int m)
     if (r < m) devs[r].ctl->barrier = 0;
 }
 
+// After it: the control blocks of the systems that hold a place in pinned memory,
+// one warp per system, the ticket last.
+template <typename Real>
+__global__ void k_batch_end(const Dev<Real>* devs, int m)
+{
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (r >= m || !devs[r].slot) return;
+    const int* src = (const int*)devs[r].ctl;
+    int* dst = (int*)&devs[r].slot->ctl;
+    for (int k = lane; k < (int)(sizeof(Ctl) / sizeof(int)); k += 32) dst[k] = src[k];
+    __syncwarp();
+    __threadfence_system();
+    if (lane == 0) *(volatile unsigned long long*)&devs[r].slot->ticket = devs[r].ticket;
+}
+
 #endif  // SWP_HAS_RESIDENT
 
 }  // namespace single / wide / SWP_BATCH_NS

@@ -110,6 +110,13 @@ cudaError_t launch_batch_begin(const Dev<Real>* devs, int m, cudaStream_t s)
 }
 
 template <typename Real>
+cudaError_t launch_batch_end(const Dev<Real>* devs, int m, cudaStream_t s)
+{
+    single::k_batch_end<Real><<<(m + 7) / 8, 256, 0, s>>>(devs, m);
+    return cudaGetLastError();
+}
+
+template <typename Real>
 cudaError_t launch_get_nlist(const Dev<Real>& d, int pc, int* rows, int* counts, int width,
                              cudaStream_t s)
 {
@@ -156,6 +163,7 @@ cudaError_t launch_eval_prep(const Dev<Real>& d, int ti, int tj, const double* t
     template cudaError_t launch_get_state<R>(const Dev<R>&, int, int, double*, double*, int*, cudaStream_t); \
     template cudaError_t launch_get_forces<R>(const Dev<R>&, int, double*, double*, cudaStream_t); \
     template cudaError_t launch_batch_begin<R>(const Dev<R>*, int, cudaStream_t);                \
+    template cudaError_t launch_batch_end<R>(const Dev<R>*, int, cudaStream_t);                  \
     template cudaError_t launch_get_nlist<R>(const Dev<R>&, int, int*, int*, int, cudaStream_t); \
     SWP_BATCH_DEFINE(R)                                                                          \
     template cudaError_t launch_param_grad<R>(const Dev<R>&, int, int, double*, double*, const double*, double*, \

@@ -192,3 +192,50 @@ def test_batch_rejects_missing_block_shape():
         with pytest.raises(A.SwpError) as e:
             SwapBatch(systems, threads=threads).run(1, 0.001, 0.1, 1.0)
         assert e.value.code == A.SWP_ERR_INVALID
+
+
+def test_batch_control_blocks_come_back_to_their_own_contexts():
+    """More systems than there are pinned places for control blocks, contexts
+    destroyed and bound elsewhere while a batch still runs, and batches after that:
+    every system reports its own steps."""
+    import torch
+    from paper_1912_08569_gb300 import SwapBatch, SwapSystem
+    from paper_1912_08569_gb300 import _abi as A
+
+    st = torch.cuda.Stream()
+    wl = inputs.workload("mix2k", n=90, density=0.2, seed=3)
+
+    def make(count, stream):
+        out = []
+        for k in range(count):
+            s = SwapSystem(wl["n"], 2, wl["box"], wl["pairs"], seed=k, stream=stream)
+            s.set_state(wl["x"], wl["v"], wl["types"])
+            out.append(s)
+        return out
+
+    many, few, other = make(520, st), make(40, st), torch.cuda.Stream()
+    SwapBatch(many).run(3, 0.001, 0.1, 1.0)
+    assert [s.thermo()["step"] for s in many] == [3] * len(many)
+    moved = many[40]
+    ws, nl = torch.empty_like(moved.workspace), torch.empty_like(moved.nlist_buf)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        torch.cuda._sleep(1_000_000_000)  # about half a second
+    b = SwapBatch(many)
+    b.run(4, 0.001, 0.1, 1.0, sync=False)  # waits behind it
+    keep = [(s.workspace, s.nlist_buf) for s in many]
+    for s in many[:40]:
+        s.close()
+    A.swp_bind_workspace(moved.ctx, ws.data_ptr(), ws.numel(), other.cuda_stream)
+    A.swp_bind_nlist(moved.ctx, nl.data_ptr(), nl.numel())
+    moved.set_state(wl["x"], wl["v"], wl["types"])
+    moved.run(2, 0.001, 0.1, 1.0)
+    assert moved.thermo()["step"] == 2
+    SwapBatch(few).run(9, 0.001, 0.1, 1.0)
+    torch.cuda.synchronize()
+    assert moved.thermo()["step"] == 2
+    assert [s.thermo()["step"] for s in few] == [9] * len(few)
+    assert [s.thermo()["step"] for s in many[41:]] == [7] * len(many[41:])
+    SwapBatch(many[41:]).run(1, 0.001, 0.1, 1.0)
+    assert [s.thermo()["step"] for s in many[41:]] == [8] * len(many[41:])
+    del keep
