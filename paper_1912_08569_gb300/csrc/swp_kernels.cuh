@@ -1295,6 +1295,7 @@ __device__ void s_pass_rows(const Dev<float>& d, const PairP<float>* tab, int pc
 // ---------------------------------------------------------------------------
 // FP64 waves.
 
+static __shared__ int s_int[64];
 static __shared__ int s_nlist;  // entries lined up
 static __shared__ int s_nkeep;  // reactive pairs whose values the S pass kept (-1: not kept)
 
@@ -1346,17 +1347,25 @@ __device__ __forceinline__ double dist2_near(const dbl4& pi, const dbl4& pj, con
 }
 
 // Lines up the entries [e0, e1) that may lie inside their cut-off behind the
-// entries already in the list (any order: results go to the entries' places),
-// zeroes the wave's results of the others, and (react) of the lined-up ones
-// too.  nres: results per entry (1 or 3).  The caller's barrier completes it.
+// entries already in the list and zeroes the wave's results of the others.
+// ordered: in entry order, so that the energies, which thread c of the evaluation
+// adds up for the c-th entries, are the same in every run (a block barrier every
+// kThreads entries); else as the warps come, which changes no force: results go to
+// the entries' places.  The force pass orders its entries on sampled steps, the S
+// pass, whose list the force pass goes on with, always (as the warps come there
+// too: 2,000 particles x 100 logged steps 1865 us, energies that did not repeat; this
+// way 1888, with a test of the step's kind in the S pass 1900).  nres: results per entry (1
+// or 3).  The caller's barriers come before and complete it.
 template <bool UNI>
 __device__ __forceinline__ void line_up(const Dev<double>& d, const PairP<double>* tab, const PairP<double>& pu,
-                                        const dbl4* pos, unsigned wb, unsigned e0, unsigned e1, int nres)
+                                        const dbl4* pos, unsigned wb, unsigned e0, unsigned e1, int nres, bool ordered)
 {
     typedef Stage<double> SM;
-    const int lane = threadIdx.x & 31;
-    for (unsigned eb = e0 + (threadIdx.x & ~31u); eb < e1; eb += kThreads) {  // the same in the whole warp
-        const unsigned e = eb + lane;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int placed = ordered ? s_nlist : 0, buf = 0;
+    // the same in the whole warp (ordered: block)
+    for (unsigned eb = e0 + (ordered ? 0u : threadIdx.x & ~31u); eb < e1; eb += kThreads) {
+        const unsigned e = eb + (ordered ? threadIdx.x : lane);
         bool in = false;
         int j = 0, o = 0;
         if (e < e1) {
@@ -1370,10 +1379,20 @@ __device__ __forceinline__ void line_up(const Dev<double>& d, const PairP<double
         }
         const unsigned m = __ballot_sync(0xffffffffu, in);
         int base = 0;
-        if (lane == 0 && m) base = atomicAdd(&s_nlist, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
+        if (ordered) {
+            if (lane == 0) s_int[buf + warp] = __popc(m);
+            __syncthreads();
+            const int c = lane < kThreads / 32 ? s_int[buf + lane] : 0;
+            base = placed + __reduce_add_sync(0xffffffffu, lane < warp ? c : 0);
+            placed += __reduce_add_sync(0xffffffffu, c);
+            buf ^= 32;
+        } else {
+            if (lane == 0 && m) base = atomicAdd(&s_nlist, __popc(m));
+            base = __shfl_sync(0xffffffffu, base, 0);
+        }
         if (in) SM::list()[base + __popc(m & ((1u << lane) - 1u))] = make_int2((int)(e - wb) | o << 16, j);
     }
+    if (ordered && e0 < e1 && threadIdx.x == 0) s_nlist = placed;
 }
 
 // Adds the results at w[k - wb] of entries [k0, k1) to f in entry order.  Zeros
@@ -1430,7 +1449,7 @@ __device__ void s_pass_waves(const Dev<double>& d, const PairP<double>* tab, int
         double s[1] = {0.0};
         for (unsigned wb = e_beg; wb < e_end; wb += SM::kWave) {
             const unsigned we = min(wb + SM::kWave, e_end);
-            line_up<UNI>(d, tab, ps, pos, wb, wb, we, 1);
+            line_up<UNI>(d, tab, ps, pos, wb, wb, we, 1, true);
             __syncthreads();
             const int m = s_nlist;
             const bool kept = keep && m <= SM::kKeep;
@@ -1923,7 +1942,7 @@ __device__ float f_pass_waves(const Dev<double>& d, const PairP<double>* tab, co
             const unsigned wr = min(max(e_rend, wb), we);  // reactive entries before, others from here
             int nre = nkeep;  // reactive pairs in the list
             if (nkeep < 0) {
-                line_up<UNI>(d, tab, ps, pos, wb, wb, wr, 3);
+                line_up<UNI>(d, tab, ps, pos, wb, wb, wr, 3, TH);
                 __syncthreads();
                 nre = s_nlist;
                 __syncthreads();
@@ -1937,7 +1956,7 @@ __device__ float f_pass_waves(const Dev<double>& d, const PairP<double>* tab, co
                     SM::w()[2 * SM::kWave + (e - wb)] = 0.0;
                 }
             }
-            line_up<UNI>(d, tab, pw, pos, wb, wr, we, 3);
+            line_up<UNI>(d, tab, pw, pos, wb, wr, we, 3, TH);
             __syncthreads();
             const int m = s_nlist;
             for (int c = t; c < m; c += kThreads) {
@@ -2074,7 +2093,6 @@ struct LoopState {
 
 static __shared__ __align__(16) unsigned char s_tab_raw[kMaxTypes * kMaxTypes * sizeof(PairP<double>)];
 static __shared__ double s_red[32];
-static __shared__ int s_int[64];
 static __shared__ LoopState s_ls;
 
 template <typename Real>

@@ -111,6 +111,28 @@ def test_resident_equals_two_barrier_path_at_the_ends(n, density):
         np.testing.assert_allclose(logs[0][k], logs[1][k], rtol=1e-5)
 
 
+# the energies of equal runs are the same bits (the wave of an FP64 block is lined
+# up by 16 warps): forces and a logged run, blocks of one wave, of several, of
+# several sub-chunks
+@pytest.mark.parametrize("n,grid", [(3000, 0), (3000, 10), (5300, 10)])
+def test_fp64_energies_repeat(n, grid):
+    wl = _wl(n, 0.5)
+    first = None
+    for _ in range(12):
+        s = make_gpu(wl, "fp64")
+        s.set_grid(grid)
+        s.compute_forces()
+        th = s.thermo()
+        s.set_thermo_log(1, 6)
+        s.run(6, 0.001, 0.1, 1.0)
+        log = s.thermo_log()
+        got = [th["U2"], th["U3"], th["W"], *(log[k] for k in ("U2", "U3", "K", "W"))]
+        if first is None:
+            first = got
+        for p, q in zip(first, got):
+            assert np.array_equal(p, q)
+
+
 # r_cut and the skin move the cell grid, and with it the arrays of the list build
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 def test_a_new_cell_grid_on_a_live_state(orc, precision):
