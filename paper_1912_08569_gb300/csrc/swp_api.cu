@@ -1742,6 +1742,15 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
     h.state = 1;
     h.need_rebuild = 1;
     SWP_CUDA(c, cudaMemcpyAsync(d.ctl, &h, sizeof(h), cudaMemcpyHostToDevice, s));
+    // kernels read and write aligned arrays only; others pass through the staging area
+    if (!aligned(x, 8)) {
+        SWP_CUDA(c, cudaMemcpyAsync(d.io, x, sizeof(double) * 3 * c->n, cudaMemcpyDeviceToDevice, s));
+        x = d.io;
+    }
+    if (!aligned(type, 4)) {
+        SWP_CUDA(c, cudaMemcpyAsync(d.io_int, type, sizeof(int) * c->n, cudaMemcpyDeviceToDevice, s));
+        type = d.io_int;
+    }
     SWP_CUDA(c, launch_set_state<Real>(d, x, nullptr, type, nullptr, nullptr, s));
 
     int bps = 0;
@@ -1768,7 +1777,9 @@ int static_forces(swp_ctx* c, const double* x, const int32_t* type, double* f, d
                       c->max_nn);
         return fail(c, SWP_ERR_NLIST_OVERFLOW, buf);
     }
-    SWP_CUDA(c, launch_get_forces<Real>(d, h.pos_cur, f, nullptr, s));
+    double* out = aligned(f, 8) ? f : d.io;
+    SWP_CUDA(c, launch_get_forces<Real>(d, h.pos_cur, out, nullptr, s));
+    if (out != f) SWP_CUDA(c, cudaMemcpyAsync(f, out, sizeof(double) * 3 * c->n, cudaMemcpyDeviceToDevice, s));
     if (thermo) {
         // [U2, U3, W xx yy zz xy xz yz, n_bonds]
         SWP_CUDA(c, cudaMemcpyAsync(thermo, &d.ctl->thermo[Q_U2], 2 * sizeof(double),

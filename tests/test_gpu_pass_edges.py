@@ -195,6 +195,30 @@ def test_unaligned_device_arrays(precision):
         assert np.array_equal(p, q)
 
 
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_unaligned_arrays_of_the_static_call(precision):
+    import torch
+    from paper_1912_08569_gb300 import _abi as A
+
+    wl = _wl(800, 0.3)
+    n = wl["n"]
+    s = make_gpu(wl, precision)
+    x, ty = torch.from_numpy(wl["x"]).cuda(), torch.from_numpy(wl["types"].astype(np.int32)).cuda()
+    f = torch.zeros((n, 3), dtype=torch.float64, device="cuda")
+    A.swp_compute_forces_static(s.ctx, x, ty, f, None, 0)
+
+    def at(t, off):
+        raw = t.contiguous().view(torch.uint8).reshape(-1)
+        buf = torch.zeros(raw.numel() + 16, dtype=torch.uint8, device="cuda")
+        buf[off:off + raw.numel()] = raw
+        return _At(buf, off)
+
+    out = at(torch.zeros_like(f), 4)
+    A.swp_compute_forces_static(s.ctx, at(x, 4), at(ty, 2), out, None, 0)
+    assert torch.equal(out.buf[4:4 + 24 * n].clone().view(torch.float64).view(n, 3), f)
+    assert not out.buf[:4].any() and not out.buf[4 + 24 * n:].any()
+
+
 def test_replayed_launches_are_seen():
     """Steps captured into a graph: every replay advances the state, and the next
     synchronising call reports what the replays did."""
