@@ -151,7 +151,9 @@ SWP_API int swp_bind_nlist(swp_ctx* ctx, void* device_ptr, size_t bytes);
 /* Set the state in user order: x [n][3] (any real numbers: wrapped into the
  * box, the wraps added to img), v [n][3] (NULL: zero), type [n] (NULL: all 0),
  * mass [n] (> 0; NULL: all 1), img [n][3] (NULL: zero).  All pointers are of
- * kind `where`.  Resets the step counter to 0.  Forces become stale. */
+ * kind `where`.  Resets the step counter to 0.  Forces become stale.  Host
+ * arrays may be reused when the call returns (under stream capture, pinned ones
+ * only once the graph's work is done); device arrays are read in stream order. */
 SWP_API int swp_set_state(swp_ctx* ctx, const double* x, const double* v, const int32_t* type,
                   const double* mass, const int32_t* img, int where);
 

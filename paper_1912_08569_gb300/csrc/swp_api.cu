@@ -529,6 +529,13 @@ void let_go(swp_ctx* c, bool ended = false)
     c->slot = -1;
 }
 
+bool capturing(const swp_ctx* c)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // Comes before everything that enqueues a change of the control block: the host
 // copy is out of date until the next wait.  Captured work changes the block at every
 // replay, unseen from here: from then on every wait copies it.
@@ -536,9 +543,7 @@ void ctl_changes(swp_ctx* c)
 {
     c->ctl_known = false;
     let_go(c);
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) cudaGetLastError();
-    if (st != cudaStreamCaptureStatusNone) c->captured = true;
+    if (capturing(c)) c->captured = true;
 }
 
 // Waits for the stream and refreshes the host copy of the control block.
@@ -1230,6 +1235,8 @@ int swp_set_state(swp_ctx* c, const double* x, const double* v, const int32_t* t
         SWP_CUDA(c, stage(io + 6 * n, mass, n));
         SWP_CUDA(c, stage(io_int, ty, n));
         SWP_CUDA(c, stage(io_int + n, im, 3 * n));
+        // the caller may reuse its arrays (pageable ones have been read by now in any case)
+        if (where == SWP_HOST && !capturing(c)) SWP_CUDA(c, cudaStreamSynchronize(c->stream));
     }
     if (c->precision == SWP_FP64) SWP_CUDA(c, launch_set_state<double>(c->dd, x, v, ty, mass, im, c->stream));
     else SWP_CUDA(c, launch_set_state<float>(c->df, x, v, ty, mass, im, c->stream));

@@ -247,6 +247,26 @@ def test_replayed_launches_are_seen():
         assert np.array_equal(p, q)
 
 
+@pytest.mark.parametrize("masses", [False, True])
+def test_host_arrays_may_be_reused_when_the_call_returns(masses):
+    """Pinned arrays, and work ahead on the stream."""
+    import torch
+    from paper_1912_08569_gb300 import _abi as A
+
+    wl = _wl(1500, 0.4)
+    s = make_gpu(wl, "fp32", stream=torch.cuda.Stream())
+    torch.cuda.synchronize()
+    want = s.state()[:2]
+    pinned = [torch.from_numpy(np.ascontiguousarray(wl[k])).pin_memory() for k in ("x", "v", "types", "mass")]
+    with torch.cuda.stream(s.stream):
+        torch.cuda._sleep(300_000_000)
+    A.swp_set_state(s.ctx, pinned[0], pinned[1], pinned[2], pinned[3] if masses else None, None, where=A.SWP_HOST)
+    for t in pinned:
+        t.zero_()
+    for p, q in zip(want, s.state()):
+        assert np.array_equal(p, q)
+
+
 def test_binding_another_workspace_and_stream():
     """Work that is still waiting on the stream bound before changes nothing of
     what the calls on the new binding report."""
