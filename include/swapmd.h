@@ -130,7 +130,9 @@ SWP_API int swp_set_pair(swp_ctx* ctx, int ti, int tj, int kind, double eps, dou
  * particle on average over each block's particles (a single row may be
  * longer).  Call before swp_nlist_size / swp_bind_nlist.
  * The box must hold >= 3 cells of edge max(cut-off) + skin per dimension:
- * SWP_ERR_INVALID otherwise. */
+ * SWP_ERR_INVALID otherwise.  The list's entries, (n + 2 x SMs) x max_nn (FP32: max_nn
+ * + 6 rounded up to a multiple of four), must stay below 2^32 - 2^16: this call,
+ * swp_nlist_size and swp_bind_nlist return SWP_ERR_INVALID otherwise. */
 SWP_API int swp_set_nlist(swp_ctx* ctx, double skin, int max_nn);
 
 /* Bytes of device workspace this context needs (state, cell list, staging). */

@@ -201,6 +201,19 @@ size_t list_particles(const swp_ctx* c) { return (size_t)std::max(c->n, 1) + c->
 
 size_t list_entries(const swp_ctx* c) { return list_particles(c) * list_stride(c); }
 
+// Entry positions are unsigned 32-bit numbers; the loops over them step past the
+// last one by a wave at most.
+constexpr size_t kMaxEntries = ((size_t)1 << 32) - ((size_t)1 << 16);
+
+int check_entries(swp_ctx* c)
+{
+    if (list_entries(c) <= kMaxEntries) return SWP_OK;
+    char buf[160];
+    std::snprintf(buf, sizeof buf, "%d particles at max_nn = %d need %zu list entries; the limit is %zu", c->n, c->max_nn,
+                  list_entries(c), kMaxEntries);
+    return fail(c, SWP_ERR_INVALID, buf);
+}
+
 size_t list_bytes(const swp_ctx* c)
 {
     return align256(list_entries(c) * 4) +
@@ -1122,7 +1135,8 @@ int swp_set_nlist(swp_ctx* c, double skin, int max_nn)
     int old_nn = c->max_nn;
     c->skin = skin;
     c->max_nn = max_nn;
-    int rc = derive_cells(c);
+    int rc = check_entries(c);
+    if (!rc) rc = derive_cells(c);
     if (rc) {
         c->skin = old_skin;
         c->max_nn = old_nn;
@@ -1155,7 +1169,7 @@ int swp_nlist_size(const swp_ctx* c, size_t* bytes)
 {
     if (!c || !bytes) return SWP_ERR_INVALID;
     *bytes = list_bytes(c);
-    return SWP_OK;
+    return check_entries(const_cast<swp_ctx*>(c));
 }
 
 int swp_bind_workspace(swp_ctx* c, void* ptr, size_t bytes, void* stream)
@@ -1181,7 +1195,8 @@ int swp_bind_nlist(swp_ctx* c, void* ptr, size_t bytes)
 {
     if (!c) return SWP_ERR_INVALID;
     size_t need = 0;
-    swp_nlist_size(c, &need);
+    const int rc = swp_nlist_size(c, &need);
+    if (rc) return rc;
     if (!ptr || ((uintptr_t)ptr & 255)) return fail(c, SWP_ERR_INVALID, "list buffer must be 256-byte aligned");
     if (bytes < need) return fail(c, SWP_ERR_INVALID, "neighbour-list buffer too small");
     c->nl = ptr;

@@ -1443,9 +1443,9 @@ __device__ void s_pass_waves(const Dev<double>& d, const PairP<double>* tab, int
         __syncthreads();
         const int4 inf = SM::info()[min(t, P - 1)];
         const int4 last = SM::info()[P - 1];
-        const unsigned e_beg = SM::info()[0].x, e_end = (unsigned)(last.x + last.y);
+        const unsigned e_beg = SM::info()[0].x, e_end = (unsigned)last.x + (unsigned)last.y;
         // the values are kept for the force pass when it takes the same wave
-        const bool keep = single && (unsigned)(last.z + last.w) - e_beg <= (unsigned)SM::kWave;
+        const bool keep = single && (unsigned)last.z + (unsigned)last.w - e_beg <= (unsigned)SM::kWave;
         double s[1] = {0.0};
         for (unsigned wb = e_beg; wb < e_end; wb += SM::kWave) {
             const unsigned we = min(wb + SM::kWave, e_end);
@@ -1935,7 +1935,7 @@ __device__ float f_pass_waves(const Dev<double>& d, const PairP<double>* tab, co
         __syncthreads();
         const int4 inf = SM::info()[min(t, P - 1)];
         const int4 last = SM::info()[P - 1];
-        const unsigned e_beg = SM::info()[0].x, e_rend = (unsigned)(last.x + last.y), e_end = (unsigned)(last.z + last.w);
+        const unsigned e_beg = SM::info()[0].x, e_rend = (unsigned)last.x + (unsigned)last.y, e_end = (unsigned)last.z + (unsigned)last.w;
         double f[3] = {0.0, 0.0, 0.0}, g[3] = {0.0, 0.0, 0.0};  // reactive and other rows' sums
         for (unsigned wb = e_beg; wb < e_end; wb += SM::kWave) {
             const unsigned we = min(wb + SM::kWave, e_end);
@@ -3492,9 +3492,9 @@ __global__ void k_get_nlist(Dev<Real> d, int pc, int* rows, int* counts, int wid
         int* out = rows + (size_t)tag * width;
         int k = 0;
         for (int m = 0; m < inf.y && k < width; m++, k++)
-            out[k] = pos_bits(d.pos[pc][d.ent_j[(unsigned)(inf.x + m)]]) >> kTypeBits;
+            out[k] = pos_bits(d.pos[pc][d.ent_j[(unsigned)inf.x + m]]) >> kTypeBits;
         for (int m = 0; m < inf.w && k < width; m++, k++)
-            out[k] = pos_bits(d.pos[pc][d.ent_j[(unsigned)(inf.z + m)]]) >> kTypeBits;
+            out[k] = pos_bits(d.pos[pc][d.ent_j[(unsigned)inf.z + m]]) >> kTypeBits;
     }
 }
 
@@ -3567,7 +3567,7 @@ __device__ __forceinline__ void pg_partners(const Dev<Real>& d, const typename D
             int j[4];
             P4 pj[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) j[u] = k + u < inf.y ? d.ent_j[(unsigned)(inf.x + k + u)] : -1;
+            for (int u = 0; u < 4; u++) j[u] = k + u < inf.y ? d.ent_j[(unsigned)inf.x + k + u] : -1;
 #pragma unroll
             for (int u = 0; u < 4; u++) pj[u] = pos[max(j[u], 0)];
 #pragma unroll

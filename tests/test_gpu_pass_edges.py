@@ -133,6 +133,30 @@ def test_fp64_energies_repeat(n, grid):
             assert np.array_equal(p, q)
 
 
+# list positions are unsigned 32-bit numbers; host calls only, no buffer of that size.
+# FP32 rows take max_nn + 6 entries rounded up to a multiple of four
+@pytest.mark.parametrize("precision,max_nn,stride", [("fp32", 64, 72), ("fp32", 4096, 4104), ("fp64", 64, 64),
+                                                     ("fp64", 4096, 4096)])
+def test_lists_beyond_32_bit_positions_are_refused(precision, max_nn, stride):
+    import torch
+    from paper_1912_08569_gb300 import _abi as A
+
+    blocks = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    limit = (2 ** 32 - 2 ** 16) // stride - min(blocks, 320)
+    code = A.SWP_FP64 if precision == "fp64" else A.SWP_FP32
+    for n, fits in ((limit, True), (limit + 1, False)):
+        ctx = A.swp_create(n, 1, [50.0] * 3, code, 0)
+        A.swp_set_nlist(ctx, 0.3, 8)
+        if fits:
+            A.swp_set_nlist(ctx, 0.3, max_nn)
+            assert A.swp_nlist_size(ctx) >= 4 * stride * n
+        else:
+            with pytest.raises(A.SwpError, match="list entries"):
+                A.swp_set_nlist(ctx, 0.3, max_nn)
+            assert A.swp_nlist_size(ctx) < 4 * 24 * (n + 1000)  # as before the refused call
+        A.swp_destroy(ctx)
+
+
 # r_cut and the skin move the cell grid, and with it the arrays of the list build
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 def test_a_new_cell_grid_on_a_live_state(orc, precision):
