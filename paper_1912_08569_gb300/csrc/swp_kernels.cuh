@@ -2185,10 +2185,12 @@ __device__ __forceinline__ void run_s_pass(const Dev<Real>& d, const RunArgs& a,
 }
 
 // Folds a thread's squared displacement into the block's shared maximum (one
-// shared atomic per warp); the barrier arrival publishes it.
+// shared atomic per warp); the barrier arrival publishes it.  A NaN (a particle
+// whose velocity is none) counts for nothing, so that the others' lists are still
+// rebuilt in time; the bits of the other values order like them.
 __device__ __forceinline__ void warp_max_disp(float v)
 {
-    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(v));  // (v >= 0: the bits order like the values)
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(v, 0.0f)));
     if ((threadIdx.x & 31) == 0 && m) atomicMax(&s_ls.dmax_bits, m);
 }
 

@@ -177,6 +177,29 @@ def test_a_new_cell_grid_on_a_live_state(orc, precision):
         _check(orc, wl, precision, s)
 
 
+def test_a_velocity_that_is_no_number_leaves_the_others_lists_alone():
+    """Device arrays are not looked through: one NaN velocity, a system dilute enough
+    that its particle meets nobody, and the list builds the others ask for."""
+    import torch
+
+    n = 2000
+    wl = _wl(n, 0.02, seed=9)
+    wl["v"] = inputs.maxwell_velocities(n, 4.0, 1.0, seed=8)
+    wl["v"][700] = np.nan
+    got = []
+    for resident in (True, False):
+        s = make_gpu(wl | dict(v=None), "fp32")
+        s.set_state(*(torch.from_numpy(wl[k]).cuda() for k in ("x", "v", "types")))
+        s.set_resident(resident)
+        s.run(60, 0.005, 0.0, 0.0)
+        th = s.thermo()
+        assert th["resident_steps"] == (60 if resident else 0)
+        got.append((th["n_rebuilds"], *s.state()))
+    assert got[0][0] == got[1][0] > 2
+    for p, q in zip(got[0][1:], got[1][1:]):
+        assert np.array_equal(p, q, equal_nan=p.dtype.kind == "f")
+
+
 class _At:
     """A device address inside a buffer, as the binding takes it."""
 
