@@ -200,6 +200,31 @@ def test_a_velocity_that_is_no_number_leaves_the_others_lists_alone():
         assert np.array_equal(p, q, equal_nan=p.dtype.kind == "f")
 
 
+def test_a_halo_that_does_not_fit_costs_little():
+    """r_cut = 3.3: a block's second halo shell has more particles than the halo's table
+    has places.  The two-barrier path takes over, and finding that out takes no longer
+    than the steps themselves (bound: three times the run without the attempt)."""
+    import torch
+
+    wl = _wl(50_000, 0.4, n=10, rcut=3.3)
+    got, ms = [], []
+    for resident in (False, True):
+        s = make_gpu(wl, "fp32")
+        s.set_resident(resident)
+        s.run(5, 0.001, 0.05, 1.0)
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record(s.stream)
+        s.run(30, 0.001, 0.05, 1.0)
+        e1.record(s.stream)
+        torch.cuda.synchronize()
+        ms.append(e0.elapsed_time(e1))
+        assert s.thermo()["resident_steps"] == 0
+        got.append(s.state())
+    for p, q in zip(*got):
+        assert np.array_equal(p, q)
+    assert ms[1] < 3.0 * ms[0], ms
+
+
 class _At:
     """A device address inside a buffer, as the binding takes it."""
 
