@@ -55,7 +55,7 @@ struct PairP {
 
 // Device-side control block (one per context, in the workspace).
 struct alignas(16) Ctl {
-    unsigned long long agree[4]; // resident steps' agreement, two 16-byte words (see r_post; zeroed before each launch)
+    unsigned long long agree[4]; // resident steps' agreement, two pairs of words (see r_post; zeroed before each launch)
     unsigned long long barrier;  // grid-barrier arrival counter (zeroed before each launch)
     int status;                  // latched SWP_* error bits (see kStatus*)
     int state;                   // 0: full step, forces valid; 1: forces invalid; 2: mid-step

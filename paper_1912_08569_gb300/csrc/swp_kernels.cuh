@@ -2322,18 +2322,25 @@ __device__ __forceinline__ void add_disp(Ctl* ctl, long long stp)
 // step (its parity over the writes of that buffer), and the blocks that hold
 // the particle in their halo read it until the bit is the expected one.  What
 // all blocks have to agree on, the displacement bound that asks for a list
-// build, comes along late: one warp posts the block's largest displacement and
-// its arrival, and waits for every block's while the others read the halo and
-// work on S and the forces; the step is thrown away before the integrator if
-// the list turns out to have to be rebuilt first.  A block posts publication k
-// after it has read its halo of publication k - 1, and writes publication k + 1
-// (into the buffer of k - 1) once all have posted k, so no snapshot is
-// overwritten early.
-// The posts are relaxed atomics on one cell of each of two 16-byte words in
-// turn: an agreement of 152 blocks that way takes 1,790 cycles, with release and
-// acquire 2,550, and with a slot per block that every block reads 6,100 (with
-// fences 9,500): the readers crowd the lines that are being written.  With a
-// grid barrier per step (arrival, poll, then the halo copies, nine block
+// build, comes along late: one thread posts the block's largest displacement and
+// its arrival once the block has read its halo, and waits for every block's while
+// the others work on S and the forces; the step is thrown away before the integrator
+// if the list turns out to have to be rebuilt first.
+//
+// The order of the accesses.  A snapshot is a relaxed 16-byte store and load of one
+// size and place, and carries its own step.  A block posts publication k after it has
+// read its halo of k, and writes publication k + 1 (into the buffer of k - 1) once it
+// has seen all post k.  The arrival is a release add, after a block barrier that all
+// the block's reads come before, and the wait ends with an acquire fence ahead of
+// the block barrier that all its writes come after: every read of publication k - 1
+// happens before the write over it, and the maximum is read after every block's part
+// of it.  (Posted ahead of the halo, whose reads then ran beside it, the release waited
+// for the block's own stores on their way out: 512 particles x 64 steps 386 us, 4,099 x
+// 100 769, 100,000 x 100 logged 1,541; behind it 368, 721, 1,465; relaxed throughout and
+// ahead of the halo, without the order above being promised, 380, 757, 1,500.  A slot
+// per block that every block reads took three times as long as one counter: the
+// readers crowd the lines that are being written.)
+// With a grid barrier per step (arrival, poll, then the halo copies, nine block
 // barriers in all) a step of 512 particles took 7.3 us (6.2 this way, 4.1 with
 // the branch-free powers of pair_power), one of 100,000 14.8 (14.2, 12.4).
 
@@ -2789,28 +2796,29 @@ struct Patience {
 __device__ __forceinline__ unsigned r_bit(int k) { return ((unsigned)(((k - 1) >> 1) & 1) ^ 1u) << 31; }
 
 // Post and agreement of publication e = 1, 2, ... of a launch (one thread of the
-// block).  The word of e's parity: (arrivals, (publication, largest squared
-// displacement)); the second only grows, so neither is ever reset.  The
-// arrival is added after the maximum has come back.
+// block).  The words of e's parity: arrivals, and (publication, largest squared
+// displacement); both only grow, so neither is ever reset.
 __device__ __forceinline__ void r_post(const Dev<float>& d, unsigned e)
 {
     unsigned long long* w = d.agree + 2 * (e & 1);
     const unsigned long long mine = (unsigned long long)e << 32 | s_ls.dmax_bits;
     s_ls.dmax_bits = 0u;
-    unsigned long long old;
-    asm volatile("atom.relaxed.gpu.global.max.u64 %0, [%1], %2;" : "=l"(old) : "l"(w + 1), "l"(mine) : "memory");
-    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"(old == ~0ull ? 0ull : 1ull) : "memory");
+    asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(w + 1), "l"(mine) : "memory");
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"(1ull) : "memory");
 }
 
 __device__ __forceinline__ void r_agree(const Dev<float>& d, const RunArgs& a, unsigned e)
 {
-    const int4* w = (const int4*)(d.agree + 2 * (e & 1));
+    const unsigned long long* w = d.agree + 2 * (e & 1);
     const unsigned long long want = (unsigned long long)((e + 1) / 2) * (unsigned)g_size();
     Patience wait;
     for (;;) {
-        const int4 v = ld_snapshot(w);
-        if (((unsigned long long)(unsigned)v.y << 32 | (unsigned)v.x) >= want) {
-            s_ls.disp += sqrtf(__int_as_float(v.z));
+        unsigned long long n, m;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(n) : "l"(w) : "memory");
+        if (n >= want) {
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(m) : "l"(w + 1) : "memory");
+            s_ls.disp += sqrtf(__uint_as_float((unsigned)m));
             return;
         }
         if (!wait.more(d.ctl, a.timeout_ns, 22)) {
@@ -2915,7 +2923,7 @@ template <bool UNI, int X>
 static __device__ int r_run(const Dev<float>& d, const RunArgs& a)
 {
     typedef RStage RS;
-    const int t = threadIdx.x, B = blockDim.x, warp = t >> 5, last_warp = (B >> 5) - 1;
+    const int t = threadIdx.x, B = blockDim.x;
     const int P = s_ls.r_np, H = s_ls.r_nh, RB = s_ls.r_rb;
     const int NQ = (P + s_ls.r_nhr + RB - 1) / RB * RB;  // positions of the rows of S
     const bool spare = RB < B;                           // the last warp has no rows
@@ -2933,10 +2941,6 @@ static __device__ int r_run(const Dev<float>& d, const RunArgs& a)
     int result = 0;
     for (;;) {
         const bool more = remaining > 1, logged = tl_left == 1, th = !more || logged;
-        if (spare && k > 0 && warp == last_warp) {
-            asm volatile("bar.sync 2, %0;" ::"r"(B) : "memory");  // every row warp's maximum is in
-            if (t == B - 32) r_post(d, epoch);
-        }
         // the halo's snapshots (complete at the first step)
         const int4* pos = d.pos[pc];
         const unsigned bit = r_bit(k), care = k > 0 ? 0x80000000u : 0u;
@@ -2977,8 +2981,10 @@ static __device__ int r_run(const Dev<float>& d, const RunArgs& a)
             if (w1) v1 = ld_snapshot(&pos[hslot[h + 3 * RB]]);
         }
         if (!__syncthreads_and(ok)) break;
-        if (spare && k > 0 && t == B - 32) r_agree(d, a, epoch);
-        if (!spare && k > 0 && t == B - 32) r_post(d, epoch);
+        if (k > 0 && t == B - 32) {
+            r_post(d, epoch);
+            if (spare) r_agree(d, a, epoch);
+        }
         int4 fd = make_int4(0, 0, 0, -1);
         float fx = 0.0f, fy = 0.0f, fz = 0.0f;
         if (t < RB) {
@@ -3065,10 +3071,7 @@ static __device__ int r_run(const Dev<float>& d, const RunArgs& a)
             result = 1;
             break;
         }
-        if (t < RB) {
-            warp_max_disp(dmax);
-            if (spare) asm volatile("bar.arrive 2, %0;" ::"r"(B) : "memory");
-        }
+        if (t < RB) warp_max_disp(dmax);
         k++;
         epoch++;
         pc ^= 1;
