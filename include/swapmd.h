@@ -416,7 +416,9 @@ SWP_API int swp_compute_forces_static(swp_ctx* ctx, const double* x_dev, const i
 
 SWP_API const char* swp_last_error(const swp_ctx* ctx);
 
-/* Free the context (not the caller's device buffers). NULL is accepted. */
+/* Free the context (not the caller's device buffers). NULL is accepted.  Host
+ * work only: launches of the context may still run, on buffers that have to stay
+ * until they end. */
 SWP_API int swp_destroy(swp_ctx* ctx);
 
 #ifdef __cplusplus

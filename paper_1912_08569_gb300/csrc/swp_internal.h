@@ -15,7 +15,7 @@ constexpr int kBlock = 768;        // threads per block of the FP32 step kernel 
 constexpr int kBlock64 = 512;      // of the FP64 step kernel
 constexpr int kMaxGrid = 320;      // largest grid of the step kernel (blocks)
 constexpr int kBlockBatch = 1024;  // threads per block of the batched kernel
-constexpr int kBlockWide = 1024;   // threads per block of the step kernel of bonded networks
+constexpr int kBlockWide = 1024;   // of the step kernel of bonded networks and of FP32 blocks of 769 to 1,024 particles
 constexpr int kMaxBonds = 4;       // harmonic bonds per particle (chains: 2)
 constexpr int kMaxTag = (1 << 27); // tags must fit in 27 bits (sign bit stays clear)
 
@@ -158,7 +158,7 @@ struct Dev {
                            // then rank -> linear index
     int* cell_cnt;     // [ncell]
     int* cell_start;   // [ncell + 1]
-    int* cell_fill;    // [ncell]
+    int* cell_fill;    // [ncell + n] fill counters, then the cells' members
     int* perm;         // [n] new slot -> old slot while the list is built; then (FP32) the particle of every thread
     int* bsum;         // [nbsum] particles in each block's chunk of cells (list build)
     int nbsum;         // max_blocks

@@ -33,9 +33,10 @@
 
 // With SWP_BATCHED 0 and SWP_WIDE 1 it is compiled into namespace swp::wide:
 // the single-system step kernel with 1024-thread blocks (two-barrier step
-// only), which bonded networks run: their gathers' latency is hidden better
-// with more warps.  That copy leaves out the resident step and the exchange
-// kernels.
+// only), which bonded networks run, whose gathers' latency is hidden better
+// with more warps, and unbonded FP32 systems of 769 to 1,024 particles per block,
+// which are one row per thread there.  That copy leaves out the resident step and
+// the exchange kernels.
 #undef SWP_HAS_RESIDENT
 #if !SWP_BATCHED && !SWP_WIDE
 #define SWP_HAS_RESIDENT 1
@@ -72,7 +73,8 @@ constexpr bool kBatched = SWP_BATCHED != 0;
 // single-system kernel runs 768 threads in FP32 (80 registers: its resident step
 // keeps a thread's row, the integrator's state and the pair arithmetic in
 // registers at once) and 512 in FP64 (128 registers: eight warps fill the FP64
-// pipe, and spills cost more than more warps bring).
+// pipe, and spills cost more than more warps bring).  FP64 batches and networks
+// exist with 1,024 threads only.
 #if SWP_BATCHED
 constexpr int kThreads = SWP_BATCH_THREADS;
 constexpr int kMinBlocks = SWP_BATCH_MINB;
@@ -104,13 +106,6 @@ __device__ __forceinline__ long long gtimer_ns()
     long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
-}
-
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p)
-{
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
 }
 
 __device__ __forceinline__ int ld_relaxed(const int* p)
@@ -386,22 +381,6 @@ __device__ __forceinline__ void normals3(unsigned long long seed, long long step
     z[2] = rb * cospi(2.0 * u3);
 }
 
-template <int LANES>
-__device__ __forceinline__ unsigned group_mask()
-{
-    if (LANES == 32) return 0xffffffffu;
-    unsigned lw = threadIdx.x & 31;
-    return ((1u << (LANES & 31)) - 1u) << (lw & ~(unsigned)(LANES - 1));
-}
-
-template <int LANES, typename T>
-__device__ __forceinline__ T group_sum(T v, unsigned mask)
-{
-#pragma unroll
-    for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o, LANES);
-    return v;
-}
-
 // ---------------------------------------------------------------------------
 // Grid barrier for the cooperative launch: split arrive / wait, every wait
 // bounded in time; on expiry the status word gets kStatusTimeout and every
@@ -614,20 +593,6 @@ __device__ __forceinline__ void block_sums_from_threads(const double* stage, int
         }
     }
     __syncthreads();
-}
-
-__device__ __forceinline__ int block_max_int(int v, int* sh)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if (lane == 0) sh[warp] = v;
-    __syncthreads();
-    int m = 0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < nw; w++) m = max(m, sh[w]);
-    __syncthreads();
-    return m;  // valid in thread 0
 }
 
 // Exclusive scan of one int per thread over the block (block 0 only).
@@ -1709,7 +1674,7 @@ __device__ __forceinline__ void bond_forces(const Dev<Real>& d, const typename D
 }
 
 // Where the S pass of the same step left the block's positions, list ranges and
-// S values in shared memory (one sub-chunk or unit per warp), they are taken
+// S values in shared memory (a block of one sub-chunk), they are taken
 // from there, and the integrator keeps the shared positions current for the
 // next S pass.  TH: the sampled step (the warps' thermo terms are left in
 // s_wacc, see block_sums_from_rows).  Returns the thread's largest squared
@@ -2083,7 +2048,6 @@ struct LoopState {
     int r_rb;            // threads that hold rows
     unsigned r_epoch;    // publications of this launch
     int r_round;         // agreement round (selects ctl->rfail[round & 1])
-    int r_fail;          // this block's structures do not fit
     int r_np, r_nh, r_nhr;  // own particles, halo particles, halo rows of S
     int r_steps;         // steps this launch took in the resident mode
     int tlog_left;       // steps up to and including the next logged one (0: no log)
@@ -2153,7 +2117,7 @@ __device__ SWP_COLD int run_rebuild(const Dev<Real>& d, const RunArgs& a)
     return 0;
 }
 
-// At most one unit per warp: the block's particles fit one shared staging.
+// One sub-chunk: the block's particles fit one shared staging.
 template <typename Real>
 __device__ __forceinline__ bool single_chunk(const Dev<Real>& d)
 {
@@ -3153,7 +3117,6 @@ __device__ __forceinline__ bool run_system(const Dev<Real>& d, const RunArgs& a)
         s_ls.r_epoch = 0;
         s_ls.ok = 1;
         s_ls.r_round = 0;
-        s_ls.r_fail = 0;
         s_ls.r_np = s_ls.r_nh = s_ls.r_nhr = 0;
         s_ls.r_steps = 0;
         s_ls.tlog_left = 0;
