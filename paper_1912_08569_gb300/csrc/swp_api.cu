@@ -990,10 +990,13 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
         for (int it = plan.item_ofs[k]; it < plan.item_ofs[k + 1]; it++)
             cs[idx[plan.items[it].x]]->grid = plan.items[it].z;
     for (int r = 0; r < m; r++) ctl_changes(cs[idx[r]]);
-    for (int r = 0; r < m && !c0->captured; r++) {
+    bool end = false;
+    for (int r = 0; r < m; r++) {
         swp_ctx* c = cs[idx[r]];
+        if (c->captured) continue;  // (replays would change the block behind the place's back)
         c->slot = slots().take();
         if (c->slot < 0) break;
+        end = true;
         devs[r].slot = &slots().at[c->slot];
         devs[r].ticket = slots().want[c->slot];
     }
@@ -1011,7 +1014,7 @@ int batch_run(swp_ctx* const* cs, const std::vector<int>& idx, std::vector<RunAr
                                  cudaMemcpyHostToDevice, c0->stream));
     SWP_CUDA(c0, launch_batch_begin<Real>(d_dev, m, c0->stream));
     SWP_CUDA(c0, launch_batch_shape<Real>(threads, d_dev, d_args, d_ofs, d_items, uni, bonds, B, c0->stream));
-    if (cs[idx[0]]->slot >= 0) SWP_CUDA(c0, launch_batch_end<Real>(d_dev, m, c0->stream));
+    if (end) SWP_CUDA(c0, launch_batch_end<Real>(d_dev, m, c0->stream));
     return SWP_OK;
 }
 

@@ -319,6 +319,26 @@ def test_replayed_launches_are_seen():
         assert np.array_equal(p, q)
 
 
+def test_replays_after_a_batch_are_seen():
+    """A system whose steps were captured takes part in a batch; a replay after that
+    changes its state again."""
+    import torch
+    from paper_1912_08569_gb300 import SwapBatch
+
+    wl = _wl(1500, 0.4)
+    st = torch.cuda.Stream()
+    a, b = make_gpu(wl, "fp32", stream=st), make_gpu(wl, "fp32", stream=st)
+    b.run(10, 0.001, 0.1, 1.0)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        b.run(10, 0.001, 0.1, 1.0, sync=False)
+    SwapBatch([a, b]).run(5, 0.001, 0.1, 1.0, sync=False)
+    with torch.cuda.stream(st):
+        g.replay()
+    assert a.thermo()["step"] == 5
+    assert b.thermo()["step"] == 25
+
+
 @pytest.mark.parametrize("masses", [False, True])
 def test_host_arrays_may_be_reused_when_the_call_returns(masses):
     """Pinned arrays, and work ahead on the stream."""
