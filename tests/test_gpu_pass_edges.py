@@ -225,6 +225,26 @@ def test_a_halo_that_does_not_fit_costs_little():
     assert ms[1] < 3.0 * ms[0], ms
 
 
+# a few large particles with rows of 180 entries (the resident step takes rows of up
+# to 255) and of 420 (the resident build has to turn them down before it sorts by them)
+@pytest.mark.parametrize("big", [1, 9])
+@pytest.mark.parametrize("rcut", [4.45, 6.0])
+def test_rows_at_the_resident_limit(orc, big, rcut):
+    wl = _wl(3000, 0.4)
+    wl["types"] = (np.arange(3000) < big).astype(np.int32)
+    wl["pairs"] = inputs.swap_pairs(lambda3=1.0, rcut=rcut)
+    got = []
+    for resident in (True, False):
+        s = make_gpu(wl, "fp32")
+        s.set_resident(resident)
+        _check(orc, wl, "fp32", s)
+        s.run(40, 0.001, 0.05, 1.0)
+        assert s.thermo()["resident_steps"] == (40 if resident and rcut < 5.0 else 0)
+        got.append(s.state())
+    for p, q in zip(*got):
+        assert np.array_equal(p, q)
+
+
 class _At:
     """A device address inside a buffer, as the binding takes it."""
 
